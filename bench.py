@@ -52,7 +52,7 @@ def _peaks():
 
 def _kernel_source_hash() -> str:
     h = hashlib.sha256()
-    for f in ("gmp_decode.cu", "gmp_internal.h"):
+    for f in ("gmp_decode.cu", "gmp_decode_common.h", "gmp_tile.cu", "gmp_internal.h"):
         with open(os.path.join(ROOT, "paper_1606_00519_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

@@ -22,7 +22,7 @@ BUILD = os.path.join(_PKG, "_build")
 LIB_PATH = os.path.join(BUILD, "libgmp.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["gmp_decode.cu", "gmp_host.cpp", "gmp_compress.cpp", "gmp_server.cpp", "gmp_noalloc.cu",
+SOURCES = ["gmp_decode.cu", "gmp_tile.cu", "gmp_host.cpp", "gmp_compress.cpp", "gmp_server.cpp", "gmp_noalloc.cu",
            "gmp_gpucompress.cu", "gmp_gpuencode.cu"]
 
 _lock = threading.Lock()

@@ -50,11 +50,10 @@
 #include <stdint.h>
 
 #include "gmp.h"
+#include "gmp_decode_common.h"
 #include "gmp_internal.h"
 
 namespace gmp {
-
-constexpr uint32_t FULL = 0xffffffffu;
 
 // Optional stage timers of the LZ77 phase (profiling builds only: compile
 // with -DGMP_PHASE_TIMERS); they add SM-clock deltas per stage into the
@@ -66,18 +65,12 @@ constexpr uint32_t FULL = 0xffffffffu;
 #define GMP_TSTAMP(v)
 #define GMP_TADD(slot, a, b)
 #endif
-constexpr int LUT_BITS = 12;  // the longest code (cwl <= 12)
-constexpr int LUT_SIZE = 1 << LUT_BITS;
 // The lookup tables cover codes of up to LLB (literal/length tree: 12 bits in
 // the 128-register kernel, 11 in the 96-register one, whose 20 warps per SM
 // need a smaller table) and OFF_BITS (offset tree) bits; the rare longer
 // codes are decoded from the tree's canonical arrays (decode_long).
 constexpr int OFF_BITS = 10;
 constexpr int OFF_SIZE = 1 << OFF_BITS;
-constexpr uint16_t LONG_CODE = 0xffff;
-constexpr int N_LL = 319;
-constexpr int N_OFF = 30;
-constexpr int MAX_SUB = 64;
 constexpr int RING = 4096;  // shared-memory output ring per warp (bytes)
 constexpr uint32_t RING_MASK = RING - 1;
 // back-reference sources at most NEAR bytes below the group start are read
@@ -91,13 +84,6 @@ constexpr int FAR_STAGE = 80;
 // the shadow (all in one sub-block) and fit, with alignment, in 32 chunks
 constexpr int LIT_STAGE = 512;
 constexpr uint32_t RING_WMASK = RING / 4 - 1;
-
-// Canonical arrays of one tree (Sec. 3.1): per code length its code count,
-// its first index in the symbol list sorted by (length, symbol), and its
-// first code.
-struct Canon {
-  uint32_t cnt[16], idx[16], first[16];
-};
 
 // Phase A: the lookup tables, the trees' canonical arrays and the sub-block
 // table of the block being decoded.
@@ -135,143 +121,11 @@ struct __align__(16) WarpSmem {
 };
 static_assert(sizeof(PhaseASmem<11>) <= sizeof(PhaseBSmem), "the 11-bit phase A fits in the phase B space");
 
-struct KParams {
-  const gmp_file_desc* files;  // batch mode; nullptr in single-stream mode
-  const uint64_t* item_start;  // batch mode: n_files + 1 prefix sums
-  uint32_t n_files;
-  gmp_file_desc single;  // single-stream mode
-  int32_t* status;       // one per file
-  unsigned long long* counter;
-  uint8_t* scratch;
-  uint64_t slot_bytes;
-  uint64_t shadow_off;  // offset of the literal shadow inside a slot (256-byte aligned)
-  uint32_t max_seq, max_out;
-  unsigned long long* stats;  // [groups, rounds, de_fallback, blocks, max_rounds, cycles x3]
-  int collect_stats;
-  int resolve;  // 0: by the stream's DE flag, 1: MRR always, 2: sequential copying (SC)
-  int spread;   // 1: first items fixed and interleaved over the CTAs; 0: all from the counter
-  // Host-to-host pipeline (all null otherwise): a file's input is complete
-  // once in_ready[file] reaches gen (written by the copy stream after the
-  // copy); out_ready[file] is set to gen once all its blocks are decoded
-  // (done[file] counts them), and by the last warp to exit (exited counts
-  // the warps) for every file.
-  const uint32_t* in_ready;
-  uint32_t* abort_wait;  // set once a wait has run out: later waits give up at once
-  unsigned long long wait_ns;
-  uint32_t* out_ready;
-  uint32_t* done;
-  uint32_t* exited;
-  uint32_t gen;
-};
-
-__device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
-
 // Two 16-byte records as one 32-byte store (p 32-byte aligned).
 __device__ __forceinline__ void st_global_32B(void* p, const uint4& a, const uint4& b) {
   asm volatile("st.global.v8.u32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
                "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
                : "memory");
-}
-
-__device__ __forceinline__ void set_status(int32_t* st, int code) { atomicCAS(st, 0, code); }
-
-// ---- host-to-host pipeline flags
-// The wait for a file's input is bounded: the host's limit (10 s unless the
-// context sets another) of the global timer, and at most 2^24 polls; past
-// that the file gets GMP_STATUS_INPUT_TIMEOUT, its blocks are skipped and
-// every later wait of the launch gives up at once, so the launch always ends.
-constexpr uint32_t kInputWaitPolls = 1u << 24;
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ uint32_t ld_acquire_sys(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.sys.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_release_sys(uint32_t* p, uint32_t v) {
-  asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// Whole warp: true once *flag has reached gen (cyclic comparison, as the
-// copy stream's flag values wrap), false if the wait ran out.  The warp polls
-// and sleeps as one: with lane 0 polling and sleeping alone while the other
-// lanes waited at a shuffle, the warps decoded their next blocks 2 to 2.7
-// times slower (measured on text256m, (In) mode).
-__device__ __noinline__ bool wait_input(const uint32_t* flag, uint32_t* abort_wait, uint32_t gen,
-                                        unsigned long long wait_ns) {
-  const unsigned long long t0 = global_ns();
-  bool ok = false;
-  for (uint32_t i = 0; i < kInputWaitPolls; i++) {
-    // lane 0 reads the flag, the abort word and the clock; every decision
-    // below is taken on its values, so the lanes leave the loop together
-    uint32_t v = 0, stop = 0;
-    if ((threadIdx.x & 31u) == 0) {
-      v = ld_acquire_sys(flag);
-      stop = *reinterpret_cast<volatile uint32_t*>(abort_wait) != 0u || global_ns() - t0 > wait_ns;
-    }
-    v = __shfl_sync(0xffffffffu, v, 0);
-    stop = __shfl_sync(0xffffffffu, stop, 0);
-    if ((int32_t)(v - gen) >= 0) {
-      ok = true;
-      break;
-    }
-    if (stop) break;
-    __nanosleep(i < 64 ? 64 : 1024);
-  }
-  if (!ok && (threadIdx.x & 31u) == 0) atomicExch(abort_wait, 1u);
-  __syncwarp();
-  return ok;
-}
-
-// Whole warp, after a block of `file` (n_blocks blocks) is decoded: every
-// lane's output stores are made visible before the block is counted, and
-// the count that completes the file publishes its out_ready flag.
-__device__ __noinline__ void block_done(uint32_t* done, uint32_t* out_ready, uint32_t gen, uint64_t n_blocks) {
-  __threadfence();
-  __syncwarp();
-  if ((threadIdx.x & 31u) == 0) {
-    const uint32_t d = atomicAdd(done, 1u) + 1u;
-    if (d == (uint32_t)n_blocks) {
-      __threadfence_system();
-      st_release_sys(out_ready, gen);
-    }
-  }
-  __syncwarp();
-}
-
-// Whole warp, on leaving the persistent loop: the last warp of the launch
-// sets every file's out_ready flag, so that no copy stream waits on a flag
-// that is never written.
-__device__ __noinline__ void pipeline_exit(uint32_t* exited, uint32_t* out_ready, uint32_t gen, uint32_t n_files,
-                                           uint32_t n_warps) {
-  __threadfence();
-  uint32_t last = 0;
-  if ((threadIdx.x & 31u) == 0) last = atomicAdd(exited, 1u) + 1u == n_warps;
-  last = __shfl_sync(0xffffffffu, last, 0);
-  if (last) {
-    __threadfence_system();
-    for (uint32_t f = threadIdx.x & 31u; f < n_files; f += 32) st_release_sys(out_ready + f, gen);
-  }
-}
-
-__device__ __forceinline__ uint32_t ld_u32_nc(const uint8_t* p) { return __ldg(reinterpret_cast<const uint32_t*>(p)); }
-__device__ __forceinline__ uint64_t ld_u64_nc(const uint8_t* p) {
-  return __ldg(reinterpret_cast<const unsigned long long*>(p));
-}
-
-// inclusive warp scan of a 32-bit value
-__device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v) {
-  const uint32_t lane = lane_id();
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    uint32_t y = __shfl_up_sync(FULL, v, d);
-    if (lane >= (uint32_t)d) v += y;
-  }
-  return v;
 }
 
 // ---------------------------------------------------------------------------
@@ -352,29 +206,6 @@ __device__ bool build_lut(Canon& C, uint32_t* run, uint16_t* sorted, const uint8
   __syncwarp();
   return true;
 }
-
-// A code longer than the table's bits, by the canonical ranges: the 12-bit
-// peek, most significant bit first, lies in length L's range [first_L,
-// first_L + cnt_L) shifted left by 12 - L.  Returns (L << 9) | symbol.
-template <int TB>
-__device__ __forceinline__ uint32_t decode_long(const Canon& C, const uint16_t* sorted, uint32_t peek12) {
-  const uint32_t v = __brev(peek12) >> (32 - LUT_BITS);
-  for (int L = TB + 1; L <= LUT_BITS; L++) {
-    const uint32_t code = v >> (LUT_BITS - L);
-    if (code - C.first[L] < C.cnt[L]) return ((uint32_t)L << 9) | sorted[C.idx[L] + code - C.first[L]];
-  }
-  return 0;
-}
-
-// ---------------------------------------------------------------------------
-// cp.async (16-byte, L2-only) global -> shared copies and their groups.
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 __device__ __forceinline__ void copy_match_global(uint8_t* out_blk, uint32_t rpos, uint32_t wpos, uint32_t ml) {
   for (uint32_t i = 0; i < ml; i++) out_blk[wpos + i] = out_blk[rpos + i];
@@ -645,69 +476,21 @@ template <bool STATS, int LLB>
 __device__ void decode_block(WarpSmem<LLB>& S, const KParams& P, const gmp_file_desc& F, uint64_t b, int32_t* status,
                              uint8_t* slot, unsigned long long* st_acc) {
   const uint32_t lane = lane_id();
-  const uint8_t* comp = F.comp;
   const long long t_begin = STATS ? clock64() : 0;
 #ifdef GMP_PHASE_TIMERS
   unsigned long long tdet[6] = {0, 0, 0, 0, 0, 0};
 #endif
-  // ---- stream header (64 bytes), block reference
-  int err = 0;
-  uint32_t flags = 0, K = 0, window = 0, max_match = 0;
-  bool byte_fmt = false;  // Gompresso/Byte block: records and raw literals, no Huffman phase
-  if (F.comp_bytes < 64 || (((uintptr_t)comp) & 15u)) {
-    if (lane == 0) set_status(status, GMP_STATUS_BAD_HEADER);
-    return;
-  }
-  {
-    uint32_t magic = ld_u32_nc(comp);
-    uint32_t w1 = ld_u32_nc(comp + 4);
-    uint32_t w3 = ld_u32_nc(comp + 12);
-    window = ld_u32_nc(comp + 16);
-    uint32_t w5 = ld_u32_nc(comp + 20);
-    flags = w1 >> 16;
-    K = w3 & 0xffffu;
-    uint32_t cwl = (w3 >> 16) & 0xffu;
-    max_match = (w5 >> 8) & 0xffu;
-    byte_fmt = !(flags & 2u);
-    if (magic != 0x31504d47u || (w1 & 0xffffu) != 1u || flags > 3u || window == 0 || window > 32768 ||
-        (w5 & 0xffu) != 3u || max_match < 3 || max_match > 64)
-      err = GMP_STATUS_BAD_HEADER;
-    else if (byte_fmt ? (K != 0 || cwl != 0) : (K == 0 || K > MAX_SUB || cwl == 0 || cwl > 12))
-      err = GMP_STATUS_BAD_HEADER;
-  }
-  const gmp_block_ref br = F.index[b];
-  if (!err) {
-    if ((br.comp_offset & 15) || br.comp_offset > F.comp_bytes || br.comp_bytes > F.comp_bytes - br.comp_offset ||
-        br.out_offset > F.out_cap || br.out_bytes > F.out_cap - br.out_offset)
-      err = GMP_STATUS_OUTPUT_OVERRUN;
-    else if (br.comp_bytes < (byte_fmt ? 16ull : (192 + 12ull * K + 15) & ~15ull))  // through the bitstream start
-      err = GMP_STATUS_BAD_HEADER;
-  }
+  BlockView V;
+  int err = open_block(F, b, V);
+  if (!err && !V.byte_fmt && (V.out_bytes > P.max_out || V.n_seq > P.max_seq)) err = GMP_STATUS_CAPACITY;
   if (err) {
     if (lane == 0) set_status(status, err);
     return;
   }
-  const uint8_t* B = comp + br.comp_offset;
-  const uint32_t n_seq = ld_u32_nc(B);
-  const uint32_t out_bytes = ld_u32_nc(B + 4);
-  // Byte blocks: literal count and the literal section's offset in the block
-  uint32_t n_lit = 0;
-  uint64_t lit_off = 0;
-  if (out_bytes != br.out_bytes) {
-    err = GMP_STATUS_BAD_HEADER;
-  } else if (byte_fmt) {
-    // the records and the padded literal section lie inside the block (whole
-    // 16-byte chunks, which the literal staging reads)
-    n_lit = ld_u32_nc(B + 8);
-    lit_off = (16ull + 4ull * n_seq + 15ull) & ~15ull;
-    if (lit_off + ((n_lit + 15ull) & ~15ull) > br.comp_bytes) err = GMP_STATUS_BAD_HEADER;
-  } else if (out_bytes > P.max_out || n_seq > P.max_seq) {
-    err = GMP_STATUS_CAPACITY;
-  }
-  if (err) {
-    if (lane == 0) set_status(status, err);
-    return;
-  }
+  const uint32_t flags = V.flags, K = V.K, window = V.window, max_match = V.max_match;
+  const bool byte_fmt = V.byte_fmt;  // Gompresso/Byte block: records and raw literals, no Huffman phase
+  const uint8_t* B = V.B;
+  const uint32_t n_seq = V.n_seq, out_bytes = V.out_bytes, n_lit = V.n_lit;
   // phase A output (Huffman blocks): records and the literal shadow in the
   // warp's scratch slot
   uint4* rec = reinterpret_cast<uint4*>(slot);
@@ -717,12 +500,12 @@ __device__ void decode_block(WarpSmem<LLB>& S, const KParams& P, const gmp_file_
   if (byte_fmt) {
     // phase B reads the records from the stream and the literals from the
     // block's literal section
-    lits = B + lit_off;
+    lits = B + V.lit_off;
     t_tables = t_phase_a = STATS ? clock64() : 0;
     __syncwarp();
   } else {
     const uint32_t bs_off = (192u + 12u * K + 15u) & ~15u;  // bitstream start within the block
-    const uint64_t bits_avail = (br.comp_bytes - bs_off) * 8ull;
+    const uint64_t bits_avail = (V.comp_bytes - bs_off) * 8ull;
 
     // ---- sub-block table: prefix sums of bit sizes, output sizes, sequences
     {
@@ -798,7 +581,7 @@ __device__ void decode_block(WarpSmem<LLB>& S, const KParams& P, const gmp_file_
     // one instruction stream for all 32 sub-blocks.
     const uint8_t* bs = B + bs_off;
     // 16-byte chunks of the block's bitstream; chunks past the block read as 0
-    const uint64_t bs_chunks = (br.comp_bytes - bs_off) / 16;
+    const uint64_t bs_chunks = (V.comp_bytes - bs_off) / 16;
     auto ld4 = [&](uint32_t c) -> uint4 {
       return (uint64_t)c < bs_chunks ? __ldg(reinterpret_cast<const uint4*>(bs) + c) : make_uint4(0, 0, 0, 0);
     };
@@ -1055,7 +838,7 @@ __device__ void decode_block(WarpSmem<LLB>& S, const KParams& P, const gmp_file_
   // Group g+1 is prepared while group g runs: its two prefix sums are taken
   // and its literal runs and far back-reference sources are copied into the
   // stage (g+1)&1 by cp.async, so that group g's work reads shared memory only.
-  uint8_t* out_blk = F.out + br.out_offset;
+  uint8_t* out_blk = F.out + V.out_offset;
   const bool vec_ok = (((uintptr_t)out_blk) & 15u) == 0;
   const bool de = (flags & 1u) != 0;
   PhaseBSmem& SB = S.u.b;
@@ -1535,6 +1318,7 @@ cudaError_t launch_decode(const LaunchShape& shape, const gmp_file_desc* files, 
   P.stats = stats;
   P.collect_stats = collect_stats;
   P.resolve = resolve;
+  if (shape.tile) return launch_tile(P, shape.grid, shape.warps_per_cta, pipe != nullptr, stream);
   const bool deep = shape.deep && shape.warps_per_cta <= 4;
   cudaError_t e = configure_kernel(deep, shape.smem_bytes);
   if (e != cudaSuccess) return e;

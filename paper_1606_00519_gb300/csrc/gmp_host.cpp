@@ -216,15 +216,21 @@ static int context_alloc_scratch(gmp_context* c) {
   // launch shape: persistent grid, as many CTAs per SM as fit
   int wpc = c->opts.warps_per_cta ? (int)c->opts.warps_per_cta : 4;
   if (wpc < 1 || wpc > 16) return GMP_ERR_INVALID_ARG;
-  // CTAs per SM of the 128-register kernel and, for CTAs of at most 4 warps,
-  // of the 96-register one (each with its own shared memory per warp);
-  // shapes beyond the first need the second
+  // the default kernel; with statistics or a forced resolution the one of
+  // gmp_decode.cu, below: CTAs per SM of its 128-register instance and, for
+  // CTAs of at most 4 warps, of its 96-register one (each with its own shared
+  // memory per warp); shapes beyond the first need the second
+  c->shape.tile = !c->opts.collect_stats && c->opts.resolve == GMP_RESOLVE_AUTO;
   const size_t smem_wide = (size_t)wpc * gmp::warp_smem_bytes(false);
   const size_t smem_deep = (size_t)wpc * gmp::warp_smem_bytes(true);
   int occ_wide = 0, occ_deep = 0;
-  GMP_CUDA(gmp::configure_kernel(false, smem_wide));
-  GMP_CUDA(gmp::occupancy(wpc, smem_wide, false, &occ_wide));
-  if (wpc <= 4) {
+  if (c->shape.tile) {
+    GMP_CUDA(gmp::tile_occupancy(wpc, &occ_wide));
+  } else {
+    GMP_CUDA(gmp::configure_kernel(false, smem_wide));
+    GMP_CUDA(gmp::occupancy(wpc, smem_wide, false, &occ_wide));
+  }
+  if (wpc <= 4 && !c->shape.tile) {
     GMP_CUDA(gmp::configure_kernel(true, smem_deep));
     GMP_CUDA(gmp::occupancy(wpc, smem_deep, true, &occ_deep));
   }
@@ -237,15 +243,16 @@ static int context_alloc_scratch(gmp_context* c) {
   c->shape.warps_per_cta = wpc;
   c->shape.deep = per_sm > occ_wide;
   c->shape.smem_bytes = c->shape.deep ? smem_deep : smem_wide;
-  // one scratch slot per resident warp: records (16 B per sequence; a block
-  // holds at most out/3 + 1 sequences) and the literal shadow (output layout
-  // plus 16 bytes of separation per sub-block)
+  // one scratch slot per resident warp: the default kernel's 8-byte records,
+  // or records (16 B per sequence; a block holds at most out/3 + 1 sequences)
+  // and the literal shadow (output layout plus 16 bytes of separation per
+  // sub-block)
   c->max_out = c->opts.max_block_out;
   c->max_seq = c->max_out / 3 + 2;
   uint64_t rec = ((uint64_t)c->max_seq * 16 + 255) & ~255ull;
   uint64_t shadow = (uint64_t)c->max_out + 16ull * gmp::kMaxSub + 64;
   c->shadow_off = rec;
-  c->slot_bytes = (rec + shadow + 255) & ~255ull;
+  c->slot_bytes = c->shape.tile ? gmp::tile_slot_bytes(c->max_out) : (rec + shadow + 255) & ~255ull;
   size_t need = (size_t)c->slot_bytes * (size_t)c->shape.grid * (size_t)wpc;
   if (c->scratch && c->scratch_bytes >= need) return GMP_OK;
   if (c->scratch) cudaFree(c->scratch);
@@ -441,16 +448,20 @@ int gmp_autotune(gmp_context* c, const gmp_file_desc* d_files, size_t n_files, i
   int rc = GMP_OK;
   for (uint32_t w : {1u, 2u, 4u, 8u, 16u}) {
     int occ_wide = 0, occ_deep = 0;
-    const size_t smem_wide = (size_t)w * gmp::warp_smem_bytes(false);
-    const size_t smem_deep = (size_t)w * gmp::warp_smem_bytes(true);
-    if (gmp::configure_kernel(false, smem_wide) != cudaSuccess ||
-        gmp::occupancy((int)w, smem_wide, false, &occ_wide) != cudaSuccess)
-      continue;
-    if (w <= 4 && (gmp::configure_kernel(true, smem_deep) != cudaSuccess ||
-                   gmp::occupancy((int)w, smem_deep, true, &occ_deep) != cudaSuccess))
-      occ_deep = 0;
-    // every SM full with the 96-register kernel, full and half full with the
-    // 128-register one
+    if (c->shape.tile) {
+      if (gmp::tile_occupancy((int)w, &occ_wide) != cudaSuccess) continue;
+    } else {
+      const size_t smem_wide = (size_t)w * gmp::warp_smem_bytes(false);
+      const size_t smem_deep = (size_t)w * gmp::warp_smem_bytes(true);
+      if (gmp::configure_kernel(false, smem_wide) != cudaSuccess ||
+          gmp::occupancy((int)w, smem_wide, false, &occ_wide) != cudaSuccess)
+        continue;
+      if (w <= 4 && (gmp::configure_kernel(true, smem_deep) != cudaSuccess ||
+                     gmp::occupancy((int)w, smem_deep, true, &occ_deep) != cudaSuccess))
+        occ_deep = 0;
+    }
+    // every SM full and half full (gmp_decode.cu: full with its 96-register
+    // instance, full and half full with the 128-register one)
     const int cands[3] = {occ_deep > occ_wide ? occ_deep : 0, occ_wide, occ_wide / 2};
     for (int cps : cands) {
       if (cps < 1 || (cps == occ_wide / 2 && occ_wide / 2 == occ_wide)) continue;
