@@ -1318,6 +1318,13 @@ cudaError_t launch_decode(const LaunchShape& shape, const gmp_file_desc* files, 
   P.stats = stats;
   P.collect_stats = collect_stats;
   P.resolve = resolve;
+  P.coop_max = 0;
+  if (shape.tile && shape.coop) return launch_coop(P, shape.grid, shape.coop, pipe != nullptr, stream);
+  if (shape.tile && shape.coop_max) {
+    P.coop_max = shape.coop_max;
+    const cudaError_t e = launch_coop(P, shape.coop_grid, 8, pipe != nullptr, stream);
+    if (e != cudaSuccess) return e;
+  }
   if (shape.tile) return launch_tile(P, shape.grid, shape.warps_per_cta, pipe != nullptr, stream);
   const bool deep = shape.deep && shape.warps_per_cta <= 4;
   cudaError_t e = configure_kernel(deep, shape.smem_bytes);

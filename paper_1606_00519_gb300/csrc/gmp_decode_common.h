@@ -42,6 +42,7 @@ struct KParams {
   unsigned long long* stats;  // [groups, rounds, de_fallback, blocks, max_rounds, cycles x3]
   int collect_stats;
   int resolve;  // 0: by the stream's DE flag, 1: MRR always, 2: sequential copying (SC)
+  uint32_t coop_max;  // 0, or: of a pair of launches the one that the number of blocks calls for runs
   int spread;   // 1: first items fixed and interleaved over the CTAs; 0: all from the counter
   // Host-to-host pipeline (all null otherwise): a file's input is complete
   // once in_ready[file] reaches gen (written by the copy stream after the
@@ -58,6 +59,7 @@ struct KParams {
 };
 
 cudaError_t launch_tile(const KParams& P, int grid, int warps_per_cta, bool pipe, cudaStream_t stream);
+cudaError_t launch_coop(const KParams& P, int grid, int warps, bool pipe, cudaStream_t stream);
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
 

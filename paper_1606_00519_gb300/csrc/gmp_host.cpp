@@ -90,6 +90,7 @@ struct gmp_context {
   gmp_context_opts opts{};
   gmp::LaunchShape shape{};
   int occ_wide = 0, occ_deep = 0;  // CTAs per SM of the two kernels at this shape's warps per CTA
+  int coop_ctas[2] = {0, 0};       // resident CTAs of 16 and of 8 warps, a block each
   uint32_t max_seq = 0, max_out = 0;
   uint64_t slot_bytes = 0, shadow_off = 0;
   uint8_t* scratch = nullptr;
@@ -226,6 +227,10 @@ static int context_alloc_scratch(gmp_context* c) {
   int occ_wide = 0, occ_deep = 0;
   if (c->shape.tile) {
     GMP_CUDA(gmp::tile_occupancy(wpc, &occ_wide));
+    for (int k = 0; k < 2; k++) {
+      GMP_CUDA(gmp::coop_occupancy(16 >> k, &c->coop_ctas[k]));
+      c->coop_ctas[k] *= c->sm_count;
+    }
   } else {
     GMP_CUDA(gmp::configure_kernel(false, smem_wide));
     GMP_CUDA(gmp::occupancy(wpc, smem_wide, false, &occ_wide));
@@ -261,6 +266,42 @@ static int context_alloc_scratch(gmp_context* c) {
   GMP_CUDA(cudaMalloc(&c->scratch, need));
   c->scratch_bytes = need;
   return GMP_OK;
+}
+
+// How a launch of n_blocks blocks (0: not known here; byte_fmt: 1 if they are
+// Byte blocks, 0 if not, -1: not known here; from_host: their input is being
+// copied in) is made with the default kernels.
+// A CTA of 16 warps decodes a block fastest, while each block has an SM; CTAs
+// of 8 warps, three on an SM, are faster than a warp per block up to about two
+// rounds of them, four for Byte blocks, which have no Huffman phase.  Measured
+// (us, one stream of 256 KiB blocks, 16 warps / 8 warps / a warp per block):
+// text of 128 blocks 363 / 421 / 1510, 256: 716 / 531 / 1520, 768: - / 1369 /
+// 1634, 1024: - / 1561 / 1637, 2048: - / 2988 / 2080; Byte records of 1024
+// blocks - / 874 / 1607, 2048: - / 1705 / 1776; text of 64 KiB blocks, 256: -
+// / 235 / 537, 1024: - / 684 / 601.  Where the device alone knows the blocks,
+// it chooses between both launches.  Blocks that are copied in meanwhile arrive
+// in order, so that finishing the first of them early counts: three rounds
+// (256 MiB of records from host memory, 1024 blocks: 1.66 ms against 2.18 with
+// a warp per block).  A context whose launches share the GPU
+// takes CTAs only for the fewest blocks, since they cost more SM time.  (The
+// scratch has a slot per warp of c->shape's grid; a CTA takes one.)
+static gmp::LaunchShape tile_shape(const gmp_context* c, uint64_t n_blocks, int byte_fmt, bool from_host = false) {
+  gmp::LaunchShape s = c->shape;
+  const uint64_t slots = (uint64_t)c->shape.grid * (uint64_t)c->shape.warps_per_cta;
+  const uint64_t g16 = std::min<uint64_t>(c->coop_ctas[0], slots), g8 = std::min<uint64_t>(c->coop_ctas[1], slots);
+  if (!s.tile || !g16 || !g8) return s;
+  const uint64_t most = c->opts.concurrent ? g16 : from_host ? 3 * g8 : 2 * g8;
+  if (n_blocks && n_blocks <= g16) {
+    s.coop = 16;
+    s.grid = (int)n_blocks;
+  } else if (n_blocks && n_blocks <= most * (byte_fmt == 1 ? 2u : 1u)) {
+    s.coop = 8;
+    s.grid = (int)std::min(n_blocks, g8);
+  } else if (!n_blocks || (byte_fmt < 0 && n_blocks <= 2 * most)) {
+    s.coop_max = (uint32_t)most;
+    s.coop_grid = (int)(n_blocks ? std::min(n_blocks, g8) : g8);
+  }
+  return s;
 }
 
 int gmp_context_create(gmp_context** ctx, int device, const gmp_context_opts* opts) {
@@ -351,7 +392,7 @@ int gmp_decompress(gmp_context* c, const uint8_t* d_comp, size_t comp_bytes, con
   if (n_blocks == 0) return GMP_OK;
   GMP_CUDA(cudaMemsetAsync(c->counter, 0, sizeof(unsigned long long), s));
   gmp_file_desc F{d_comp, comp_bytes, d_index, n_blocks, d_out, out_cap};
-  gmp::LaunchShape shape = c->shape;
+  gmp::LaunchShape shape = tile_shape(c, n_blocks, -1);
   // when the 128-register kernel holds a warp for every block, it decodes
   // each block faster; at most one CTA per block, and the kernel spreads the
   // blocks over the CTAs (a CTA's first warp, then its second, ...), so that
@@ -380,7 +421,7 @@ int gmp_decompress_batch(gmp_context* c, const gmp_file_desc* d_files, size_t n_
   GMP_CUDA(cudaMemsetAsync(d_status, 0, n_files * sizeof(int32_t), s));
   GMP_CUDA(cudaMemsetAsync(c->counter, 0, sizeof(unsigned long long), s));
   GMP_CUDA(gmp::launch_batch_prefix(d_files, (uint32_t)n_files, c->item_start, s));
-  GMP_CUDA(gmp::launch_decode(c->shape, d_files, c->item_start, (uint32_t)n_files, nullptr, d_status, c->counter,
+  GMP_CUDA(gmp::launch_decode(tile_shape(c, 0, -1), d_files, c->item_start, (uint32_t)n_files, nullptr, d_status, c->counter,
                               c->scratch, c->slot_bytes, c->shadow_off, c->max_seq, c->max_out, c->stats,
                               (int)c->opts.collect_stats, (int)c->opts.resolve, s, c->opts.concurrent ? 0 : 1));
   return GMP_OK;
@@ -737,7 +778,11 @@ static int decompress_from_host(gmp_context* c, size_t n_files, const void* cons
                               to_device ? nullptr : done,
                               to_device ? nullptr : done + fn,
                               gen};
-      ce = gmp::launch_decode(c->shape, reinterpret_cast<const gmp_file_desc*>(c->h_meta + desc_off),
+      int byte_fmt = -1;  // of all the streams
+      for (size_t f = 0; f < n_files; f++)
+        if (!files[f].idx.empty()) byte_fmt = (files[f].info.flags & 2u) || byte_fmt == 0 ? 0 : 1;
+      const gmp::LaunchShape shape = tile_shape(c, items, std::max(byte_fmt, 0), true);
+      ce = gmp::launch_decode(shape, reinterpret_cast<const gmp_file_desc*>(c->h_meta + desc_off),
                               reinterpret_cast<const uint64_t*>(c->h_meta + pre_off), (uint32_t)n_pieces, nullptr,
                               c->h_status, counter, c->scratch, c->slot_bytes, c->shadow_off, c->max_seq, c->max_out,
                               c->stats, (int)c->opts.collect_stats, (int)c->opts.resolve, c->pipe, 1, &pf);

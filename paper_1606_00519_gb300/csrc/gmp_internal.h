@@ -16,7 +16,10 @@ struct LaunchShape {
   int warps_per_cta;  // one block of a stream per warp at a time
   size_t smem_bytes;  // dynamic shared memory per CTA
   bool deep;          // the 96-register kernel (more than 16 warps per SM; warps_per_cta <= 4)
-  bool tile;          // the default kernel of gmp_tile.cu (resolve = auto, no statistics)
+  bool tile;          // the default kernels of gmp_tile.cu (resolve = auto, no statistics)
+  int coop;           // with tile: 0, or the warps (8, 16) of a CTA that decodes a block together (grid CTAs)
+  uint32_t coop_max;  // with coop = 0: 0, or launch coop_grid CTAs of 8 warps too, which take up to this many blocks
+  int coop_grid;
 };
 
 // warps per SM that the 128-register kernel holds
@@ -27,9 +30,11 @@ constexpr int kWideWarpsPerSm = 16;
 size_t warp_smem_bytes(bool deep);
 cudaError_t configure_kernel(bool deep, size_t smem_bytes);
 cudaError_t occupancy(int warps_per_cta, size_t smem_bytes, bool deep, int* ctas_per_sm);
-// The default decode kernel (gmp_tile.cu): CTAs per SM at this many warps per
-// CTA, and the scratch a warp's slot needs for blocks of up to max_out bytes.
+// The default decode kernels (gmp_tile.cu): CTAs per SM, a warp per block at
+// this many warps per CTA, or a CTA of 8 or 16 warps per block; and the scratch
+// a block's slot needs for blocks of up to max_out bytes.
 cudaError_t tile_occupancy(int warps_per_cta, int* ctas_per_sm);
+cudaError_t coop_occupancy(int warps, int* ctas_per_sm);
 uint64_t tile_slot_bytes(uint64_t max_out);
 // Flags of a host-to-host launch (device arrays, one word per file of the
 // launch; see gmp_host.cpp): in_ready[f] reaches gen when file f's input has

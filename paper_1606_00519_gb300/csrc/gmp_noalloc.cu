@@ -28,7 +28,6 @@ namespace {
 
 constexpr uint32_t kMaxBlockOut = 256u << 10;
 constexpr uint32_t kSlots = 32;
-constexpr uint32_t kWarpsPerCta = 4;
 constexpr uint32_t kMaxSeq = kMaxBlockOut / 3 + 2;
 constexpr uint64_t kRecBytes = ((uint64_t)kMaxSeq * 16 + 255) & ~uint64_t(255);
 constexpr uint64_t kShadowBytes = (uint64_t)kMaxBlockOut + 16ull * gmp::kMaxSub + 64;
@@ -132,13 +131,14 @@ int gmp_decompress_noalloc(const uint8_t* d_comp, size_t comp_bytes, const gmp_b
   // the work counter (and the statistics words after it) must start at zero
   if (cudaMemsetAsync(scratch, 0, kHeaderBytes, s) != cudaSuccess) return GMP_ERR_CUDA;
   gmp::LaunchShape shape;
-  shape.warps_per_cta = (int)kWarpsPerCta;
+  shape.warps_per_cta = 16;
   shape.smem_bytes = 0;
   shape.deep = false;
   shape.tile = true;
-  shape.grid = (int)(kSlots / kWarpsPerCta);
-  const uint64_t ctas_needed = (n_blocks + kWarpsPerCta - 1) / kWarpsPerCta;
-  if ((uint64_t)shape.grid > ctas_needed) shape.grid = (int)ctas_needed;
+  shape.coop = 16;  // a CTA of 16 warps per block and slot
+  shape.coop_max = 0;
+  shape.coop_grid = 0;
+  shape.grid = (int)(n_blocks < kSlots ? n_blocks : kSlots);
   gmp_file_desc F{d_comp, comp_bytes, d_index, n_blocks, d_out, out_cap};
   unsigned long long* counter = reinterpret_cast<unsigned long long*>(scratch);
   cudaError_t e = gmp::launch_decode(shape, nullptr, nullptr, 0, &F, d_status, counter, scratch + kHeaderBytes,

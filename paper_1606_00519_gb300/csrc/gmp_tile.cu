@@ -55,23 +55,22 @@ namespace {
 
 // ---------------------------------------------------------------------------
 // Phase A tables.  Literal/length entry of an LLB-bit peek: bits 0-3 code
-// bits consumed (0 = no code), 4-5 literals (0..2, in bytes 2 and 3), byte 1
-// the match (0 none, kEndCode the end symbol, else the length).  With an
+// bits consumed, 4-5 literals (0..2, in bytes 2 and 3), byte 1 the match (0
+// none, else the length; as a signed byte -1 for the end symbol and -2 for
+// lengths above the stream's longest match, which leave the fast path).  With an
 // 11-bit table a prefix of 12-bit codes has kLongLL set and the two codes as
-// halves (the upper one for a next bit of 0): byte or match in bits 0-7, bit
-// 8 for a literal.  Offset entry:
-// byte 0 holds 32 minus the bits of the code and its extra bits, byte 1 32
-// minus the extra bits, the upper half the distance base; a prefix of codes
-// longer than the table's bits is kLongOff, and the canonical arrays decide
-// (codes of 10 bits and more are about 0.3 % of a block's offsets).  No code:
-// a base that is above every window.
-constexpr uint32_t kLongLL = 1u << 15, kLongOff = 0xffffffffu;
-constexpr uint32_t kEndCode = 1;
+// 9-bit halves (bits 23-31 for a next bit of 0, 14-22 for 1): byte or match,
+// bit 8 for a literal.  Offset entry: byte 0 holds 32 minus the bits of the
+// code and its extra bits, byte 1 32 minus the extra bits, the upper half the
+// distance base; a prefix of codes longer than the table's bits is kLongOff,
+// and the canonical arrays decide (codes of 10 bits and more are about 0.3 %
+// of a block's offsets).  No code: a base above every window.
+constexpr uint32_t kLongLL = 1u << 7, kLongOff = 0xffffffffu;
 constexpr uint32_t kNoOff = 0xffff2020u, kNoMatch = 0x2020u;
 
-__device__ __forceinline__ uint32_t ll_entry(uint32_t sym, uint32_t len) {
-  if (sym < 256) return len | (1u << 4) | (sym << 16);
-  return len | ((sym == 256 ? kEndCode : sym - 254u) << 8);
+// The symbol's part of an entry: a literal's byte, or the match.
+__device__ __forceinline__ uint32_t match_code(uint32_t sym, uint32_t max_match) {
+  return sym == 256 ? 0xffu : sym - 254u > max_match ? 0xfeu : sym - 254u;
 }
 __device__ __forceinline__ uint32_t off_entry(uint32_t os, uint32_t len) {
   const uint32_t ne = os < 4 ? 0u : (os >> 1) - 1u;
@@ -130,9 +129,10 @@ static_assert(kBuf % 16 == 0 && sizeof(TileSmem) % 16 == 0, "16-byte copies");
 static_assert(sizeof(TileSmem) * 4 + 1024 <= 57 * 1024, "16 warps per SM in CTAs of 4");
 
 // First record of sub-block j, whose output starts at `out`: a record covers
-// at least 3 bytes of output but for a sub-block's last one; a multiple of 4,
-// so that four records are 32-byte aligned.
-__device__ __forceinline__ uint32_t rec_start(uint32_t out, uint32_t j) { return (out / 3 + 5 * j + 3) & ~3u; }
+// at least 3 bytes of output but for a sub-block's last one, and a corrupt
+// stream may write two more; a multiple of 4, so that four records are
+// 32-byte aligned.
+__device__ __forceinline__ uint32_t rec_start(uint32_t out, uint32_t j) { return (out / 3 + 7 * j + 3) & ~3u; }
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t lds_u8(uint32_t a) {
@@ -209,8 +209,8 @@ __device__ __forceinline__ uint32_t code_length(const uint32_t (&lim)[TB + 1], u
 
 // The two lookup tables from the canonical arrays; threads t of n.
 template <int TB>
-__device__ __forceinline__ void fill_ll(uint32_t* lut, const Canon& C, const uint16_t* sorted, bool empty, uint32_t t,
-                                        uint32_t n) {
+__device__ __forceinline__ void fill_ll(uint32_t* lut, const Canon& C, const uint16_t* sorted, bool empty,
+                                        uint32_t max_match, uint32_t t, uint32_t n) {
   uint32_t lim[TB + 1];
 #pragma unroll
   for (int L = 1; L <= TB; L++) lim[L] = (C.first[L] + C.cnt[L]) << (TB - L);
@@ -222,19 +222,21 @@ __device__ __forceinline__ void fill_ll(uint32_t* lut, const Canon& C, const uin
       x = 0;
     } else if (L > (uint32_t)TB) {  // the prefix's two 12-bit codes
       const uint32_t i = C.idx[TB + 1] + 2 * v - C.first[TB + 1];
-      auto half = [](uint32_t s) { return s < 256 ? 256u | s : s == 256 ? kEndCode : s - 254u; };
-      x = kLongLL | (half(sorted[i]) << 16) | half(sorted[i + 1]);
+      auto half = [&](uint32_t s) { return s < 256 ? 256u | s : match_code(s, max_match); };
+      x = kLongLL | (half(sorted[i]) << 23) | (half(sorted[i + 1]) << 14);
     } else {
       const uint32_t s = sorted[C.idx[L] + (v >> (TB - L)) - C.first[L]];
-      x = ll_entry(s, L);
-      if (s < 256 && L < (uint32_t)TB) {
-        // a literal: the next code too, if it lies in the remaining bits
+      if (s >= 256) {
+        x = L | (match_code(s, max_match) << 8);
+      } else {
+        x = L | (1u << 4) | (s << 16);
+        // the next code too, if it lies in the remaining bits
         const uint32_t v2 = (v << L) & ((1u << TB) - 1u);
         const uint32_t L2 = code_length<TB>(lim, v2);
         if (L + L2 <= (uint32_t)TB) {
           const uint32_t s2 = sorted[C.idx[L2] + (v2 >> (TB - L2)) - C.first[L2]];
           x = (L + L2) | (s << 16);
-          x |= s2 < 256 ? (2u << 4) | (s2 << 24) : (1u << 4) | ((s2 == 256 ? kEndCode : s2 - 254u) << 8);
+          x |= s2 < 256 ? (2u << 4) | (s2 << 24) : (1u << 4) | (match_code(s2, max_match) << 8);
         }
       }
     }
@@ -283,6 +285,11 @@ __device__ __forceinline__ void st_global_32B_if(uint2* p, const uint2& a, const
       "r"(a.x), "r"(a.y), "r"(b.x), "r"(b.y), "r"(c.x), "r"(c.y), "r"(d.x), "r"(d.y), "r"((uint32_t)on)
       : "memory");
 }
+__device__ __forceinline__ int byte1_signed(uint32_t v) {
+  int r;
+  asm("prmt.b32 %0, %1, 0, 0x9991;" : "=r"(r) : "r"(v));
+  return r;
+}
 __device__ __forceinline__ uint32_t shl_clamp(uint32_t v, uint32_t n) {  // 0 for n >= 32
   uint32_t r;
   asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
@@ -296,19 +303,22 @@ __device__ __forceinline__ uint32_t shr_clamp(uint32_t v, uint32_t n) {
 template <int LLB, int OFB, bool QUAD>
 __device__ __forceinline__ uint32_t huffman_lane(const uint32_t* ll_lut, const uint32_t* off_lut, const Canon& coff,
                                                  const uint16_t* sorted_off, const uint32_t* ring, const uint8_t* bs,
-                                                 uint32_t n_chunks, bool act, const SubBlock& sb, uint32_t n_seq,
-                                                 uint32_t window, uint32_t max_match, uint2* rec, int& err) {
+                                                 uint32_t n_chunks, bool act, bool empty, const SubBlock& sb,
+                                                 uint32_t n_seq, uint32_t window, uint2* rec, int& err) {
   const uint32_t ring_s = smem_addr(ring);  // 64-byte aligned
-  const uint32_t end = sb.pos + sb.bits, out_end = sb.out + sb.out_n, rec_cap = sb.out_n / 3 + 1;
-  uint32_t outp = sb.out;                 // output position of the current record
-  uint32_t rem = act ? sb.seq_n : 0u;     // sequences to go
-  // the end symbol only closes the block's last sequence
-  const uint32_t end_rem = sb.seq + sb.seq_n == n_seq ? 1u : 0u;
+  // bit positions are counted from 64, so that a position's word is the one
+  // two ahead
+  const uint32_t end = sb.pos + sb.bits + 64u, out_end = sb.out + sb.out_n, rec_cap = sb.out_n / 3 + 1;
+  uint32_t outp = sb.out;              // output position of the current record
+  uint32_t rem = act ? sb.seq_n : 0u;  // sequences to go
+  if (rem && empty) {                  // no literal/length code at all
+    err = GMP_STATUS_CORRUPT_SYMBOL;
+    rem = 0;
+  }
   auto chunk_in = [&](uint32_t c, bool ask) {
     const bool in = c < n_chunks;
     cp_async16_if(ring_s | ((c & (kChunksAhead - 1)) * 16u), bs + (in ? 16ull * c : 0ull), in ? 16u : 0u, ask);
   };
-  // bit position, counted from 64 so that its word is the one two ahead
   uint32_t pos = sb.pos + 64u;
   uint32_t asked = (sb.pos >> 7) + kChunksAhead;  // chunks below it have been asked for
 #pragma unroll
@@ -332,84 +342,99 @@ __device__ __forceinline__ uint32_t huffman_lane(const uint32_t* ll_lut, const u
   };
   uint32_t lits = 0, ln8 = 0, cnt = 0;
   uint2 q0 = make_uint2(0, 0), q1 = q0, q2 = q0, q3 = q0;  // QUAD: the last four records
-  // what one step leaves for the checks
-  struct Step {
-    uint32_t L, mc, e2, ml, dist, wpos, pos, rem;
-    bool bad;
-  };
-  auto one = [&]() -> Step {
-    const uint32_t pk = __funnelshift_r(w0, w1, pos);
+  // the entry of a peek
+  auto ll_of = [&](uint32_t pk) -> uint32_t {
     uint32_t e = ll_lut[pk & ((1u << LLB) - 1u)];
     if (LLB < LUT_BITS) {
-      const uint32_t h = e >> (((pk >> (LLB - 4)) & 16u) ^ 16u);
+      const uint32_t h = e >> (((pk >> LLB) & 1u) ? 14u : 23u);
       const uint32_t v = h & 255u, x = (h & 256u) ? (v << 16) | 28u : (v << 8) | 12u;
       e = (e & kLongLL) ? x : e;
     }
-    Step t;
-    t.rem = rem;
+    return e;
+  };
+  auto off_long = [&](uint32_t pk2) -> uint32_t {
+    const uint32_t x = decode_long<OFB>(coff, sorted_off, pk2 & (LUT_SIZE - 1));
+    return x ? off_entry(x & 511u, x >> 9) : kNoOff;
+  };
+  bool odd = false;  // what the checks after a pair of steps look at
+  auto one = [&]() {
+    const uint32_t pk = __funnelshift_r(w0, w1, pos);
+    uint32_t e = ll_of(pk);
     e = rem ? e : 0u;
-    t.L = e & 15u;
-    t.mc = __byte_perm(e, 0, 0x4441);
-    advance(t.L);
+    const int mc = byte1_signed(e);
+    advance(e & 15u);
     lits |= (e >> 16) << ln8;
     ln8 += (e >> 1) & 24u;
     const uint32_t pk2 = __funnelshift_r(w0, w1, pos);
-    const bool match = t.mc > kEndCode;
     uint32_t e2 = off_lut[pk2 & ((1u << OFB) - 1u)];
-    e2 = match ? e2 : kNoMatch;
+    e2 = mc > 0 ? e2 : kNoMatch;
     if (OFB < LUT_BITS && __any_sync(FULL, e2 == kLongOff)) {
-      if (e2 == kLongOff) {
-        const uint32_t x = decode_long<OFB>(coff, sorted_off, pk2 & (LUT_SIZE - 1));
-        e2 = x ? off_entry(x & 511u, x >> 9) : kNoOff;
-      }
+      if (e2 == kLongOff) e2 = off_long(pk2);
     }
-    t.e2 = e2;
     const uint32_t s1 = e2 & 63u, s2 = __byte_perm(e2, 0, 0x4441);
-    t.dist = (e2 >> 16) + shr_clamp(shl_clamp(pk2, s1), s2);
+    const uint32_t dist = (e2 >> 16) + shr_clamp(shl_clamp(pk2, s1), s2);
     advance(32u - s1);
-    t.pos = pos;
-    t.ml = match ? t.mc : 0u;
-    t.wpos = outp + (ln8 >> 3);
-    // e2's base of kNoOff is above every window
-    t.bad = (rem && t.L == 0) || pos > end + 64u || (t.mc == kEndCode && rem != end_rem) ||
-            (match && (t.ml > max_match || t.dist > min(window, t.wpos) || t.wpos + t.ml > out_end));
-    const bool emit = t.mc != 0 || ln8 >= 24u;
-    const uint2 r = make_uint2(lits, t.dist | (t.ml << 16) | (ln8 << 21));
-    // past the region only on a corrupt stream (caught below)
+    const uint32_t ml = (uint32_t)max(mc, 0), wpos = outp + (ln8 >> 3);
+    odd = odd || mc < 0 || dist > min(window, wpos);
+    const bool emit = mc != 0 || ln8 >= 24u;
+    const uint2 r = make_uint2(lits, dist | (ml << 16) | (ln8 << 21));
     if (QUAD) {
       q0 = emit ? q1 : q0;
       q1 = emit ? q2 : q1;
       q2 = emit ? q3 : q2;
       q3 = emit ? r : q3;
       cnt += emit ? 1u : 0u;
-      st_global_32B_if(rec + (cnt - 4u), q0, q1, q2, q3, emit && (cnt & 3u) == 0 && cnt <= rec_cap);
+      st_global_32B_if(rec + (cnt - 4u), q0, q1, q2, q3, emit && (cnt & 3u) == 0);
     } else {
-      st_global_if(rec + cnt, r, emit && cnt < rec_cap);
+      st_global_if(rec + cnt, r, emit);
       cnt += emit ? 1u : 0u;
     }
-    outp = emit ? t.wpos + t.ml : outp;
+    outp = emit ? wpos + ml : outp;
     lits = emit ? 0u : lits;
     ln8 = emit ? 0u : ln8;
-    rem -= t.mc != 0 ? 1u : 0u;
-    return t;
+    rem -= mc != 0 ? 1u : 0u;
   };
   while (__any_sync(FULL, rem != 0)) {
-    const Step t0 = one();
-    const Step t1 = one();
-    if (__any_sync(FULL, t0.bad || t1.bad)) {
-      // a lane that runs past its sub-block stops here (this bounds the loop
-      // on corrupt input); sizes are checked when the sub-block ends
-      auto status = [&](const Step& t) {
-        if (!t.bad || !t.rem || err) return;
-        if (t.L == 0) err = GMP_STATUS_CORRUPT_SYMBOL;
-        else if (t.pos > end + 64u) err = GMP_STATUS_BITSTREAM;
-        else if (t.mc == kEndCode || t.e2 == kNoOff || t.ml > max_match) err = GMP_STATUS_CORRUPT_SYMBOL;
-        else if (t.dist > window || t.dist > t.wpos) err = GMP_STATUS_BAD_OFFSET;
-        else err = GMP_STATUS_OUTPUT_OVERRUN;
-      };
-      status(t0);
-      status(t1);
+    const uint32_t pos0 = pos, out0 = outp + (ln8 >> 3), rem0 = rem;
+    odd = false;
+    one();
+    one();
+    if (__any_sync(FULL, odd || pos > end || outp > out_end)) {
+      // an end symbol or a corrupt stream: the pair of steps again, with every
+      // check.  A lane that runs past its sub-block stops here, which bounds
+      // the loop; literals past the sub-block's output are noticed when it ends.
+      uint32_t p = pos0, o = out0, left = rem0;
+      for (int k = 0; k < 2 && left && !err; k++) {
+        auto peek = [&]() {
+          return __funnelshift_r(ring[((p >> 5) - 2u) & 15u], ring[((p >> 5) - 1u) & 15u], p);
+        };
+        const uint32_t e = ll_of(peek());
+        const int mc = byte1_signed(e);
+        p += e & 15u;
+        o += (e >> 4) & 3u;
+        if (mc > 0 || mc == -2) {
+          const uint32_t pk2 = peek();
+          uint32_t e2 = off_lut[pk2 & ((1u << OFB) - 1u)];
+          if (OFB < LUT_BITS && e2 == kLongOff) e2 = off_long(pk2);
+          const uint32_t s1 = e2 & 63u, ml = (uint32_t)mc;
+          const uint32_t dist = (e2 >> 16) + shr_clamp(shl_clamp(pk2, s1), __byte_perm(e2, 0, 0x4441));
+          p += 32u - s1;
+          if (p > end) err = GMP_STATUS_BITSTREAM;
+          else if (e2 == kNoOff || mc < 0) err = GMP_STATUS_CORRUPT_SYMBOL;
+          else if (dist > window || dist > o) err = GMP_STATUS_BAD_OFFSET;
+          else if (ml > out_end - min(o, out_end)) err = GMP_STATUS_OUTPUT_OVERRUN;
+          o += ml;
+          left--;
+        } else if (p > end) {
+          err = GMP_STATUS_BITSTREAM;
+        } else if (mc < 0) {
+          // the end symbol, which only closes the block's last sequence
+          if (left != 1u || sb.seq + sb.seq_n != n_seq) err = GMP_STATUS_CORRUPT_SYMBOL;
+          left--;
+        }
+      }
       if (err) rem = 0;
+      cnt = min(cnt, rec_cap);
     }
     const bool ask = rem && ((pos - 64u) >> 7) + kChunksAhead > asked;
     chunk_in(asked, ask);
@@ -425,7 +450,7 @@ __device__ __forceinline__ uint32_t huffman_lane(const uint32_t* ll_lut, const u
     if (n > 0) rec[cnt - 1u] = q3;
   }
   outp += ln8 >> 3;
-  if (!err && pos != end + 64u) err = GMP_STATUS_BITSTREAM;
+  if (!err && pos != end) err = GMP_STATUS_BITSTREAM;
   if (!err && outp != out_end) err = GMP_STATUS_OUTPUT_OVERRUN;
   return cnt;
 }
@@ -497,7 +522,7 @@ __device__ bool huffman_block(TileSmem& S, const BlockView& V, int32_t* status, 
     if (lane == 0) set_status(status, GMP_STATUS_BAD_HEADER);
     return false;
   }
-  fill_ll<kLLBits>(A.ll, T.cll, T.sorted_ll, n_ll == 0, lane, 32);
+  fill_ll<kLLBits>(A.ll, T.cll, T.sorted_ll, n_ll == 0, V.max_match, lane, 32);
   fill_off<kOffBits>(A.off, A.coff, A.sorted_off, n_off == 0, lane, 32);
   __syncwarp();  // the ring takes the build's place
   const uint8_t* bs = V.B + bs_off;
@@ -509,8 +534,8 @@ __device__ bool huffman_block(TileSmem& S, const BlockView& V, int32_t* status, 
       const uint8_t* e = V.B + 192 + 12 * j;
       sb = SubBlock{A.sb_bit[j], ld_u32_nc(e), S.sb_out[j], ld_u32_nc(e + 4), A.sb_seq[j], ld_u32_nc(e + 8)};
     }
-    const uint32_t cnt = huffman_lane<kLLBits, kOffBits, true>(A.ll, A.off, A.coff, A.sorted_off, A.u.bits[lane], bs, n_chunks, j < V.K, sb,
-                                      V.n_seq, V.window, V.max_match, rec + rec_start(sb.out, j), err);
+    const uint32_t cnt = huffman_lane<kLLBits, kOffBits, true>(A.ll, A.off, A.coff, A.sorted_off, A.u.bits[lane], bs, n_chunks, j < V.K, n_ll == 0,
+                                      sb, V.n_seq, V.window, rec + rec_start(sb.out, j), err);
     if (j < V.K) S.sb_cnt[j] = cnt;
   }
   if (err) set_status(status, err);
@@ -533,7 +558,7 @@ struct Group {
   bool slow;  // a Byte group too large for the window or the literal staging
 };
 
-__device__ __forceinline__ void slide(TileSmemB& S, Window& w, uint32_t shift) {
+__device__ __forceinline__ void slide(uint8_t* buf, Window& w, uint32_t shift) {
   const uint32_t lane = lane_id();
   // ascending strips, each loaded whole before it is stored: a strip's
   // destination ends at or below every later strip's source
@@ -541,35 +566,50 @@ __device__ __forceinline__ void slide(TileSmemB& S, Window& w, uint32_t shift) {
   for (uint32_t u = 0; u < n; u += 512u) {
     const uint32_t c = u + 16u * lane;
     uint4 v = make_uint4(0, 0, 0, 0);
-    if (c < n) v = *reinterpret_cast<const uint4*>(S.buf + shift + c);
+    if (c < n) v = *reinterpret_cast<const uint4*>(buf + shift + c);
     __syncwarp();
-    if (c < n) *reinterpret_cast<uint4*>(S.buf + c) = v;
+    if (c < n) *reinterpret_cast<uint4*>(buf + c) = v;
     __syncwarp();
   }
   w.cur -= shift;
   w.base += shift;
 }
 
-__device__ __forceinline__ void flush(const TileSmemB& S, Window& w, uint8_t* out_blk, bool vec_ok) {
+// Stores the output's whole rows up to w.g0; thread t of n.
+__device__ __forceinline__ void flush(const uint8_t* buf, Window& w, uint8_t* out_blk, bool vec_ok, uint32_t t,
+                                      uint32_t n) {
   if (w.g0 - w.flushed < kFlush) return;
-  const uint32_t lane = lane_id(), end = w.g0 & ~(kFlush - 1u);
+  const uint32_t end = w.g0 & ~(kFlush - 1u);
   if (vec_ok) {
-    for (uint32_t c = w.flushed + 16u * lane; c < end; c += kFlush)
-      *reinterpret_cast<uint4*>(out_blk + c) = *reinterpret_cast<const uint4*>(S.buf + (c - w.base));
+    for (uint32_t c = w.flushed + 16u * t; c < end; c += 16u * n)
+      *reinterpret_cast<uint4*>(out_blk + c) = *reinterpret_cast<const uint4*>(buf + (c - w.base));
   } else {
-    for (uint32_t c = w.flushed + lane; c < end; c += 32u) out_blk[c] = S.buf[c - w.base];
+    for (uint32_t c = w.flushed + t; c < end; c += n) out_blk[c] = buf[c - w.base];
   }
   w.flushed = end;
   __syncwarp();
 }
 
-// A Byte group that does not fit the fast path: record after record, the
-// whole warp copying each literal string and each match.
-__device__ __noinline__ void slow_group(TileSmemB& S, Window& w, const uint8_t* recs, uint32_t t0, uint32_t t1,
-                                        const uint8_t* lits, uint8_t* out_blk, bool vec_ok) {
+// What is not flushed at the block's end.
+__device__ __forceinline__ void flush_rest(const uint8_t* buf, const Window& w, uint8_t* out_blk, bool vec_ok,
+                                           uint32_t t, uint32_t n) {
+  uint32_t c = w.flushed;
+  if (vec_ok) {
+    for (uint32_t x = c + 16u * t; x + 16u <= w.g0; x += 16u * n)
+      *reinterpret_cast<uint4*>(out_blk + x) = *reinterpret_cast<const uint4*>(buf + (x - w.base));
+    c = w.g0 & ~15u;
+  }
+  for (c += t; c < w.g0; c += n) out_blk[c] = buf[c - w.base];
+}
+
+// A Byte group that does not fit the fast path: record after record, one
+// warp copying each literal string and each match (window of `cap` bytes,
+// `hist` of them kept).
+__device__ __noinline__ void slow_group(uint8_t* buf, uint32_t cap, uint32_t hist, Window& w, const uint8_t* recs,
+                                        uint32_t t0, uint32_t t1, const uint8_t* lits, uint8_t* out_blk, bool vec_ok) {
   const uint32_t lane = lane_id();
   auto room = [&](uint32_t n) {
-    if (w.cur + n > kBuf) slide(S, w, (w.cur - kHist) & ~15u);
+    if (w.cur + n > cap) slide(buf, w, (w.cur - hist) & ~15u);
   };
   for (uint32_t t = t0; t < t1; t++) {
     const uint32_t r = ld_u32_nc(recs + 4ull * t), m = (r >> 10) & 63u, dist = (r >> 16) + 1u;
@@ -578,25 +618,25 @@ __device__ __noinline__ void slow_group(TileSmemB& S, Window& w, const uint8_t* 
     while (left) {
       const uint32_t n = min(left, kFlush);
       room(n);
-      for (uint32_t i = lane; i < n; i += 32) S.buf[w.cur + i] = __ldg(lits + i);
+      for (uint32_t i = lane; i < n; i += 32) buf[w.cur + i] = __ldg(lits + i);
       __syncwarp();
       w.cur += n;
       w.g0 += n;
       lits += n;
       left -= n;
-      flush(S, w, out_blk, vec_ok);
+      flush(buf, w, out_blk, vec_ok, lane, 32);
     }
     if (ml) {
       room(ml);
       for (uint32_t i = lane; i < ml; i += 32) {
         // an overlapping copy repeats the dist bytes before it
         const uint32_t src = w.g0 - dist + (dist < ml ? i % dist : i);
-        S.buf[w.cur + i] = src >= w.base ? S.buf[src - w.base] : (uint8_t)__ldcg(out_blk + src);
+        buf[w.cur + i] = src >= w.base ? buf[src - w.base] : (uint8_t)__ldcg(out_blk + src);
       }
       __syncwarp();
       w.cur += ml;
       w.g0 += ml;
-      flush(S, w, out_blk, vec_ok);
+      flush(buf, w, out_blk, vec_ok, lane, 32);
     }
   }
 }
@@ -778,7 +818,7 @@ __device__ __forceinline__ void lz_block(TileSmem& SS, const BlockView& V, int32
     }
     if (BYTE && G.slow) {
       cp_async_wait<0>();
-      slow_group(S, w, recs, t_cur, min(t_cur + 32u, V.n_seq), lits + litpos, out_blk, vec_ok);
+      slow_group(S.buf, kBuf, kHist, w, recs, t_cur, min(t_cur + 32u, V.n_seq), lits + litpos, out_blk, vec_ok);
       litpos += G.lits;
       G = Group{0, 0, 0, 0, false};
     }
@@ -797,26 +837,17 @@ __device__ __forceinline__ void lz_block(TileSmem& SS, const BlockView& V, int32
     cp_async_commit();
     cp_async_wait<1>();
     __syncwarp();
-    if (G.shift) slide(S, w, G.shift);
+    if (G.shift) slide(S.buf, w, G.shift);
     tiles(G, w.cur, stage ^ 1);
     w.g0 += G.total;
     w.cur += G.total;
     litpos += G.lits;
-    flush(S, w, out_blk, vec_ok);
+    flush(S.buf, w, out_blk, vec_ok, lane, 32);
     G = N;
   }
   cp_async_wait<0>();
   __syncwarp();
-  // what is not flushed yet
-  {
-    uint32_t c = w.flushed;
-    if (vec_ok) {
-      for (uint32_t x = c + 16u * lane; x + 16u <= w.g0; x += 512u)
-        *reinterpret_cast<uint4*>(out_blk + x) = *reinterpret_cast<const uint4*>(S.buf + (x - w.base));
-      c = w.g0 & ~15u;
-    }
-    for (c += lane; c < w.g0; c += 32u) out_blk[c] = S.buf[c - w.base];
-  }
+  flush_rest(S.buf, w, out_blk, vec_ok, lane, 32);
   if ((w.g0 != V.out_bytes || (BYTE && litpos != V.n_lit)) && lane == 0) set_status(status, GMP_STATUS_OUTPUT_OVERRUN);
 }
 
@@ -849,6 +880,17 @@ __device__ __forceinline__ uint32_t find_file(const KParams& P, uint64_t item) {
   return lo;
 }
 
+// A launch whose number of blocks only the device knows is made twice, a CTA
+// per block and a warp per block, and one of the two returns at once.  True if
+// this launch is to be the former: up to coop_max blocks, twice as many when
+// the (first) stream has Byte blocks, whose chains have no phase A.
+__device__ __forceinline__ bool takes_coop(const KParams& P, uint64_t total) {
+  const gmp_file_desc F = P.files ? P.files[0] : P.single;
+  bool byte_fmt = false;
+  if (F.n_blocks && F.comp_bytes >= 64 && !(((uintptr_t)F.comp) & 3u)) byte_fmt = !((ld_u32_nc(F.comp + 4) >> 16) & 2u);
+  return total <= (uint64_t)P.coop_max * (byte_fmt ? 2u : 1u);
+}
+
 // Persistent kernel: warps take blocks until none are left (the first one
 // fixed and interleaved over the CTAs when P.spread, as in gmp_decode.cu).
 template <bool PIPE>
@@ -859,6 +901,7 @@ __global__ void __launch_bounds__(512, 1) tile_kernel(const KParams P) {
   const uint64_t gw = (uint64_t)blockIdx.x * (blockDim.x >> 5) + warp;
   uint8_t* slot = P.scratch + gw * P.slot_bytes;
   const uint64_t total = P.files ? P.item_start[P.n_files] : P.single.n_blocks;
+  if (P.coop_max && takes_coop(P, total)) return;
   const unsigned long long fixed = P.spread ? (unsigned long long)gridDim.x * (blockDim.x >> 5) : 0ull;
   unsigned long long item = 0;
   if (P.spread) {
@@ -891,11 +934,481 @@ __global__ void __launch_bounds__(512, 1) tile_kernel(const KParams P) {
     pipeline_exit(P.exited, P.out_ready, P.gen, P.files ? P.n_files : 1u, gridDim.x * (blockDim.x >> 5));
 }
 
+// ---------------------------------------------------------------------------
+// A block by a CTA of W warps, for launches with too few blocks to fill the
+// GPU with a warp for each.  Phase A deals the sub-blocks out over the warps
+// (fewer lanes per warp: fewer paths and table conflicts per step) with
+// tables of 12 bits, which leave no long codes.  Phase B takes W groups at a
+// time, a warp each.  The window holds everything a match may reach, so that
+// nothing is staged.  The W groups' bytes (a wave) are written at once: each
+// byte whose source lies below the wave is copied, the others note their
+// source's place in the wave, and after a barrier follow it from byte to
+// byte; a byte's note is replaced by its source's until that one is a value
+// (pointer doubling), so that a chain of k copies takes about log2 k looks.
+// What bounds it is latency: of a 256 KiB block of CSV rows' 0.31 ms with 16
+// warps, about half is the chain of 1,000 Huffman steps in a lane (about 300
+// cycles each), half 34 waves of four dependent parts (scan, lay out and copy,
+// follow, flush).  One warp took 1.55 ms for it: 16 KiB 156 -> 51 us, 1 MiB of
+// 64 KiB blocks 754 -> 195, 16 MiB of records 1554 -> 310, 64 MiB of text 1599
+// -> 548, 128 MiB of Byte records 1541 -> 540.
+constexpr uint32_t kLitWave = 1984;  // most literal bytes of a wave of a Byte block
+constexpr uint32_t kLitRing = 4096;  // literal bytes of a Byte block held; the first kLitOver again at the end
+constexpr uint32_t kLitOver = 1024;
+constexpr uint32_t kCoopRecs = 2;  // a lane's records of a group
+constexpr uint32_t kCoopGroupMax = kCoopRecs * kGroupMax;
+// most output bytes of a wave (a group of text or of CSV rows is about 520)
+__host__ __device__ constexpr uint32_t wave_bytes(int W) { return 768 * W; }
+__host__ __device__ constexpr uint32_t coop_buf(int W) { return 32768 + 16 + wave_bytes(W) + (W <= 8 ? 4096 : 32768); }
+constexpr uint32_t kFollow = 12;  // tiles followed at once
+constexpr uint32_t kValue = 0x8000;  // note: bits 0-7 are the byte; else its source's place in the wave
+static_assert(kCoopGroupMax <= wave_bytes(8) && wave_bytes(16) < kValue && 2 * kLitWave + 16 <= kLitRing, "wave sizes");
+
+struct CoopSmemA {
+  uint32_t ll[LUT_SIZE], off[LUT_SIZE];
+  uint32_t bits[MAX_SUB][4 * kChunksAhead];
+  BuildSmem build;
+  Canon coff;
+  uint32_t run_off[16];
+  uint16_t sorted_off[N_OFF + 2];
+  uint32_t sb_bit[MAX_SUB], sb_seq[MAX_SUB];
+};
+template <int W>
+struct CoopSmemB {
+  uint8_t lit[W][128 * kCoopRecs];
+  uint32_t seg[W][64 * kCoopRecs];
+  uint32_t mark[W][(kCoopGroupMax + 127) / 128 * 4];
+  uint8_t blit[kLitRing + kLitOver];
+  uint16_t note[wave_bytes(W)];
+  uint8_t buf[coop_buf(W) + 160];  // a last batch of tiles may read up to 127 bytes past the wave
+};
+template <int W>
+struct __align__(64) CoopSmem {
+  union {
+    CoopSmemA a;
+    CoopSmemB<W> b;
+  } u;
+  uint32_t sb_out[MAX_SUB], sb_cnt[MAX_SUB];
+  uint32_t tot[2][W], tot_l[2][W];  // each group's output bytes; literal bytes of Byte blocks
+  Window win;          // after a slow group
+  int32_t result[3];   // of the parts of the table build
+  uint32_t bad;        // Byte: lowest warp << 8 | status of a failed check, else ~0
+  unsigned long long item;
+};
+
+__device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
+  uint16_t v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void sts_u16(uint32_t a, uint32_t v) {
+  asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)v) : "memory");
+}
+
+__device__ __forceinline__ void sts_u8_if(uint32_t a, uint32_t v, bool on) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p st.shared.u8 [%0], %1;\n}\n" ::"r"(a), "r"(v),
+               "r"((uint32_t)on)
+               : "memory");
+}
+__device__ __forceinline__ void sts_u16_if(uint32_t a, uint32_t v, bool on) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p st.shared.u16 [%0], %1;\n}\n" ::"r"(a),
+               "h"((uint16_t)v), "r"((uint32_t)on)
+               : "memory");
+}
+
+// Phase A of one block by the CTA; false: the block's status is set.
+template <int W>
+__device__ bool coop_huffman(CoopSmem<W>& S, const BlockView& V, int32_t* status, uint2* rec) {
+  const uint32_t t = threadIdx.x, warp = t >> 5, lane = lane_id();
+  CoopSmemA& A = S.u.a;
+  BuildSmem& T = A.build;
+  const uint32_t bs_off = (192u + 12u * V.K + 15u) & ~15u;  // bitstream start within the block
+  unpack_lens(T.lens, V.B, t, 32 * W);
+  __syncthreads();
+  if (warp < 3) {
+    int r;
+    if (warp == 0) r = sub_block_table(V, (V.comp_bytes - bs_off) * 8ull, A.sb_bit, S.sb_out, A.sb_seq);
+    else if (warp == 1) r = build_canon(T.cll, T.run, T.sorted_ll, T.lens, N_LL);
+    else r = build_canon(A.coff, A.run_off, A.sorted_off, T.lens + N_LL, N_OFF);
+    if (lane == 0) S.result[warp] = r;
+  }
+  __syncthreads();
+  const int n_ll = S.result[1], n_off = S.result[2];
+  int err = S.result[0] ? S.result[0] : n_ll < 0 || n_off < 0 ? (int)GMP_STATUS_BAD_HEADER : 0;
+  if (err) {
+    if (t == 0) set_status(status, err);
+    return false;
+  }
+  fill_ll<LUT_BITS>(A.ll, T.cll, T.sorted_ll, n_ll == 0, V.max_match, t, 32 * W);
+  fill_off<LUT_BITS>(A.off, A.coff, A.sorted_off, n_off == 0, t, 32 * W);
+  __syncthreads();
+  const uint8_t* bs = V.B + bs_off;
+  const uint32_t n_chunks = (uint32_t)min((uint64_t)0xffffffffu, (V.comp_bytes - bs_off) / 16);
+  // warps of phase A: lanes spread over more warps meet fewer paths and bank
+  // conflicts per step, but with several CTAs on an SM their instructions
+  // count (64 MiB of text, 8 warps: 0.92 ms with 8 of them, 0.60 with 4)
+  constexpr uint32_t HW = W == 16 ? 8 : 4;
+  const uint32_t j = warp < HW ? lane * HW + warp : MAX_SUB;
+  SubBlock sb{0, 0, 0, 0, 0, 0};
+  if (j < V.K) {
+    const uint8_t* e = V.B + 192 + 12 * j;
+    sb = SubBlock{A.sb_bit[j], ld_u32_nc(e), S.sb_out[j], ld_u32_nc(e + 4), A.sb_seq[j], ld_u32_nc(e + 8)};
+  }
+  const uint32_t cnt = huffman_lane<LUT_BITS, LUT_BITS, false>(
+      A.ll, A.off, A.coff, A.sorted_off, A.bits[min(j, (uint32_t)MAX_SUB - 1u)], bs, n_chunks, j < V.K, n_ll == 0,
+      sb, V.n_seq, V.window, rec + rec_start(sb.out, j), err);
+  if (j < V.K) S.sb_cnt[j] = cnt;
+  if (err) set_status(status, err);
+  return !__syncthreads_or(err != 0);  // the records are visible to the whole CTA
+}
+
+template <int W, bool BYTE>
+__device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int32_t* status, const uint2* rec,
+                                        uint8_t* out_blk) {
+  CoopSmemB<W>& S = SS.u.b;
+  constexpr uint32_t NT = 32 * W, CB = coop_buf(W), kWave = wave_bytes(W), R = kCoopRecs, GR = 32 * R;
+  const uint32_t t = threadIdx.x, warp = t >> 5, lane = lane_id();
+  const uint32_t le = (2u << lane) - 1u;
+  const bool vec_ok = (((uintptr_t)out_blk) & 15u) == 0;
+  const uint8_t* recs = V.B + 16;         // Byte blocks: the stream's records
+  const uint8_t* lits = V.B + V.lit_off;  // and literals
+  const uint32_t buf_a = smem_addr(S.buf), note_a = smem_addr(S.note);
+  // kept below a wave: what a match reaches, and what is not flushed
+  const uint32_t hist = max((V.window + 15u) & ~15u, kFlush);
+
+  // groups of GR records: the block's for Byte blocks, else each sub-block's
+  uint32_t n_groups;
+  if (BYTE) {
+    n_groups = V.n_seq / GR + (V.n_seq % GR ? 1u : 0u);
+  } else {
+    uint32_t g = 0;
+    for (uint32_t j = lane; j < V.K; j += 32) g += (SS.sb_cnt[j] + GR - 1u) / GR;
+    n_groups = __reduce_add_sync(FULL, g);
+  }
+  // the warp's group: record i0 of sub-block j (whose records start at rec_j)
+  uint32_t j = 0, i0 = GR * warp, n_j = BYTE ? V.n_seq : SS.sb_cnt[0];
+  const uint2* rec_j = rec;
+  auto settle = [&]() {
+    if constexpr (!BYTE) {
+      if (i0 < n_j) return;
+      while (j < V.K) {
+        const uint32_t whole = (n_j + GR - 1u) / GR * GR;
+        if (i0 < whole) break;
+        i0 -= whole;
+        j++;
+        n_j = j < V.K ? SS.sb_cnt[j] : 0u;
+      }
+      if (j < V.K) rec_j = rec + rec_start(SS.sb_out[j], j);
+    }
+  };
+  // the lane's R adjacent records: {literals, distance | match length << 16 |
+  // literal count << 24}, Byte blocks {-, the stream's word}; zero past the end
+  struct Recs {
+    uint2 r[R];
+  };
+  auto load = [&]() -> Recs {
+    const uint32_t i = i0 + R * lane;
+    Recs x;
+#pragma unroll
+    for (uint32_t k = 0; k < R; k++) x.r[k] = make_uint2(0, 0);
+    if (BYTE) {
+#pragma unroll
+      for (uint32_t k = 0; k < R; k++)
+        if (i + k < n_j) x.r[k].y = ld_u32_nc(recs + 4ull * (i + k));
+    } else {
+      // whole pairs: a sub-block's records have room for one more
+      if (i < n_j) {
+        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(rec_j + i));
+        x.r[0] = make_uint2(v.x, v.y);
+        if (i + 1u < n_j) x.r[R - 1] = make_uint2(v.z, v.w);
+      }
+    }
+    return x;
+  };
+  rec_j = BYTE ? rec : rec + rec_start(SS.sb_out[0], 0);
+  settle();
+  Recs r = load();
+
+  // Byte literals: a ring of kLitRing bytes filled at each wave's start for
+  // the waves after it
+  uint32_t litpos = 0, lit_asked = 0;
+  auto fill = [&]() {
+    const uint32_t upto = min((V.n_lit + 15u) & ~15u, (litpos & ~15u) + kLitRing);
+    for (uint32_t c = lit_asked + 16u * t; c < upto; c += 16u * NT) {
+      const uint32_t at = c & (kLitRing - 1u);
+      cp_async16(S.blit + at, lits + c);
+      if (at < kLitOver) cp_async16(S.blit + kLitRing + at, lits + c);
+    }
+    lit_asked = max(lit_asked, upto);
+  };
+  if (t == 0) SS.bad = ~0u;
+  if (BYTE) fill();
+
+  Window w{0, 0, 0, 0};  // at the wave's start; the same in every thread
+  for (uint32_t it = 0; it * W < n_groups; it++) {
+    // lengths of the lane's records; one scan gives output positions and (from
+    // bit 20) the number of the segments before
+    uint32_t ll[R], ml[R], dist[R], own = 0, own_l = 0, inc_l = 0;
+#pragma unroll
+    for (uint32_t k = 0; k < R; k++) {
+      const uint32_t y = r.r[k].y;
+      if (BYTE) {
+        const uint32_t m = (y >> 10) & 63u;
+        ll[k] = y & 1023u;
+        ml[k] = m ? m + 2u : 0u;  // code 63 has no length; as 65 it fails the check below
+        dist[k] = (y >> 16) + 1u;
+      } else {
+        ll[k] = y >> 24;
+        ml[k] = (y >> 16) & 255u;
+        dist[k] = y & 0xffffu;
+        *reinterpret_cast<uint32_t*>(S.lit[warp] + 4u * (R * lane + k)) = r.r[k].x;
+      }
+      own += ll[k] + ml[k] + (ll[k] ? 1u << 20 : 0u) + (ml[k] ? 1u << 20 : 0u);
+      own_l += ll[k];
+    }
+    const uint32_t inc = warp_incl_scan(own);
+    const uint32_t dst0 = (inc - own) & 0xfffffu, seg0 = (inc - own) >> 20;
+    const uint32_t total = __shfl_sync(FULL, inc, 31) & 0xfffffu;
+    if (lane == 0) SS.tot[it & 1u][warp] = total;
+    if (BYTE) {
+      inc_l = warp_incl_scan(own_l);
+      if (lane == 31) SS.tot_l[it & 1u][warp] = inc_l;
+    }
+    const uint32_t t_cur = i0;  // the group's first record
+    i0 += GR * W;
+    settle();
+    r = load();
+    if (BYTE) cp_async_wait<0>();
+    __syncthreads();  // the wave before is complete, the totals are known
+    const uint32_t T_i = lane < (uint32_t)W ? SS.tot[it & 1u][lane] : 0u;
+    const uint32_t L_i = BYTE && lane < (uint32_t)W ? SS.tot_l[it & 1u][lane] : 0u;
+    const bool slow_i = BYTE && (T_i > kCoopGroupMax || L_i > kLitWave);
+    for (uint32_t lo = 0; lo < (uint32_t)W;) {
+      // the wave: as many of the groups from lo on as fit, all of them as a rule
+      uint32_t hi = W, sum = __reduce_add_sync(FULL, lane >= lo ? T_i : 0u);
+      uint32_t sum_l = BYTE ? __reduce_add_sync(FULL, lane >= lo ? L_i : 0u) : 0u;
+      bool slow = false;
+      if (sum > kWave || (BYTE && (sum_l > kLitWave || __any_sync(FULL, slow_i)))) {
+        const uint32_t s_t = warp_incl_scan(lane >= lo ? T_i : 0u), s_l = BYTE ? warp_incl_scan(lane >= lo ? L_i : 0u) : 0u;
+        const uint32_t fit = __ballot_sync(FULL, lane >= lo && !slow_i && s_t <= kWave && s_l <= kLitWave);
+        const uint32_t out = ~(fit >> lo);
+        hi = min(lo + (out ? (uint32_t)__ffs(out) - 1u : 32u), (uint32_t)W);
+        slow = hi == lo;
+        if (slow) hi = lo + 1;
+        sum = __shfl_sync(FULL, s_t, hi - 1);
+        if (BYTE) sum_l = __shfl_sync(FULL, s_l, hi - 1);
+      }
+      const uint32_t pre = __reduce_add_sync(FULL, lane >= lo && lane < warp ? T_i : 0u);
+      const uint32_t pre_l = BYTE ? __reduce_add_sync(FULL, lane >= lo && lane < warp ? L_i : 0u) : 0u;
+      const bool mine = warp >= lo && warp < hi;
+      if (lo) {
+        if (BYTE) cp_async_wait<0>();
+        __syncthreads();  // the wave before is complete
+      }
+      flush(S.buf, w, out_blk, vec_ok, t, NT);
+      if (!slow && w.cur + sum > CB) {
+        // strips as in slide(), every thread's loads before any store
+        const uint32_t shift = (w.cur - hist) & ~15u, n = w.cur - shift;
+        for (uint32_t u = 0; u < n; u += 16u * NT) {
+          const uint32_t c = u + 16u * t;
+          uint4 v = make_uint4(0, 0, 0, 0);
+          if (c < n) v = *reinterpret_cast<const uint4*>(S.buf + shift + c);
+          __syncthreads();
+          if (c < n) *reinterpret_cast<uint4*>(S.buf + c) = v;
+        }
+        w.cur -= shift;
+        w.base += shift;
+        __syncthreads();
+      }
+      int err = 0;  // a group that fails its checks is neither laid out nor copied
+      if (BYTE && mine) {
+        bool long_match = false, far = false;
+        uint32_t at = w.g0 + pre + dst0;
+#pragma unroll
+        for (uint32_t k = 0; k < R; k++) {
+          at += ll[k];
+          long_match = long_match || ml[k] > V.max_match;
+          far = far || (ml[k] > 0 && (dist[k] > V.window || dist[k] > at));
+          at += ml[k];
+        }
+        if (__any_sync(FULL, long_match)) err = GMP_STATUS_CORRUPT_SYMBOL;
+        else if (__any_sync(FULL, far)) err = GMP_STATUS_BAD_OFFSET;
+        else if ((uint64_t)w.g0 + pre + total > V.out_bytes ||
+                 (uint64_t)litpos + pre_l + __shfl_sync(FULL, L_i, warp) > V.n_lit)
+          err = GMP_STATUS_OUTPUT_OVERRUN;
+        if (err && lane == 0) atomicMin(&SS.bad, (warp << 8) | (uint32_t)err);
+      }
+      if (BYTE && slow) {
+        __syncthreads();
+        if (SS.bad != ~0u) break;
+        if (warp == lo) {
+          Window x = w;
+          slow_group(S.buf, CB, hist, x, recs, t_cur, min(t_cur + GR, V.n_seq), lits + litpos, out_blk, vec_ok);
+          if (lane == 0) SS.win = x;
+        }
+        __syncthreads();
+        w = SS.win;
+        litpos += sum_l;
+        lit_asked = litpos & ~15u;
+        fill();
+        lo = hi;
+        continue;
+      }
+      if (BYTE) fill();
+      const uint32_t wave_a = buf_a + w.cur;
+      if (mine && !err) {
+        // segment starts and entries, as in lz_block
+        uint32_t* mark = S.mark[warp];
+        uint32_t* seg = S.seg[warp];
+        for (uint32_t x = lane; x < ((total + 127u) >> 7) * 4u; x += 32) mark[x] = 0;
+        __syncwarp();
+        uint32_t at = dst0, n = seg0, lit_at = litpos + pre_l + inc_l - own_l;
+#pragma unroll
+        for (uint32_t k = 0; k < R; k++) {
+          if (ll[k]) {
+            atomicOr(mark + (at >> 5), 1u << (at & 31u));
+            seg[n++] = (BYTE ? smem_addr(S.blit) + (lit_at & (kLitRing - 1u))
+                             : smem_addr(S.lit[warp]) + 4u * (R * lane + k)) -
+                       at;
+          }
+          at += ll[k];
+          lit_at += ll[k];
+          if (ml[k]) {
+            atomicOr(mark + (at >> 5), 1u << (at & 31u));
+            seg[n++] = wave_a + pre - dist[k];
+          }
+          at += ml[k];
+        }
+        __syncwarp();
+        uint32_t before = 0xffffffffu;  // segments started before the tile, less one
+        for (uint32_t x = 0; x < total; x += 128) {
+          const uint4 m = *reinterpret_cast<const uint4*>(mark + (x >> 5));
+          const uint32_t c0 = before + __popc(m.x), c1 = c0 + __popc(m.y), c2 = c1 + __popc(m.z);
+          const uint32_t o = x + lane;
+          const uint32_t a0 = seg[before + __popc(m.x & le)] + o, a1 = seg[c0 + __popc(m.y & le)] + o + 32u;
+          const uint32_t a2 = seg[c1 + __popc(m.z & le)] + o + 64u, a3 = seg[c2 + __popc(m.w & le)] + o + 96u;
+          before = c2 + __popc(m.w);
+          auto put = [&](uint32_t a, uint32_t at) {
+            const bool in = at < total, follow = a >= wave_a;
+            const uint32_t v = lds_u8(a);
+            sts_u16_if(note_a + 2u * (pre + at), follow ? a - wave_a : kValue | v, in);
+            sts_u8_if(wave_a + pre + at, v, in && !follow);
+          };
+          put(a0, o);
+          put(a1, o + 32u);
+          put(a2, o + 64u);
+          put(a3, o + 96u);
+        }
+      }
+      __syncthreads();  // every byte of the wave is written or noted
+      if (BYTE && SS.bad != ~0u) break;
+      if (mine) {
+        for (uint32_t x = lane; x < total + lane; x += 32u * kFollow) {
+          uint32_t v[kFollow], all = kValue, mine_to_write = 0;
+#pragma unroll
+          for (uint32_t i = 0; i < kFollow; i++) {
+            const bool in = x + 32u * i < total;
+            v[i] = lds_u16(in ? note_a + 2u * (pre + x + 32u * i) : note_a);
+            v[i] = in ? v[i] : kValue;
+            all &= v[i];
+            mine_to_write |= (v[i] & kValue) ? 0u : 1u << i;
+          }
+          // a source's note may still be a place, but only one below it, and
+          // the wave's lowest such byte always finds a value
+          for (uint32_t spin = 0; __any_sync(FULL, !all); spin++) {
+            if (spin == 1u << 20) {
+              if (lane == 0) set_status(status, GMP_STATUS_MRR_NO_PROGRESS);
+              break;
+            }
+            all = kValue;
+#pragma unroll
+            for (uint32_t i = 0; i < kFollow; i++) {
+              const bool on = !(v[i] & kValue);
+              const uint32_t n = lds_u16(on ? note_a + 2u * v[i] : note_a);
+              v[i] = on ? n : v[i];
+              all &= v[i];
+              sts_u16_if(note_a + 2u * (pre + x + 32u * i), v[i], on);
+            }
+          }
+#pragma unroll
+          for (uint32_t i = 0; i < kFollow; i++) sts_u8_if(wave_a + pre + x + 32u * i, v[i], (mine_to_write >> i) & 1u);
+        }
+      }
+      w.g0 += sum;
+      w.cur += sum;
+      litpos += sum_l;
+      lo = hi;
+    }
+    if (BYTE && SS.bad != ~0u) break;
+  }
+  if (BYTE) cp_async_wait<0>();
+  __syncthreads();
+  if (BYTE && SS.bad != ~0u) {
+    if (t == 0) set_status(status, (int)(SS.bad & 255u));
+    return;
+  }
+  flush_rest(S.buf, w, out_blk, vec_ok, t, NT);
+  if (t == 0 && (w.g0 != V.out_bytes || (BYTE && litpos != V.n_lit))) set_status(status, GMP_STATUS_OUTPUT_OVERRUN);
+}
+
+// Persistent kernel, a CTA of W warps per block.
+template <int W, bool PIPE>
+__global__ void __launch_bounds__(32 * W, W == 16 ? 1 : 3) coop_kernel(const KParams P) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  CoopSmem<W>& S = *reinterpret_cast<CoopSmem<W>*>(smem_raw);
+  const uint32_t t = threadIdx.x;
+  uint2* rec = reinterpret_cast<uint2*>(P.scratch + blockIdx.x * P.slot_bytes);
+  const uint64_t total = P.files ? P.item_start[P.n_files] : P.single.n_blocks;
+  if (P.coop_max && !takes_coop(P, total)) return;
+  unsigned long long item = blockIdx.x;
+  for (bool first = true;; first = false) {
+    if (!first || !P.spread) {
+      __syncthreads();
+      if (t == 0) S.item = (P.spread ? gridDim.x : 0u) + atomicAdd(P.counter, 1ull);
+      __syncthreads();
+      item = S.item;
+    }
+    if (item >= total) break;
+    uint32_t file = 0;
+    uint64_t b = item;
+    gmp_file_desc F = P.single;
+    if (P.files) {
+      file = find_file(P, item);
+      b = item - P.item_start[file];
+      F = P.files[file];
+    }
+    int32_t* status = P.status + file;
+    bool ok = true;
+    if (PIPE && P.in_ready) {
+      ok = wait_input(P.in_ready + file, P.abort_wait, P.gen, P.wait_ns);
+      ok = !__syncthreads_or(!ok);
+      if (!ok && t == 0) set_status(status, GMP_STATUS_INPUT_TIMEOUT);
+    }
+    if (ok) {
+      BlockView V;
+      int err = open_block(F, b, V);
+      if (!err && !V.byte_fmt && (V.out_bytes > P.max_out || V.n_seq > P.max_seq)) err = GMP_STATUS_CAPACITY;
+      if (err) {
+        if (t == 0) set_status(status, err);
+      } else if (V.byte_fmt) {
+        coop_lz<W, true>(S, V, status, rec, F.out + V.out_offset);
+      } else if (coop_huffman<W>(S, V, status, rec)) {
+        coop_lz<W, false>(S, V, status, rec, F.out + V.out_offset);
+      }
+    }
+    if (PIPE && P.out_ready) {
+      __threadfence();
+      __syncthreads();  // every thread's output is stored
+      if (t < 32) block_done(P.done + file, P.out_ready + file, P.gen, F.n_blocks);
+    }
+  }
+  if (PIPE && P.out_ready) pipeline_exit(P.exited, P.out_ready, P.gen, P.files ? P.n_files : 1u, gridDim.x * W);
+}
+
 }  // namespace
 
 uint64_t tile_slot_bytes(uint64_t max_out) {
   // rec_start of the last sub-block and its records
-  return ((max_out / 3 + 5ull * MAX_SUB + 8) * sizeof(uint2) + 255) & ~255ull;
+  return ((max_out / 3 + 7ull * MAX_SUB + 8) * sizeof(uint2) + 255) & ~255ull;
 }
 
 // The shared memory limit is per kernel and process-wide: always the widest
@@ -921,6 +1434,39 @@ cudaError_t launch_tile(const KParams& P, int grid, int warps_per_cta, bool pipe
   if (pipe) tile_kernel<true><<<grid, warps_per_cta * 32, smem, stream>>>(P);
   else tile_kernel<false><<<grid, warps_per_cta * 32, smem, stream>>>(P);
   return cudaGetLastError();
+}
+
+template <int W>
+static cudaError_t configure_coop() {
+  const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(coop_kernel<W, false>, a, (int)sizeof(CoopSmem<W>));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(coop_kernel<W, true>, a, (int)sizeof(CoopSmem<W>));
+  return e;
+}
+
+template <int W>
+static cudaError_t coop(const KParams& P, int grid, bool pipe, cudaStream_t stream) {
+  cudaError_t e = configure_coop<W>();
+  if (e != cudaSuccess) return e;
+  if (pipe) coop_kernel<W, true><<<grid, 32 * W, sizeof(CoopSmem<W>), stream>>>(P);
+  else coop_kernel<W, false><<<grid, 32 * W, sizeof(CoopSmem<W>), stream>>>(P);
+  return cudaGetLastError();
+}
+
+cudaError_t coop_occupancy(int warps, int* ctas_per_sm) {
+  if (warps == 16) {
+    const cudaError_t e = configure_coop<16>();
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, coop_kernel<16, false>, 512,
+                                                         sizeof(CoopSmem<16>));
+  }
+  const cudaError_t e = configure_coop<8>();
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, coop_kernel<8, false>, 256, sizeof(CoopSmem<8>));
+}
+
+cudaError_t launch_coop(const KParams& P, int grid, int warps, bool pipe, cudaStream_t stream) {
+  return warps == 16 ? coop<16>(P, grid, pipe, stream) : coop<8>(P, grid, pipe, stream);
 }
 
 }  // namespace gmp
