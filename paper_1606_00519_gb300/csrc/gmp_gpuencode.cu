@@ -10,10 +10,8 @@
 //
 //  plan_kernel, one CTA per block:
 //   - checks every token against its block;
-//   - frequencies of both alphabets: the literal/length histogram is the
-//     histogram of all the block's bytes, minus the bytes that
-//     back-references cover, plus one match-length or end symbol per token,
-//     so that long literal runs spread over the CTA;
+//   - frequencies of both alphabets (long literal strings are counted by a
+//     warp each, so that they spread over the CTA);
 //   - code lengths limited to cwl bits per tree (one warp each): Huffman
 //     code lengths by the two-queue method (van Leeuwen, 1976) on the
 //     symbols sorted by frequency, then limited to cwl bits by the
@@ -24,13 +22,15 @@
 //     (a token costs its literals + 1 lookups): a scan of per-thread token
 //     costs and, per sub-block, a search for the token where the running
 //     cost reaches (j + 1) / K of the total;
-//   - the bits of every sub-block (the same decomposition: code bits of all
-//     bytes of its output range, minus those of the bytes back-references
-//     cover, plus each token's length, offset and extra bits), hence the
-//     block's encoded size.
+//   - the bits of every sub-block, hence the block's encoded size, and of
+//     every share: the block's tokens in kEncThreads runs of equal work, each
+//     with its bit offset, since sub-blocks follow each other without gaps.
+//  Counting every byte and taking off those under back-references, and one
+//  thread per sub-block in write_kernel, took 4.0 ms for 64 MiB of text (256
+//  blocks of 32 sub-blocks); with literals counted and a thread per share 1.2.
 //  write_kernel, one CTA per block at the offset the host computed from the
 //   sizes: the block header (code lengths, sub-block table), canonical codes
-//   (Sec. 3.1) from the lengths, then thread j packs sub-block j's codes
+//   (Sec. 3.1) from the lengths, then thread j packs share j's codes
 //   LSB-first at its bit offset (the words it shares with its neighbours by
 //   atomicOr, the others by plain stores).
 //  Byte blocks (Gompresso/Byte) get their 4-byte records and literal bytes
@@ -44,7 +44,8 @@
 namespace gmp {
 namespace {
 
-constexpr int kEncThreads = 256;
+constexpr int kEncThreads = kEncShares;
+constexpr uint32_t kMaxLong = 1024;  // literal strings of a block that are counted by a warp each
 constexpr int kMaxDepth = 64;
 constexpr uint32_t kNLL = kLitLenSyms, kNOff = kOffsetSyms;
 constexpr uint32_t kSymEnd = 256;
@@ -70,6 +71,9 @@ struct PlanSmem {
   TreeWS ws[2];
   unsigned long long total_cost;
   uint32_t n_lit, err;
+  uint32_t share[kEncThreads + 1];  // first token of each share
+  uint32_t share_bits[kEncThreads];
+  uint32_t longs[kMaxLong], n_long;
 };
 
 // Distance code of the stream format: symbol, extra bit count and extra bits
@@ -205,14 +209,20 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
     const uint32_t K = E.byte_mode ? 0u : E.n_sub;
     for (uint32_t i = tid; i < kNLL + 1; i += kEncThreads) S.h1[i] = 0;
     if (tid < kNOff + 2) S.h2[tid] = 0;
-    if (tid == 0) S.err = (n == 0 || n > E.stride) ? 1u : 0u;
+    if (tid == 0) {
+      S.err = (n == 0 || n > E.stride) ? 1u : 0u;
+      S.n_long = 0;
+    }
+    S.share_bits[tid] = 0;
     __syncthreads();
     const uint32_t nn = min(n, (uint32_t)E.stride);
     const uint32_t C = (nn + kEncThreads - 1) / kEncThreads;
     const uint32_t k0 = min(tid * C, nn), k1 = min(k0 + C, nn);
-    // pass 1 over the thread's tokens: checks, work and literal counts, the
-    // symbol frequencies, and the bytes under back-references out of the
-    // byte histogram
+    // literal strings from this length on are left to the warps (there are at
+    // most kMaxLong of them)
+    const uint32_t long_lit = max(256u, (len + kMaxLong - 1) / kMaxLong);
+    // pass 1 over the thread's tokens: checks, work and literal counts, and
+    // the symbol frequencies
     unsigned long long cost = 0;
     uint32_t lits = 0;
     bool bad = false;
@@ -236,19 +246,27 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
           dist_symbol(d, sym, ne, ex);
           atomicAdd(&S.h1[254 + ml], 1u);
           atomicAdd(&S.h2[sym], 1u);
-          const uint8_t* src = blk + p + ll;
-          for (uint32_t i = 0; i < ml; i++) atomicSub(&S.h1[src[i]], 1u);
         } else {
           atomicAdd(&S.h1[kSymEnd], 1u);
+        }
+        if (ll < long_lit) {
+          for (uint32_t i = 0; i < ll; i++) atomicAdd(&S.h1[blk[p + i]], 1u);
+        } else {
+          S.longs[min(atomicAdd(&S.n_long, 1u), kMaxLong - 1u)] = k;
         }
       }
     }
     S.csum[tid] = cost;
     S.lsum[tid] = lits;
     if (bad) atomicOr(&S.err, 1u);
-    if (!E.byte_mode)
-      for (uint32_t x = tid; x < len; x += kEncThreads) atomicAdd(&S.h1[blk[x]], 1u);
     __syncthreads();
+    // (tokens that fail their checks may not lie in the block)
+    if (!S.err) {
+      for (uint32_t i = warp; i < S.n_long; i += kEncThreads / 32) {
+        const uint32_t k = S.longs[i], ll = t[k].lit_len, p = tp[k];
+        for (uint32_t x = tid & 31u; x < ll; x += 32) atomicAdd(&S.h1[blk[p + x]], 1u);
+      }
+    }
     if (tid == 0) {
       unsigned long long rc = 0;
       uint32_t rl = 0;
@@ -312,6 +330,17 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
       }
       S.g[tid] = T > 0 ? g : 0xffffffffu;  // T = 0: the sub-block is empty
     }
+    {
+      // shares, likewise: the first token whose running cost passes tid / 256
+      // of the total
+      const unsigned long long T = S.total_cost * tid / kEncThreads;
+      const uint32_t c = last_le<unsigned long long>(S.csum, kEncThreads, T);
+      unsigned long long run = S.csum[c];
+      uint32_t k = min(c * C, nn);
+      for (const uint32_t c1 = min(k + C, nn); k < c1 && run < T; k++) run += t[k].lit_len + 1ull;
+      S.share[tid] = k;
+      if (tid == 0) S.share[kEncThreads] = nn;
+    }
     __syncthreads();
     if (tid == 0) {
       uint32_t qi = 0;
@@ -329,49 +358,43 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
     if (tid <= K) S.so[tid] = S.qs[tid] < nn ? tp[S.qs[tid]] : len;
     if (tid < K) S.sbits[tid] = 0;
     __syncthreads();
-    // bits per sub-block: literal codes of every byte of its output range
-    // (a contiguous range of bytes per thread) ...
-    {
-      const uint32_t L = (len + kEncThreads - 1) / kEncThreads;
-      const uint32_t x0 = min(tid * L, len), x1 = min(x0 + L, len);
-      if (x0 < x1) {
-        uint32_t j = last_le<uint32_t>(S.so, K, x0);
-        long long acc = 0;
-        for (uint32_t x = x0; x < x1; x++) {
-          while (j + 1 < K && x >= S.so[j + 1]) {
-            atomicAdd(&S.sbits[j], (unsigned long long)acc);
-            acc = 0;
-            j++;
-          }
-          acc += S.lens[blk[x]];
-        }
-        atomicAdd(&S.sbits[j], (unsigned long long)acc);
+    // bits of each sub-block and each share: the long literal strings, a warp
+    // each, then each thread's share
+    for (uint32_t i = warp; i < S.n_long; i += kEncThreads / 32) {
+      const uint32_t k = S.longs[i], ll = t[k].lit_len, p = tp[k];
+      uint32_t bits = 0;
+      for (uint32_t x = tid & 31u; x < ll; x += 32) bits += S.lens[blk[p + x]];
+      bits = __reduce_add_sync(0xffffffffu, bits);
+      if ((tid & 31u) == 0) {
+        atomicAdd(&S.sbits[last_le<uint32_t>(S.qs, K, k)], (unsigned long long)bits);
+        atomicAdd(&S.share_bits[last_le<uint32_t>(S.share, kEncThreads, k)], bits);
       }
     }
-    // ... minus the bytes under back-references, plus each token's length
-    // or end code and its offset code and extra bits
-    if (k0 < k1) {
-      uint32_t j = last_le<uint32_t>(S.qs, K, k0);
-      while (j + 1 < K && S.qs[j + 1] <= k0) j++;  // empty sub-blocks share a start
-      long long acc = 0;
-      for (uint32_t k = k0; k < k1; k++) {
+    const uint32_t w0 = S.share[tid], w1 = S.share[tid + 1];
+    if (w0 < w1) {
+      uint32_t j = last_le<uint32_t>(S.qs, K, w0), all = 0, acc = 0;
+      for (uint32_t k = w0; k < w1; k++) {
         while (j + 1 < K && k >= S.qs[j + 1]) {
           atomicAdd(&S.sbits[j], (unsigned long long)acc);
+          all += acc;
           acc = 0;
           j++;
         }
         const uint32_t ll = t[k].lit_len, ml = t[k].match & 0xffu, d = t[k].match >> 8;
+        if (ll < long_lit) {
+          const uint8_t* src = blk + tp[k];
+          for (uint32_t i = 0; i < ll; i++) acc += S.lens[src[i]];
+        }
         if (ml) {
           uint32_t sym, ne, ex;
           dist_symbol(d, sym, ne, ex);
-          acc += (long long)S.lens[254 + ml] + S.lens[kNLL + sym] + ne;
-          const uint8_t* src = blk + tp[k] + ll;
-          for (uint32_t i = 0; i < ml; i++) acc -= S.lens[src[i]];
+          acc += S.lens[254 + ml] + S.lens[kNLL + sym] + ne;
         } else {
           acc += S.lens[kSymEnd];
         }
       }
       atomicAdd(&S.sbits[j], (unsigned long long)acc);
+      atomicAdd(&S.share_bits[tid], all + acc);
     }
     __syncthreads();
     if (tid < K) {
@@ -380,7 +403,14 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
       P.sub_bits[tid] = S.sbits[tid];
     }
     for (uint32_t i = tid; i < kNLL + kNOff; i += kEncThreads) P.lens[i] = S.lens[i];
+    P.share_first[tid] = S.share[tid];
     if (tid == 0) {
+      P.share_first[kEncThreads] = nn;
+      uint32_t at = 0;
+      for (int c = 0; c < kEncThreads; c++) {
+        P.share_bit[c] = at;
+        at += S.share_bits[c];
+      }
       unsigned long long bits = 0;
       for (uint32_t j = 0; j < K; j++) bits += S.sbits[j];
       P.sub_first[K] = nn;
@@ -486,14 +516,14 @@ __global__ void __launch_bounds__(kEncThreads) write_kernel(const EncParams E, c
       }
     }
     __syncthreads();
-    if (tid < K) {
-      // sub-block tid's bits, from its bit offset in the block's bitstream
-      uint64_t start = 0;
-      for (uint32_t j = 0; j < tid; j++) start += P.sub_bits[j];
+    const uint32_t w0 = P.share_first[tid], w1 = P.share_first[tid + 1];
+    if (w0 < w1) {
+      // the share's bits, from its bit offset in the block's bitstream
+      const uint32_t start = P.share_bit[tid];
       uint32_t* W = reinterpret_cast<uint32_t*>(dst + hdr);
-      uint64_t w = start >> 5;
+      uint32_t w = start >> 5;
       unsigned long long acc = 0;
-      uint32_t na = (uint32_t)(start & 31u);
+      uint32_t na = start & 31u;
       bool first = true;
       auto put = [&](uint32_t bits, uint32_t nb) {
         acc |= (unsigned long long)bits << na;
@@ -507,7 +537,7 @@ __global__ void __launch_bounds__(kEncThreads) write_kernel(const EncParams E, c
           na -= 32;
         }
       };
-      for (uint32_t k = P.sub_first[tid]; k < P.sub_first[tid + 1]; k++) {
+      for (uint32_t k = w0; k < w1; k++) {
         const uint32_t ll = t[k].lit_len, ml = t[k].match & 0xffu, d = t[k].match >> 8;
         const uint8_t* src = blk + tp[k];
         for (uint32_t i = 0; i < ll; i++) {

@@ -80,12 +80,16 @@ struct ParseToken {
 // GPU entropy coding of GPU parses (gmp_gpuencode.cu): per block, a plan
 // (token checks, code lengths, sub-block split and sizes), then the block's
 // bytes at an offset computed from the planned sizes.
+constexpr uint32_t kEncShares = 256;
 struct EncBlockPlan {
   uint64_t bytes, bits;  // encoded size (a multiple of 16), bitstream bits
   uint32_t n_seq, out_bytes, n_lit, err;
   uint32_t sub_first[kMaxSub + 1];  // first token of each sub-block; [K] = n_seq
   uint32_t sub_out[kMaxSub];        // output bytes of each sub-block
   uint64_t sub_bits[kMaxSub];       // bits of each sub-block
+  // the tokens in kEncShares runs of about equal work, a writing thread each:
+  // first token, first bit
+  uint32_t share_first[kEncShares + 1], share_bit[kEncShares];
   uint8_t lens[kLitLenSyms + kOffsetSyms];
 };
 struct EncLaunch {
