@@ -8,23 +8,27 @@
 // gmp_compress.  The host only lays out the blocks from their sizes and
 // writes the 64-byte file header and the block offset table.
 //
-//  match_kernel: one CTA per block.  The CTA walks the block 512 positions
-//  at a time, one per thread, with the block's bytes streaming through a ring
-//  in shared memory.  Hash-chain heads of 3-byte prefixes and the chain
-//  links are in shared memory too; each thread follows its bucket's chain
-//  for up to chain_depth candidates within the window, keeps the longest
-//  match (at most max_match bytes) and stores its length and distance; then
-//  every position of the step is linked in.  Lookups of a step see only
-//  positions of earlier steps, so a candidate always lies before its
-//  position, in the same block.
-//  parse_kernel: one warp per block stages the per-position matches in
-//  shared memory and lane 0 walks them from the block start: a match of at
+//  chain_kernel: a CTA per block walks it 512 positions at a time, one per
+//  thread, and writes each position's link: the distance to the latest
+//  position of an earlier step with the same hash of its 3-byte prefix (0 =
+//  none).  Positions of one step do not see each other, so every chain runs
+//  through at most one position of a step.
+//  search_kernel: given the links, every position's search is independent.  A
+//  CTA takes a run of positions of one block, with the window before them and
+//  all their links in shared memory.  A lane follows its position's chain for
+//  up to chain_depth candidates within the window, keeps the longest match (at
+//  most max_match bytes, the nearest of equals) and stores its length and
+//  distance; then it takes the next position of its warp's share, so that
+//  lanes whose chains are short do not wait for the longest one.
+//  parse_kernel: a CTA per block parses it from its start: a match of at
 //  least 3 bytes is taken unless the next position has a longer one
-//  (one-step lazy evaluation), otherwise the byte becomes a literal.  For DE
-//  streams a candidate is cut at the first source byte that an earlier
-//  back-reference of the same 32-sequence group writes, as in gmp_compress;
-//  for Byte streams literal strings are cut into runs of at most 1023
-//  bytes, which count as sequences of their group.
+//  (one-step lazy evaluation), otherwise the byte becomes a literal.  What
+//  follows from the matches alone is worked out for every position at once,
+//  so that one thread has one lookup to do per token.  For DE streams a
+//  candidate is cut at the first source byte that an earlier back-reference
+//  of the same 32-sequence group writes, as in gmp_compress; for Byte streams
+//  literal strings are cut into runs of at most 1023 bytes, which count as
+//  sequences of their group.
 //  Every token's position in its block is written beside it for the
 //  entropy coder.
 //
@@ -44,115 +48,156 @@ namespace {
 
 constexpr uint32_t kFull = 0xffffffffu;
 constexpr uint32_t kByteMaxLit = 1023;
-constexpr int kMatchThreads = 512;       // positions per step of the match search
+constexpr uint32_t kStep = 512;          // positions of one step do not see each other
 constexpr int kHeadBits = 12;            // hash buckets of 3-byte prefixes
-constexpr uint32_t kLinkRing = 32768;    // chain links kept (>= the window)
-constexpr uint32_t kInRing = 65536;      // input bytes kept (the window, a step and a match past it)
 constexpr uint32_t kLook = 64;           // longest match
+constexpr int kSearchThreads = 1024;
+constexpr int kSearchSmemMax = 3 * (32768 + 32768) + 64 + 64;  // window and run of 32 Ki positions
+constexpr uint32_t kShare = 128;         // positions that a warp takes at a time
+constexpr uint32_t kCompareAt = 10;      // lanes with a promising candidate that make the warp compare
+constexpr uint32_t kRefillAt = 6;        // idle lanes that make the warp deal out positions
 
-struct MatchSmem {
-  uint32_t head[1 << kHeadBits];  // per bucket: latest position + 1 of an earlier step, 0 = none
-  uint16_t link[kLinkRing];       // per position: distance to the bucket's previous position, 0 = none
-  uint8_t ring[kInRing];          // the block's bytes [loaded - kInRing, loaded)
-};
-
-// Bytes x .. x + 3 of the ring (positions taken modulo its size), the first
-// in the low byte: two aligned words and a funnel shift.
-__device__ __forceinline__ uint32_t ring_word(const uint8_t* ring, uint32_t x) {
-  constexpr uint32_t WM = kInRing / 4 - 1;
-  const uint32_t* r = reinterpret_cast<const uint32_t*>(ring);
-  const uint32_t wa = x >> 2;
-  return __funnelshift_r(r[wa & WM], r[(wa + 1) & WM], (x & 3u) * 8u);
+__device__ __forceinline__ uint32_t prefix_hash(uint32_t b012) {
+  return (b012 * 0x9E3779B1u) >> (32 - kHeadBits);
 }
 
-__device__ __forceinline__ uint32_t prefix_hash(uint32_t b0, uint32_t b1, uint32_t b2) {
-  return ((b0 | (b1 << 8) | (b2 << 16)) * 0x9E3779B1u) >> (32 - kHeadBits);
-}
-
-// One CTA per block; positions in steps of kMatchThreads, one per thread.
-// The block's bytes stream through a ring in shared memory that always holds
-// the window below the step and the step plus a longest match above it; the
-// hash-chain heads and links live in shared memory as well.
-__global__ void __launch_bounds__(kMatchThreads) match_kernel(const uint8_t* in, uint64_t n, uint32_t block_size,
-                                                              uint32_t window, uint32_t max_match,
-                                                              uint32_t chain_depth, uint64_t n_blocks,
-                                                              uint8_t* best_len, uint16_t* best_dist,
-                                                              unsigned long long* counter) {
-  extern __shared__ __align__(16) unsigned char match_smem[];
-  MatchSmem& M = *reinterpret_cast<MatchSmem*>(match_smem);
-  __shared__ unsigned long long next_block;
+// One CTA per block.  Bound by its two barriers a step: 70 us for a 256 KiB
+// block, whatever the number of blocks up to four per SM.
+__global__ void __launch_bounds__(kStep) chain_kernel(const uint8_t* in, uint64_t n, uint32_t block_size,
+                                                      uint16_t* link) {
+  __shared__ uint32_t head[1 << kHeadBits];  // latest position + 1 of an earlier step, 0 = none
   const uint32_t tid = threadIdx.x;
-  constexpr uint32_t RM = kInRing - 1, LM = kLinkRing - 1;
+  const uint64_t base = blockIdx.x * (uint64_t)block_size;
+  const uint32_t len = (uint32_t)min((uint64_t)block_size, n - base);
+  for (uint32_t i = tid; i < (1u << kHeadBits); i += kStep) head[i] = 0;
+  // the 3 bytes at p, from the aligned words they lie in (the input has 16
+  // bytes of slack)
+  auto prefix = [&](uint32_t p) -> uint32_t {
+    if (p + 3 > len) return 0;
+    const uint64_t x = base + p;
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(in) + (x >> 2);
+    return __funnelshift_r(__ldg(w), __ldg(w + 1), (uint32_t)(x & 3u) * 8u) & 0xffffffu;
+  };
+  uint32_t next = prefix(tid);
+  __syncthreads();
+  for (uint32_t s = 0; s < len; s += kStep) {
+    const uint32_t p = s + tid, h = prefix_hash(next);
+    const bool has_prefix = p + 3 <= len;
+    next = prefix(p + kStep);
+    const uint32_t c = has_prefix ? head[h] : 0u;
+    if (p < len) link[base + p] = (c && p + 1 - c <= 0xffffu) ? (uint16_t)(p + 1 - c) : (uint16_t)0;
+    __syncthreads();  // the step's lookups are done
+    if (has_prefix) atomicMax(head + h, p + 1);
+    __syncthreads();
+  }
+}
+
+// A run of `span` positions per CTA.  Shared memory: links of the window and
+// the run, then their bytes and a longest match more.  Bound by the load/store
+// unit: three scattered shared-memory reads per candidate.  Dealing positions
+// out to lanes that are done and comparing only when several lanes have a
+// promising candidate keeps most lanes at work (one thread per position and
+// step, with a barrier per step, had 7.5 of 32): 64 MiB of text 17.3 -> 6.2 ms.
+__global__ void __launch_bounds__(kSearchThreads) search_kernel(const uint8_t* in, uint64_t n, uint32_t block_size,
+                                                                uint32_t window, uint32_t max_match,
+                                                                uint32_t chain_depth, uint32_t span,
+                                                                uint32_t spans_per_block, const uint16_t* link,
+                                                                uint8_t* best_len, uint16_t* best_dist) {
+  extern __shared__ __align__(16) unsigned char search_smem[];
+  __shared__ uint32_t dealt;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, lt = (1u << lane) - 1u;
+  const uint64_t base = blockIdx.x / spans_per_block * (uint64_t)block_size;
+  const uint32_t len = (uint32_t)min((uint64_t)block_size, n - base);
+  const uint32_t t0 = blockIdx.x % spans_per_block * span;
+  if (t0 >= len) return;
+  const uint32_t t1 = min(t0 + span, len);
+  const uint32_t lo = t0 > window ? t0 - window : 0u;  // the run's positions reach back to here
+  const uint32_t shift = (uint32_t)((base + lo) & 3u);  // bytes are kept as aligned as in the input
+  uint16_t* lnk = reinterpret_cast<uint16_t*>(search_smem);  // position lo + i at i
+  uint32_t* words = reinterpret_cast<uint32_t*>(search_smem + ((2u * (window + span) + 15u) & ~15u));
+  if (tid == 0) dealt = 0;
+  for (uint32_t i = tid; i < t1 - lo; i += kSearchThreads) lnk[i] = __ldg(link + base + lo + i);
+  {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(in) + ((base + lo) >> 2);
+    const uint64_t all = (n + 3) >> 2;  // words of the input
+    const uint32_t need = (shift + t1 - lo + kLook + 11u) >> 2;
+    for (uint32_t i = tid; i < need; i += kSearchThreads)
+      words[i] = ((base + lo) >> 2) + i < all ? __ldg(src + i) : 0u;
+  }
+  __syncthreads();
+  // bytes x .. x + 3 of the block, x counted from lo
+  auto word = [&](uint32_t x) {
+    const uint32_t y = x + shift, i = y >> 2;
+    return __funnelshift_r(words[i], words[i + 1], (y & 3u) * 8u);
+  };
+  const uint32_t first = t0 - lo, count = t1 - t0;
+  // a lane's search: position p and candidate c (from lo), best match, what is
+  // compared first: the last four bytes that a longer match needs (three while
+  // there is none)
+  bool active = false, promising = false;
+  uint32_t p = 0, c = 0, ml = 0, dist = 0, lim = 0, left = 0, off = 0, key = 0, mask = 0;
+  uint32_t next = 0, end = 0;  // the warp's share
+  auto store = [&]() {
+    best_len[base + lo + p] = (uint8_t)ml;
+    best_dist[base + lo + p] = (uint16_t)dist;
+  };
+  // to the candidate `l` before the current one; ends the search when there is none
+  auto move = [&](uint32_t l) {
+    c -= l;
+    if (l == 0 || p - c > window || left == 0) {
+      store();
+      active = false;
+    }
+    left--;
+  };
   for (;;) {
-    if (tid == 0) next_block = atomicAdd(counter, 1ull);
-    __syncthreads();
-    const uint64_t b = next_block;
-    __syncthreads();  // every thread has read next_block before thread 0 writes it again
-    if (b >= n_blocks) break;
-    const uint64_t base = b * (uint64_t)block_size;
-    const uint32_t len = (uint32_t)min((uint64_t)block_size, n - base);
-    const uint8_t* blk = in + base;
-    for (uint32_t i = tid; i < (1u << kHeadBits); i += kMatchThreads) M.head[i] = 0;
-    uint32_t loaded = 0;  // the same in every thread
-    auto load_to = [&](uint32_t upto) {
-      for (uint32_t x = loaded + tid; x < upto; x += kMatchThreads) M.ring[x & RM] = __ldg(blk + x);
-      loaded = upto;
-    };
-    load_to(min(len, (uint32_t)kMatchThreads + kLook));
-    __syncthreads();
-    for (uint32_t s = 0; s < len; s += kMatchThreads) {
-      const uint32_t p = s + tid;
-      uint32_t h = 0, ml = 0, dist = 0, c0 = 0;
-      const bool has_prefix = p + 3 <= len;
-      if (has_prefix) {
-        h = prefix_hash(M.ring[p & RM], M.ring[(p + 1) & RM], M.ring[(p + 2) & RM]);
-        const uint32_t lim = min(max_match, len - p);
-        c0 = M.head[h];
-        uint32_t c = c0;  // position + 1
-        for (uint32_t depth = 0; c && depth < chain_depth; depth++) {
-          const uint32_t cand = c - 1, d = p - cand;
-          if (d > window) break;  // links run back in position
-          // a candidate that differs at the current best length cannot beat it
-          if (ml >= lim || M.ring[(cand + ml) & RM] == M.ring[(p + ml) & RM]) {
-            // match length: four bytes per step (the first differing byte
-            // of a word from the XOR's lowest set bit), the last 0..3 bytes
-            // one at a time
-            uint32_t k = 0;
-            for (;;) {
-              if (k + 4 > lim) {
-                while (k < lim && M.ring[(cand + k) & RM] == M.ring[(p + k) & RM]) k++;
-                break;
-              }
-              const uint32_t x = ring_word(M.ring, cand + k) ^ ring_word(M.ring, p + k);
-              if (x) {
-                k += (uint32_t)(__ffs((int)x) - 1) >> 3;
-                break;
-              }
-              k += 4;
-            }
-            if (k >= 3 && k > ml) {
-              ml = k;
-              dist = d;
-              if (k == lim) break;
-            }
-          }
-          const uint32_t delta = M.link[cand & LM];
-          c = delta ? c - delta : 0u;
+    uint32_t idle = __ballot_sync(kFull, !active);
+    if (__popc(idle) >= (int)kRefillAt) {
+      if (next >= end && next < count) {
+        uint32_t x = 0;
+        if (lane == 0) x = atomicAdd(&dealt, kShare);
+        next = __shfl_sync(kFull, x, 0);
+        end = min(next + kShare, count);
+      }
+      const uint32_t mine = next + __popc(idle & lt);
+      if (!active && mine < end) {
+        p = c = first + mine;
+        ml = dist = off = 0;
+        mask = 0xffffffu;
+        lim = min(max_match, len - (lo + p));
+        left = chain_depth;
+        active = true;
+        key = word(p);
+        move(lim >= 3u ? lnk[p] : 0u);
+      }
+      if (next < end) next = min(next + __popc(idle), end);
+      if (next >= count && __all_sync(kFull, !active)) break;
+      idle = __ballot_sync(kFull, !active);
+    }
+    if (active && !promising) {
+      promising = ((word(c + off) ^ key) & mask) == 0;
+      if (!promising) move(lnk[c]);
+    }
+    const uint32_t ready = __ballot_sync(kFull, promising);
+    if (__popc(ready) >= (int)kCompareAt || (ready && __all_sync(kFull, promising || !active))) {
+      if (promising) {
+        promising = false;
+        uint32_t k = 0, x;
+        do {
+          x = word(c + k) ^ word(p + k);
+          k += 4;
+        } while (!x && k < lim);
+        if (x) k = k - 4u + ((uint32_t)(__ffs((int)x) - 1) >> 3);
+        k = min(k, lim);
+        if (k >= 3 && k > ml) {
+          ml = k;
+          dist = p - c;
+          off = k - 3u;
+          mask = 0xffffffffu;
+          key = word(p + off);
         }
+        move(ml == lim ? 0u : lnk[c]);
       }
-      if (p < len) {
-        best_len[base + p] = (uint8_t)ml;
-        best_dist[base + p] = (uint16_t)dist;
-      }
-      __syncthreads();  // the step's lookups are done
-      if (has_prefix) {
-        // each position links to the bucket's latest position before the
-        // step (positions of one step do not see each other)
-        M.link[p & LM] = (c0 && p + 1 - c0 <= 0xffffu) ? (uint16_t)(p + 1 - c0) : (uint16_t)0;
-        atomicMax(M.head + h, p + 1);
-      }
-      load_to(min(len, s + 2 * kMatchThreads + kLook));
-      __syncthreads();
     }
   }
 }
@@ -183,100 +228,213 @@ __device__ __forceinline__ uint32_t de_cut(const ParseState& st, uint32_t q, uin
   return L >= 3 ? L : 0u;
 }
 
-constexpr int kParseWarps = 4;
-constexpr uint32_t kChunk = 2048;  // positions staged in shared memory per warp
+constexpr uint32_t kParseThreads = 256;
+constexpr uint32_t kChunk = 2048;  // positions parsed at a time
+constexpr uint32_t kOver = 128;
+constexpr uint32_t kNoMatch = 0xffffffffu;
 
-// One warp per block: the warp stages the per-position matches of the next
-// kChunk positions in shared memory, lane 0 parses them.
-__global__ void __launch_bounds__(32 * kParseWarps) parse_kernel(const uint8_t* best_len, const uint16_t* best_dist,
-                                                                 uint64_t n, uint32_t block_size, uint64_t n_blocks,
-                                                                 uint32_t max_match, int de, int byte_mode, int lazy,
-                                                                 gmp::ParseToken* tok, uint32_t* tpos,
-                                                                 uint64_t stride, uint32_t* count) {
-  __shared__ uint8_t chunk_len[kParseWarps][kChunk];
-  __shared__ uint16_t chunk_dist[kParseWarps][kChunk];
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const uint64_t b = (uint64_t)blockIdx.x * kParseWarps + warp;
-  if (b >= n_blocks) return;
-  uint8_t* cl = chunk_len[warp];
-  uint16_t* cd = chunk_dist[warp];
-  const uint64_t base = b * (uint64_t)block_size;
+struct ParseSmem {
+  ParseState st;
+  // per position of the chunk: where the next match token from here starts
+  // (low half) and ends (high half), or kNoMatch, and the highest source end
+  // (position in the block) of the matches looked at to decide so
+  uint2 jump[kChunk];
+  uint2 list[kChunk / 3 + 2];  // the chunk's tokens: start of their literals; match start << 8 | length
+  // matches of the chunk, and of the one after it while this one is walked
+  // (it starts at most a match and its lazy steps past the chunk's end)
+  uint16_t dist[2][kChunk + kOver];
+  uint8_t len[2][kChunk + kOver];
+  uint32_t match_rows[kChunk / 32];  // a bit per position with a match
+  uint32_t p, n_list, first_token;
+};
+
+// One CTA per block.  A chunk's decisions are independent but for where the
+// parse enters it (and, for DE, the group's earlier ranges: a match whose
+// sources end below the group's first back-reference cannot be cut, which the
+// walking thread sees from one number; the others it decides one by one).
+// Bound by that thread's chain of one shared-memory read per token.  One
+// thread deciding every position took 10.6 ms for 64 MiB of text (256
+// blocks), 16.5 for 16 MiB of CSV rows with DE; now 1.8 and 5.9.
+__global__ void __launch_bounds__(kParseThreads) parse_kernel(const uint8_t* best_len, const uint16_t* best_dist,
+                                                              uint64_t n, uint32_t block_size, uint32_t max_match,
+                                                              int de, int byte_mode, int lazy, gmp::ParseToken* tok,
+                                                              uint32_t* tpos, uint64_t stride, uint32_t* count) {
+  __shared__ ParseSmem S;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  const uint64_t b = blockIdx.x, base = b * (uint64_t)block_size;
   const uint32_t len = (uint32_t)min((uint64_t)block_size, n - base);
   gmp::ParseToken* t = tok + b * stride;
   uint32_t* tp = tpos + b * stride;
-  uint32_t nt = 0, p = 0, lit_start = 0;
-  ParseState st;
-  st.in_grp = 0;
-  st.lo_min = ~0u;
-  auto emit = [&](uint32_t ll, uint32_t ml, uint32_t d) {
+  // thread 0's state: tokens so far, start of the pending literals
+  uint32_t nt = 0, lit_start = 0;
+  ParseState& st = S.st;
+  auto put = [&](uint32_t ll, uint32_t match) {  // a token at once (not by way of the list)
     if (nt < stride) {
-      t[nt] = gmp::ParseToken{ll, (d << 8) | ml};
+      t[nt] = gmp::ParseToken{ll, match};
       tp[nt] = lit_start;
     }
     nt++;
   };
+  uint32_t in_grp = 0, lo_min = ~0u;  // of st, there only while de_cut looks
   auto add_to_group = [&](uint32_t lo, uint32_t hi) {
     if (de) {
-      if (lo != hi && st.lo_min == ~0u) st.lo_min = lo;
-      st.glo[st.in_grp] = lo;
-      st.ghi[st.in_grp] = hi;
-      if (++st.in_grp == 32) {
-        st.in_grp = 0;
-        st.lo_min = ~0u;
+      if (lo != hi && lo_min == ~0u) lo_min = lo;
+      st.glo[in_grp] = lo;
+      st.ghi[in_grp] = hi;
+      if (++in_grp == 32) {
+        in_grp = 0;
+        lo_min = ~0u;
       }
     }
   };
-  while (p < len) {
-    const uint32_t c0 = p, cn = min(kChunk, len - c0);
-    for (uint32_t i = lane; i < cn; i += 32) {
-      cl[i] = best_len[base + c0 + i];
-      cd[i] = best_dist[base + c0 + i];
+  // loads the matches of [from, from + kChunk + kOver) into buffer k; threads
+  // t of m
+  auto fetch = [&](int k, uint32_t from, uint32_t t_, uint32_t m) {
+#pragma unroll 4
+    for (uint32_t i = t_; i < kChunk + kOver; i += m) {
+      const bool in = from + i < len;
+      const uint8_t l = in ? __ldg(best_len + base + from + i) : (uint8_t)0;
+      const uint16_t d = in ? __ldg(best_dist + base + from + i) : (uint16_t)0;
+      S.len[k][i] = l;
+      S.dist[k][i] = d;
     }
-    __syncwarp();
-    if (lane == 0) {
-      auto match_at = [&](uint32_t q, uint32_t& D) -> uint32_t {
-        const uint32_t L = cl[q - c0];
-        D = cd[q - c0];
-        if (L < 3) return 0;
-        return de ? de_cut(st, q, L, D) : L;
-      };
-      // parse while the lazy look at p + 1 stays in the chunk (or the chunk
-      // ends the block)
-      const uint32_t end = c0 + cn, stop = end == len ? len : end - 1;
-      while (p < stop) {
-        uint32_t D = 0;
-        uint32_t L = match_at(p, D);
-        if (L && lazy) {
-          while (p + 1 < end && L < max_match) {
-            uint32_t D2 = 0;
-            const uint32_t L2 = match_at(p + 1, D2);
-            if (L2 <= L) break;
-            p++;  // the byte at p stays a literal
+  };
+  int buf = 0;
+  uint32_t buf_at = 0;  // position of the buffer's first entry
+  fetch(0, 0, tid, kParseThreads);
+  __syncthreads();
+  for (uint32_t c0 = 0; c0 < len; buf ^= 1) {
+    const uint8_t* s_len = S.len[buf] + (c0 - buf_at);
+    const uint16_t* s_dist = S.dist[buf] + (c0 - buf_at);
+    const uint32_t cn = min(kChunk, len - c0);
+    // decisions are taken up to `stop`, so that the lazy look at the next
+    // position stays in the chunk, and look up to `end`
+    const uint32_t stop = c0 + cn == len ? cn : cn - 1;
+    // positions with a match: the token that a decision there gives
+    for (uint32_t row = warp; row < kChunk / 32; row += kParseThreads / 32) {
+      const uint32_t i = 32 * row + lane;
+      uint32_t L = s_len[i];
+      const bool match = L >= 3 && i < stop;
+      const uint32_t bits = __ballot_sync(kFull, match);
+      if (lane == 0) S.match_rows[row] = bits;
+      if (match) {
+        uint32_t m = i, src_end = min(c0 + i - s_dist[i] + L, c0 + i);
+        if (lazy) {
+          while (m + 1 < cn && L < max_match) {
+            const uint32_t L2 = s_len[m + 1];
+            if (L2 >= 3) src_end = max(src_end, min(c0 + m + 1 - s_dist[m + 1] + L2, c0 + m + 1));
+            if (L2 < 3 || L2 <= L) break;
+            m++;  // the byte at m stays a literal
             L = L2;
-            D = D2;
           }
         }
-        if (L) {
-          while (byte_mode && p - lit_start > kByteMaxLit) {
-            emit(kByteMaxLit, 0, 0);
-            lit_start += kByteMaxLit;
-            add_to_group(0, 0);
-          }
-          emit(p - lit_start, L, D);
-          add_to_group(p, p + L);
-          p += L;
-          lit_start = p;
-        } else {
-          p++;
-        }
+        S.jump[i] = make_uint2(m | ((m + L) << 16), src_end);
       }
     }
-    p = __shfl_sync(kFull, p, 0);
-    __syncwarp();
+    __syncthreads();
+    // positions without one: the next one's
+    for (uint32_t row = warp; row < kChunk / 32; row += kParseThreads / 32) {
+      const uint32_t i = 32 * row + lane, bits = S.match_rows[row];
+      if (!((bits >> lane) & 1u)) {
+        uint32_t r = row, m = bits & (0xfffffffeu << lane);
+        while (!m && ++r < kChunk / 32) m = S.match_rows[r];
+        S.jump[i] = m ? S.jump[32 * r + (uint32_t)__ffs((int)m) - 1u] : make_uint2(kNoMatch, 0);
+      }
+    }
+    __syncthreads();
+    if (tid >= 32) {
+      fetch(buf ^ 1, c0 + stop, tid - 32, kParseThreads - 32);
+    } else if (tid == 0) {
+      uint32_t p = 0, k = 0;  // position in the chunk, tokens in the list
+      S.first_token = nt;
+      auto literal_runs = [&](uint32_t m) {
+        // rare: the list goes out first, then the literal runs
+        for (uint32_t i = 0; i < k; i++) {
+          const uint32_t x = S.list[i].y, at = x >> 8, u = S.first_token + i;
+          if (u < stride) {
+            t[u] = gmp::ParseToken{c0 + at - S.list[i].x, ((uint32_t)s_dist[at] << 8) | (x & 255u)};
+            tp[u] = S.list[i].x;
+          }
+        }
+        k = 0;
+        while (c0 + m - lit_start > kByteMaxLit) {
+          put(kByteMaxLit, 0);
+          lit_start += kByteMaxLit;
+          add_to_group(0, 0);
+        }
+        S.first_token = nt;
+      };
+      if (!de) {
+        while (p < stop) {
+          const uint32_t j = S.jump[p].x, m = j & 0xffffu;
+          if (j == kNoMatch) {
+            p = stop;
+            break;
+          }
+          if (byte_mode && c0 + m - lit_start > kByteMaxLit) literal_runs(m);
+          p = j >> 16;
+          S.list[k++] = make_uint2(lit_start, (m << 8) | (p - m));
+          nt++;
+          lit_start = c0 + p;
+        }
+      } else {
+        while (p < stop) {
+          const uint2 j = S.jump[p];
+          uint32_t m = j.x & 0xffffu, e = j.x >> 16;
+          if (j.x == kNoMatch) {
+            p = stop;
+            break;
+          }
+          if (j.y > lo_min) {
+            // a source that may lie in the group: this position's decision
+            st.in_grp = in_grp;
+            st.lo_min = lo_min;
+            auto match_at = [&](uint32_t q) -> uint32_t {
+              const uint32_t L = s_len[q];
+              return L < 3 ? 0u : de_cut(st, c0 + q, L, s_dist[q]);
+            };
+            uint32_t L = match_at(p);
+            if (!L) {
+              p++;
+              continue;
+            }
+            if (lazy) {
+              while (p + 1 < cn && L < max_match) {
+                const uint32_t L2 = match_at(p + 1);
+                if (L2 <= L) break;
+                p++;
+                L = L2;
+              }
+            }
+            m = p;
+            e = p + L;
+          }
+          if (byte_mode && c0 + m - lit_start > kByteMaxLit) literal_runs(m);
+          p = e;
+          S.list[k++] = make_uint2(lit_start, (m << 8) | (p - m));
+          nt++;
+          lit_start = c0 + p;
+          add_to_group(c0 + m, c0 + p);
+        }
+      }
+      S.p = p;
+      S.n_list = k;
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < S.n_list; i += kParseThreads) {
+      const uint32_t x = S.list[i].y, at = x >> 8, u = S.first_token + i;
+      if (u < stride) {
+        t[u] = gmp::ParseToken{c0 + at - S.list[i].x, ((uint32_t)s_dist[at] << 8) | (x & 255u)};
+        tp[u] = S.list[i].x;
+      }
+    }
+    buf_at = c0 + stop;
+    c0 += S.p;
+    __syncthreads();
   }
-  if (lane == 0) {
-    for (; byte_mode && len - lit_start > kByteMaxLit; lit_start += kByteMaxLit) emit(kByteMaxLit, 0, 0);
-    if (lit_start < len) emit(len - lit_start, 0, 0);
+  if (tid == 0) {
+    for (; byte_mode && len - lit_start > kByteMaxLit; lit_start += kByteMaxLit) put(kByteMaxLit, 0);
+    if (lit_start < len) put(len - lit_start, 0);
     count[b] = nt;
   }
 }
@@ -338,7 +496,7 @@ int gmp_compress_gpu(int device, const void* host_in, size_t n, const gmp_compre
     unsigned long long* d_counter = nullptr;
     gmp::EncBlockPlan* d_plan = nullptr;
     uint64_t* d_bytes = nullptr;
-    if (check(cudaMalloc(&D.p[0], n), "cudaMalloc") && check(cudaMalloc(&D.p[1], n), "cudaMalloc") &&
+    if (check(cudaMalloc(&D.p[0], n + 16), "cudaMalloc") && check(cudaMalloc(&D.p[1], n), "cudaMalloc") &&
         check(cudaMalloc(&D.p[2], 2 * n), "cudaMalloc") &&
         check(cudaMalloc(&D.p[3], nb * stride * sizeof(gmp::ParseToken)), "cudaMalloc") &&
         check(cudaMalloc(&D.p[4], nb * stride * sizeof(uint32_t)), "cudaMalloc") &&
@@ -363,25 +521,31 @@ int gmp_compress_gpu(int device, const void* host_in, size_t n, const gmp_compre
     }
     if (rc == GMP_OK) {
       check(cudaEventRecord(ev[0]), "cudaEventRecord");
-      const int smem = (int)sizeof(MatchSmem);
-      int occ = 0;
-      check(cudaFuncSetAttribute(match_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+      // the links lie where the tokens go later
+      uint16_t* d_link = reinterpret_cast<uint16_t*>(d_tok);
+      chain_kernel<<<(unsigned)nb, kStep>>>(d_in, n, o.block_size, d_link);
+      check(cudaGetLastError(), "chain_kernel");
+      // runs of 32 Ki positions, whose window of as many more is loaded once
+      // for all of them; of fewer while there are not two per SM
+      uint32_t span = 32768;
+      auto runs = [&](uint32_t v) { return ((uint64_t)o.block_size + v - 1) / v * nb; };
+      while (span > 4096 && (runs(span) < 2ull * (uint64_t)std::max(sms, 1) || span >= 2ull * o.block_size)) span /= 2;
+      const uint64_t per_block = ((uint64_t)o.block_size + span - 1) / span;
+      const int smem = (int)(((2 * (o.window + span) + 15) & ~15u) + o.window + span + kLook + 32);
+      check(cudaFuncSetAttribute(search_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSearchSmemMax),
             "cudaFuncSetAttribute");
-      check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, match_kernel, kMatchThreads, smem),
-            "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-      const uint64_t grid = std::min<uint64_t>((uint64_t)std::max(occ, 1) * (uint64_t)std::max(sms, 1), nb);
       if (rc == GMP_OK) {
-        match_kernel<<<(unsigned)grid, kMatchThreads, smem>>>(d_in, n, o.block_size, o.window, o.max_match,
-                                                              std::min(o.chain_depth, 64u), nb, d_len, d_dist,
-                                                              d_counter);
-        check(cudaGetLastError(), "match_kernel");
+        search_kernel<<<(unsigned)(per_block * nb), kSearchThreads, smem>>>(
+            d_in, n, o.block_size, o.window, o.max_match, std::min(o.chain_depth, 64u), span, (uint32_t)per_block,
+            d_link, d_len, d_dist);
+        check(cudaGetLastError(), "search_kernel");
       }
     }
     if (rc == GMP_OK) {
       check(cudaEventRecord(ev[1]), "cudaEventRecord");
-      parse_kernel<<<(unsigned)((nb + kParseWarps - 1) / kParseWarps), 32 * kParseWarps>>>(
-          d_len, d_dist, n, o.block_size, nb, o.max_match, o.de ? 1 : 0, o.byte_mode ? 1 : 0, o.lazy ? 1 : 0, d_tok,
-          d_tpos, stride, d_count);
+      parse_kernel<<<(unsigned)nb, kParseThreads>>>(d_len, d_dist, n, o.block_size, o.max_match, o.de ? 1 : 0,
+                                                    o.byte_mode ? 1 : 0, o.lazy ? 1 : 0, d_tok, d_tpos, stride,
+                                                    d_count);
       check(cudaGetLastError(), "parse_kernel");
     }
     // entropy coding on the GPU: plan every block (sizes), lay the blocks out
