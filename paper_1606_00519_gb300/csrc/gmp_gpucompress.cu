@@ -24,7 +24,7 @@
 //  least 3 bytes is taken unless the next position has a longer one
 //  (one-step lazy evaluation), otherwise the byte becomes a literal.  What
 //  follows from the matches alone is worked out for every position at once,
-//  so that one thread has one lookup to do per token.  For DE streams a
+//  so that one warp has one lookup to do per token.  For DE streams a
 //  candidate is cut at the first source byte that an earlier back-reference
 //  of the same 32-sequence group writes, as in gmp_compress; for Byte streams
 //  literal strings are cut into runs of at most 1023 bytes, which count as
@@ -55,6 +55,7 @@ constexpr int kSearchThreads = 1024;
 constexpr int kSearchSmemMax = 3 * (32768 + 32768) + 64 + 64;  // window and run of 32 Ki positions
 constexpr uint32_t kShare = 128;         // positions that a warp takes at a time
 constexpr uint32_t kCompareAt = 10;      // lanes with a promising candidate that make the warp compare
+constexpr int kWalkSteps = 4;           // candidates between the warp's votes
 constexpr uint32_t kRefillAt = 6;        // idle lanes that make the warp deal out positions
 
 __device__ __forceinline__ uint32_t prefix_hash(uint32_t b012) {
@@ -97,7 +98,7 @@ __global__ void __launch_bounds__(kStep) chain_kernel(const uint8_t* in, uint64_
 // unit: three scattered shared-memory reads per candidate.  Dealing positions
 // out to lanes that are done and comparing only when several lanes have a
 // promising candidate keeps most lanes at work (one thread per position and
-// step, with a barrier per step, had 7.5 of 32): 64 MiB of text 17.3 -> 6.2 ms.
+// step, with a barrier per step, had 7.5 of 32): 64 MiB of text 17.3 -> 3.6 ms.
 __global__ void __launch_bounds__(kSearchThreads) search_kernel(const uint8_t* in, uint64_t n, uint32_t block_size,
                                                                 uint32_t window, uint32_t max_match,
                                                                 uint32_t chain_depth, uint32_t span,
@@ -116,7 +117,11 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(const uint8_t* i
   uint16_t* lnk = reinterpret_cast<uint16_t*>(search_smem);  // position lo + i at i
   uint32_t* words = reinterpret_cast<uint32_t*>(search_smem + ((2u * (window + span) + 15u) & ~15u));
   if (tid == 0) dealt = 0;
-  for (uint32_t i = tid; i < t1 - lo; i += kSearchThreads) lnk[i] = __ldg(link + base + lo + i);
+  // no link: one beyond every window
+  for (uint32_t i = tid; i < t1 - lo; i += kSearchThreads) {
+    const uint16_t l = __ldg(link + base + lo + i);
+    lnk[i] = l ? l : (uint16_t)0xffffu;
+  }
   {
     const uint32_t* src = reinterpret_cast<const uint32_t*>(in) + ((base + lo) >> 2);
     const uint64_t all = (n + 3) >> 2;  // words of the input
@@ -128,31 +133,30 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(const uint8_t* i
   // bytes x .. x + 3 of the block, x counted from lo
   auto word = [&](uint32_t x) {
     const uint32_t y = x + shift, i = y >> 2;
-    return __funnelshift_r(words[i], words[i + 1], (y & 3u) * 8u);
+    return __funnelshift_r(words[i], words[i + 1], y << 3);
   };
   const uint32_t first = t0 - lo, count = t1 - t0;
-  // a lane's search: position p and candidate c (from lo), best match, what is
-  // compared first: the last four bytes that a longer match needs (three while
-  // there is none)
-  bool active = false, promising = false;
-  uint32_t p = 0, c = 0, ml = 0, dist = 0, lim = 0, left = 0, off = 0, key = 0, mask = 0;
+  // a lane's search: position p and candidate c (from lo), the lowest one
+  // allowed, best match, and what is compared first: the last four bytes that
+  // a longer match needs (three while there is none).  A lane walks its chain,
+  // or waits with a promising candidate, or is done.
+  bool walk = false, promising = false, has = false;
+  int c = 0, c_min = 0;
+  uint32_t p = 0, ml = 0, dist = 0, lim = 0, left = 0, off = 0, key = 0, mask = 0;
   uint32_t next = 0, end = 0;  // the warp's share
-  auto store = [&]() {
-    best_len[base + lo + p] = (uint8_t)ml;
-    best_dist[base + lo + p] = (uint16_t)dist;
-  };
-  // to the candidate `l` before the current one; ends the search when there is none
-  auto move = [&](uint32_t l) {
-    c -= l;
-    if (l == 0 || p - c > window || left == 0) {
-      store();
-      active = false;
-    }
+  auto move = [&]() {  // to the candidate before
+    c -= lnk[c];
     left--;
+    walk = c >= c_min && left != 0;
   };
   for (;;) {
-    uint32_t idle = __ballot_sync(kFull, !active);
+    const uint32_t idle = __ballot_sync(kFull, !(walk || promising));
     if (__popc(idle) >= (int)kRefillAt) {
+      if (!(walk || promising) && has) {
+        best_len[base + lo + p] = (uint8_t)ml;
+        best_dist[base + lo + p] = (uint16_t)dist;
+        has = false;
+      }
       if (next >= end && next < count) {
         uint32_t x = 0;
         if (lane == 0) x = atomicAdd(&dealt, kShare);
@@ -160,26 +164,34 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(const uint8_t* i
         end = min(next + kShare, count);
       }
       const uint32_t mine = next + __popc(idle & lt);
-      if (!active && mine < end) {
-        p = c = first + mine;
+      if (!(walk || promising) && mine < end) {
+        p = first + mine;
+        c = (int)p;
+        c_min = max((int)p - (int)window, 0);
         ml = dist = off = 0;
         mask = 0xffffffu;
         lim = min(max_match, len - (lo + p));
-        left = chain_depth;
-        active = true;
+        left = chain_depth + 1;
+        has = true;
         key = word(p);
-        move(lim >= 3u ? lnk[p] : 0u);
+        if (lim >= 3u) move();
       }
       if (next < end) next = min(next + __popc(idle), end);
-      if (next >= count && __all_sync(kFull, !active)) break;
-      idle = __ballot_sync(kFull, !active);
+      if (next >= count && !__any_sync(kFull, walk || promising || has)) break;
     }
-    if (active && !promising) {
-      promising = ((word(c + off) ^ key) & mask) == 0;
-      if (!promising) move(lnk[c]);
+#pragma unroll
+    for (int u = 0; u < kWalkSteps; u++) {
+      if (walk) {
+        if (((word(c + off) ^ key) & mask) == 0) {
+          promising = true;
+          walk = false;
+        } else {
+          move();
+        }
+      }
     }
     const uint32_t ready = __ballot_sync(kFull, promising);
-    if (__popc(ready) >= (int)kCompareAt || (ready && __all_sync(kFull, promising || !active))) {
+    if (__popc(ready) >= (int)kCompareAt || (ready && !__any_sync(kFull, walk))) {
       if (promising) {
         promising = false;
         uint32_t k = 0, x;
@@ -191,42 +203,54 @@ __global__ void __launch_bounds__(kSearchThreads) search_kernel(const uint8_t* i
         k = min(k, lim);
         if (k >= 3 && k > ml) {
           ml = k;
-          dist = p - c;
+          dist = p - (uint32_t)c;
           off = k - 3u;
           mask = 0xffffffffu;
           key = word(p + off);
         }
-        move(ml == lim ? 0u : lnk[c]);
+        if (ml != lim) move();
       }
     }
   }
 }
 
-struct ParseState {
-  uint32_t glo[32], ghi[32];  // DE: output ranges of the current group's back-references
-  uint32_t in_grp;
-  uint32_t lo_min;            // start of the group's first back-reference (~0u: none yet)
-};
-
-// DE rule (Sec. 4.2, as read in gmp_compress): the source bytes before the
-// current position must avoid the group's earlier back-references; the
-// candidate is cut at the first such byte (0 if fewer than 3 bytes remain).
-// The group's ranges rise with their index (empty ranges stand for
-// literal-only sequences): a source that ends below the first of them is
-// free (the common case: most sources lie before the group); otherwise the
-// scan runs backwards and stops at the first range that ends at or below
-// the source.
-__device__ __forceinline__ uint32_t de_cut(const ParseState& st, uint32_t q, uint32_t L, uint32_t D) {
-  if (L == 0) return 0;
-  const uint32_t src = q - D, src_end = min(src + L, q);
-  if (src_end <= st.lo_min) return L >= 3 ? L : 0u;
-  for (int g = (int)st.in_grp - 1; g >= 0; g--) {
-    if (st.glo[g] == st.ghi[g]) continue;
-    if (st.ghi[g] <= src) break;
-    if (st.glo[g] < src_end) L = min(L, st.glo[g] > src ? st.glo[g] - src : 0u);
+// DE rule (Sec. 4.2, as read in gmp_compress): a match's source bytes before
+// its own position must avoid the bytes that earlier back-references of its
+// 32-sequence group write; it is cut at the first such byte (to nothing if
+// fewer than 3 bytes remain).  Lane g holds the g-th range of the group
+// (empty: a literal run), so that a cut is one reduction over the warp; the
+// other values are the same in every lane.
+struct Group {
+  uint32_t lo = 0, hi = 0;  // this lane's range
+  uint32_t n = 0;           // ranges so far
+  uint32_t lo_min = ~0u;    // start of the first back-reference
+  __device__ void add(uint32_t from, uint32_t to) {
+    const bool here = (threadIdx.x & 31u) == n;
+    lo = here ? from : lo;
+    hi = here ? to : hi;
+    lo_min = from != to ? min(lo_min, from) : lo_min;  // ranges rise
+    if (++n == 32) {
+      n = lo = hi = 0;
+      lo_min = ~0u;
+    }
   }
-  return L >= 3 ? L : 0u;
-}
+  __device__ void grow(uint32_t a, uint32_t first) {  // a ranges, set by their lanes, from `first` on
+    lo_min = min(lo_min, first);
+    n += a;
+    if (n == 32) {
+      n = lo = hi = 0;
+      lo_min = ~0u;
+    }
+  }
+  // what a match of L >= 3 bytes at q, distance D, is cut to
+  __device__ uint32_t cut(uint32_t q, uint32_t L, uint32_t D) const {
+    const uint32_t src = q - D, end = min(src + L, q);
+    if (end <= lo_min) return L;
+    // (an empty range is 0, 0)
+    L = __reduce_min_sync(kFull, lo < end && hi > src ? max(lo, src) - src : L);
+    return L >= 3 ? L : 0u;
+  }
+};
 
 constexpr uint32_t kParseThreads = 256;
 constexpr uint32_t kChunk = 2048;  // positions parsed at a time
@@ -234,16 +258,16 @@ constexpr uint32_t kOver = 128;
 constexpr uint32_t kNoMatch = 0xffffffffu;
 
 struct ParseSmem {
-  ParseState st;
   // per position of the chunk: where the next match token from here starts
   // (low half) and ends (high half), or kNoMatch, and the highest source end
   // (position in the block) of the matches looked at to decide so
   uint2 jump[kChunk];
+  uint16_t next[kChunk + kOver];  // that end; where no token follows the chunk's stop; itself from there on
   uint2 list[kChunk / 3 + 2];  // the chunk's tokens: start of their literals; match start << 8 | length
   // matches of the chunk, and of the one after it while this one is walked
   // (it starts at most a match and its lazy steps past the chunk's end)
-  uint16_t dist[2][kChunk + kOver];
-  uint8_t len[2][kChunk + kOver];
+  // (length | distance << 8)
+  uint32_t match[2][kChunk + kOver];
   uint32_t match_rows[kChunk / 32];  // a bit per position with a match
   uint32_t p, n_list, first_token;
 };
@@ -251,10 +275,10 @@ struct ParseSmem {
 // One CTA per block.  A chunk's decisions are independent but for where the
 // parse enters it (and, for DE, the group's earlier ranges: a match whose
 // sources end below the group's first back-reference cannot be cut, which the
-// walking thread sees from one number; the others it decides one by one).
-// Bound by that thread's chain of one shared-memory read per token.  One
+// walking warp sees from one number; the others it decides one by one).
+// Bound by that warp's chain of one shared-memory read per token.  One
 // thread deciding every position took 10.6 ms for 64 MiB of text (256
-// blocks), 16.5 for 16 MiB of CSV rows with DE; now 1.8 and 5.9.
+// blocks), 16.5 for 16 MiB of CSV rows with DE; now 1.4 and 1.7.
 __global__ void __launch_bounds__(kParseThreads) parse_kernel(const uint8_t* best_len, const uint16_t* best_dist,
                                                               uint64_t n, uint32_t block_size, uint32_t max_match,
                                                               int de, int byte_mode, int lazy, gmp::ParseToken* tok,
@@ -265,27 +289,15 @@ __global__ void __launch_bounds__(kParseThreads) parse_kernel(const uint8_t* bes
   const uint32_t len = (uint32_t)min((uint64_t)block_size, n - base);
   gmp::ParseToken* t = tok + b * stride;
   uint32_t* tp = tpos + b * stride;
-  // thread 0's state: tokens so far, start of the pending literals
+  // warp 0's state: tokens so far, start of the pending literals, DE group
   uint32_t nt = 0, lit_start = 0;
-  ParseState& st = S.st;
+  Group grp;
   auto put = [&](uint32_t ll, uint32_t match) {  // a token at once (not by way of the list)
-    if (nt < stride) {
+    if (nt < stride && lane == 0) {
       t[nt] = gmp::ParseToken{ll, match};
       tp[nt] = lit_start;
     }
     nt++;
-  };
-  uint32_t in_grp = 0, lo_min = ~0u;  // of st, there only while de_cut looks
-  auto add_to_group = [&](uint32_t lo, uint32_t hi) {
-    if (de) {
-      if (lo != hi && lo_min == ~0u) lo_min = lo;
-      st.glo[in_grp] = lo;
-      st.ghi[in_grp] = hi;
-      if (++in_grp == 32) {
-        in_grp = 0;
-        lo_min = ~0u;
-      }
-    }
   };
   // loads the matches of [from, from + kChunk + kOver) into buffer k; threads
   // t of m
@@ -295,8 +307,7 @@ __global__ void __launch_bounds__(kParseThreads) parse_kernel(const uint8_t* bes
       const bool in = from + i < len;
       const uint8_t l = in ? __ldg(best_len + base + from + i) : (uint8_t)0;
       const uint16_t d = in ? __ldg(best_dist + base + from + i) : (uint16_t)0;
-      S.len[k][i] = l;
-      S.dist[k][i] = d;
+      S.match[k][i] = l | ((uint32_t)d << 8);
     }
   };
   int buf = 0;
@@ -304,8 +315,7 @@ __global__ void __launch_bounds__(kParseThreads) parse_kernel(const uint8_t* bes
   fetch(0, 0, tid, kParseThreads);
   __syncthreads();
   for (uint32_t c0 = 0; c0 < len; buf ^= 1) {
-    const uint8_t* s_len = S.len[buf] + (c0 - buf_at);
-    const uint16_t* s_dist = S.dist[buf] + (c0 - buf_at);
+    const uint32_t* match = S.match[buf] + (c0 - buf_at);
     const uint32_t cn = min(kChunk, len - c0);
     // decisions are taken up to `stop`, so that the lazy look at the next
     // position stays in the chunk, and look up to `end`
@@ -313,16 +323,17 @@ __global__ void __launch_bounds__(kParseThreads) parse_kernel(const uint8_t* bes
     // positions with a match: the token that a decision there gives
     for (uint32_t row = warp; row < kChunk / 32; row += kParseThreads / 32) {
       const uint32_t i = 32 * row + lane;
-      uint32_t L = s_len[i];
-      const bool match = L >= 3 && i < stop;
-      const uint32_t bits = __ballot_sync(kFull, match);
+      const uint32_t x = match[i];
+      uint32_t L = x & 255u;
+      const bool any = L >= 3 && i < stop;
+      const uint32_t bits = __ballot_sync(kFull, any);
       if (lane == 0) S.match_rows[row] = bits;
-      if (match) {
-        uint32_t m = i, src_end = min(c0 + i - s_dist[i] + L, c0 + i);
+      if (any) {
+        uint32_t m = i, src_end = min(c0 + i - (x >> 8) + L, c0 + i);
         if (lazy) {
           while (m + 1 < cn && L < max_match) {
-            const uint32_t L2 = s_len[m + 1];
-            if (L2 >= 3) src_end = max(src_end, min(c0 + m + 1 - s_dist[m + 1] + L2, c0 + m + 1));
+            const uint32_t x2 = match[m + 1], L2 = x2 & 255u;
+            if (L2 >= 3) src_end = max(src_end, min(c0 + m + 1 - (x2 >> 8) + L2, c0 + m + 1));
             if (L2 < 3 || L2 <= L) break;
             m++;  // the byte at m stays a literal
             L = L2;
@@ -340,91 +351,124 @@ __global__ void __launch_bounds__(kParseThreads) parse_kernel(const uint8_t* bes
         while (!m && ++r < kChunk / 32) m = S.match_rows[r];
         S.jump[i] = m ? S.jump[32 * r + (uint32_t)__ffs((int)m) - 1u] : make_uint2(kNoMatch, 0);
       }
+      const uint32_t j = S.jump[i].x;
+      S.next[i] = (uint16_t)(i >= stop ? i : j == kNoMatch ? stop : j >> 16);
     }
+    if (tid < kOver) S.next[kChunk + tid] = (uint16_t)(kChunk + tid);
     __syncthreads();
     if (tid >= 32) {
       fetch(buf ^ 1, c0 + stop, tid - 32, kParseThreads - 32);
-    } else if (tid == 0) {
-      uint32_t p = 0, k = 0;  // position in the chunk, tokens in the list
-      S.first_token = nt;
-      auto literal_runs = [&](uint32_t m) {
-        // rare: the list goes out first, then the literal runs
-        for (uint32_t i = 0; i < k; i++) {
-          const uint32_t x = S.list[i].y, at = x >> 8, u = S.first_token + i;
-          if (u < stride) {
-            t[u] = gmp::ParseToken{c0 + at - S.list[i].x, ((uint32_t)s_dist[at] << 8) | (x & 255u)};
-            tp[u] = S.list[i].x;
-          }
-        }
-        k = 0;
-        while (c0 + m - lit_start > kByteMaxLit) {
-          put(kByteMaxLit, 0);
-          lit_start += kByteMaxLit;
-          add_to_group(0, 0);
-        }
-        S.first_token = nt;
+    } else {
+      // the warp walks: up to 32 tokens (DE: the rest of the group) by one
+      // read each, every lane keeping where one of them was decided; then each
+      // lane looks its token up, and the warp takes those before the first
+      // that needs a closer look
+      uint32_t p = 0, k = 0, first_token = nt;  // position in the chunk, tokens in the list
+      auto list = [&](uint32_t at, uint32_t lits, uint32_t m, uint32_t e) {
+        S.list[at] = make_uint2(lits, (m << 8) | (e - m));
       };
-      if (!de) {
-        while (p < stop) {
-          const uint32_t j = S.jump[p].x, m = j & 0xffffu;
-          if (j == kNoMatch) {
-            p = stop;
-            break;
+      while (p < stop) {
+        const uint32_t n = de ? grp.n : 0u;
+        uint32_t mine = kChunk, q = p;
+        for (uint32_t x = n; x < 32u && q < stop; x += 8) {
+#pragma unroll
+          for (uint32_t y = 0; y < 8; y++) {
+            mine = lane == x + y ? q : mine;
+            q = S.next[q];
           }
-          if (byte_mode && c0 + m - lit_start > kByteMaxLit) literal_runs(m);
-          p = j >> 16;
-          S.list[k++] = make_uint2(lit_start, (m << 8) | (p - m));
-          nt++;
-          lit_start = c0 + p;
         }
-      } else {
-        while (p < stop) {
-          const uint2 j = S.jump[p];
-          uint32_t m = j.x & 0xffffu, e = j.x >> 16;
-          if (j.x == kNoMatch) {
-            p = stop;
-            break;
+        bool valid = lane >= n && mine < stop;
+        const uint2 j = valid ? S.jump[mine] : make_uint2(kNoMatch, 0);
+        valid = valid && j.x != kNoMatch;
+        const uint32_t m = j.x & 0xffffu, e = j.x >> 16, lits = lane == n ? lit_start : c0 + mine;
+        const uint32_t all = __ballot_sync(kFull, valid);  // lanes from n on, without gaps
+        const uint32_t m_n = __shfl_sync(kFull, m, n);
+        const uint32_t lo_min = lane == n ? grp.lo_min : min(grp.lo_min, c0 + m_n);
+        const bool look = valid && ((de && j.y > lo_min) || (byte_mode && c0 + m - lits > kByteMaxLit));
+        const uint32_t looks = __ballot_sync(kFull, look);
+        const uint32_t taken = looks ? all & ((looks & (0u - looks)) - 1u) : all;
+        const uint32_t a = (uint32_t)__popc(taken);
+        if ((taken >> lane) & 1u) {
+          list(k + lane - n, lits, m, e);
+          grp.lo = c0 + m;
+          grp.hi = c0 + e;
+        }
+        if (a) {
+          p = __shfl_sync(kFull, e, n + a - 1u);
+          lit_start = c0 + p;
+          k += a;
+          nt += a;
+          if (de) grp.grow(a, c0 + m_n);
+        }
+        if (!looks) {
+          if (n + a < 32u && __shfl_sync(kFull, mine, n + a) < stop) p = stop;  // no further match
+          continue;
+        }
+        // the decision at p: in a DE stream a source may lie in the group;
+        // in a Byte stream the literals before the match may be too many
+        uint32_t from = p;
+        if (de) {
+          auto match_at = [&](uint32_t y) -> uint32_t {
+            const uint32_t x = match[y], L = x & 255u;
+            return L < 3 ? 0u : grp.cut(c0 + y, L, x >> 8);
+          };
+          for (uint32_t x; !(x = __ballot_sync(kFull, (match[p + lane] & 255u) >= 3)) || !(x & 1u);)
+            p += x ? (uint32_t)__ffs((int)x) - 1u : 32u;  // there is a match before the chunk's stop
+          uint32_t L = match_at(p);
+          if (!L) {
+            p++;
+            continue;
           }
-          if (j.y > lo_min) {
-            // a source that may lie in the group: this position's decision
-            st.in_grp = in_grp;
-            st.lo_min = lo_min;
-            auto match_at = [&](uint32_t q) -> uint32_t {
-              const uint32_t L = s_len[q];
-              return L < 3 ? 0u : de_cut(st, c0 + q, L, s_dist[q]);
-            };
-            uint32_t L = match_at(p);
-            if (!L) {
+          if (lazy) {
+            while (p + 1 < cn && L < max_match) {
+              const uint32_t L2 = match_at(p + 1);
+              if (L2 <= L) break;
               p++;
-              continue;
+              L = L2;
             }
-            if (lazy) {
-              while (p + 1 < cn && L < max_match) {
-                const uint32_t L2 = match_at(p + 1);
-                if (L2 <= L) break;
-                p++;
-                L = L2;
-              }
-            }
-            m = p;
-            e = p + L;
           }
-          if (byte_mode && c0 + m - lit_start > kByteMaxLit) literal_runs(m);
-          p = e;
-          S.list[k++] = make_uint2(lit_start, (m << 8) | (p - m));
-          nt++;
-          lit_start = c0 + p;
-          add_to_group(c0 + m, c0 + p);
+          from = p;
+          p += L;
+        } else {
+          from = S.jump[p].x & 0xffffu;
+          p = S.jump[p].x >> 16;
         }
+        if (byte_mode && c0 + from - lit_start > kByteMaxLit) {
+          // the list goes out first, then the literal runs
+          __syncwarp();
+          for (uint32_t i = lane; i < k; i += 32) {
+            const uint32_t x = S.list[i].y, at = x >> 8, u = first_token + i;
+            if (u < stride) {
+              t[u] = gmp::ParseToken{c0 + at - S.list[i].x, (match[at] & ~255u) | (x & 255u)};
+              tp[u] = S.list[i].x;
+            }
+          }
+          __syncwarp();
+          k = 0;
+          while (c0 + from - lit_start > kByteMaxLit) {
+            put(kByteMaxLit, 0);
+            lit_start += kByteMaxLit;
+            if (de) grp.add(0, 0);
+          }
+          first_token = nt;
+        }
+        list(k, lit_start, from, p);  // the same from every lane
+        k++;
+        nt++;
+        lit_start = c0 + p;
+        if (de) grp.add(c0 + from, c0 + p);
       }
-      S.p = p;
-      S.n_list = k;
+      if (lane == 0) {
+        S.p = p;
+        S.n_list = k;
+        S.first_token = first_token;
+      }
     }
     __syncthreads();
     for (uint32_t i = tid; i < S.n_list; i += kParseThreads) {
       const uint32_t x = S.list[i].y, at = x >> 8, u = S.first_token + i;
       if (u < stride) {
-        t[u] = gmp::ParseToken{c0 + at - S.list[i].x, ((uint32_t)s_dist[at] << 8) | (x & 255u)};
+        t[u] = gmp::ParseToken{c0 + at - S.list[i].x, (match[at] & ~255u) | (x & 255u)};
         tp[u] = S.list[i].x;
       }
     }
@@ -432,10 +476,10 @@ __global__ void __launch_bounds__(kParseThreads) parse_kernel(const uint8_t* bes
     c0 += S.p;
     __syncthreads();
   }
-  if (tid == 0) {
+  if (tid < 32) {
     for (; byte_mode && len - lit_start > kByteMaxLit; lit_start += kByteMaxLit) put(kByteMaxLit, 0);
     if (lit_start < len) put(len - lit_start, 0);
-    count[b] = nt;
+    if (lane == 0) count[b] = nt;
   }
 }
 
