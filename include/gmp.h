@@ -229,7 +229,7 @@ typedef struct gmp_context gmp_context;
 
 typedef struct {
   uint32_t max_block_out;   /* largest block output the scratch must hold (default 256 KiB) */
-  uint32_t warps_per_cta;   /* 0 = tuned default */
+  uint32_t warps_per_cta;   /* blocks decoded at once by a CTA (0 = tuned default) */
   uint32_t ctas_per_sm;     /* 0 = as many as fit */
   uint32_t collect_stats;   /* 1: count groups and MRR rounds (small cost) */
   uint32_t max_files;       /* largest n_files of gmp_decompress_batch (default 65536) */

@@ -270,34 +270,41 @@ static int context_alloc_scratch(gmp_context* c) {
 
 // How a launch of n_blocks blocks (0: not known here; byte_fmt: 1 if they are
 // Byte blocks, 0 if not, -1: not known here; from_host: their input is being
-// copied in) is made with the default kernels.
+// copied in, to_host: and their output back) is made with the default kernels.
 // A CTA of 16 warps decodes a block fastest, while each block has an SM; CTAs
-// of 8 warps, three on an SM, are faster than a warp per block up to about two
-// rounds of them, four for Byte blocks, which have no Huffman phase.  Measured
-// (us, one stream of 256 KiB blocks, 16 warps / 8 warps / a warp per block):
-// text of 128 blocks 363 / 421 / 1510, 256: 716 / 531 / 1520, 768: - / 1369 /
-// 1634, 1024: - / 1561 / 1637, 2048: - / 2988 / 2080; Byte records of 1024
-// blocks - / 874 / 1607, 2048: - / 1705 / 1776; text of 64 KiB blocks, 256: -
-// / 235 / 537, 1024: - / 684 / 601.  Where the device alone knows the blocks,
-// it chooses between both launches.  Blocks that are copied in meanwhile arrive
-// in order, so that finishing the first of them early counts: three rounds
-// (256 MiB of records from host memory, 1024 blocks: 1.66 ms against 2.18 with
-// a warp per block).  A context whose launches share the GPU
-// takes CTAs only for the fewest blocks, since they cost more SM time.  (The
-// scratch has a slot per warp of c->shape's grid; a CTA takes one.)
-static gmp::LaunchShape tile_shape(const gmp_context* c, uint64_t n_blocks, int byte_fmt, bool from_host = false) {
+// of 8 warps, three on an SM, are faster than a pair of warps per block up to
+// 7/4 rounds of them, two for Byte blocks, which have no Huffman phase.
+// Measured (us, one stream of 256 KiB blocks, 16 warps / 8 warps / a pair per
+// block; a round is 456 CTAs of 8 warps): text of 152 blocks 384 / 438 / 1065,
+// 304: 736 / 542 / 1164, 760: - / 1164 / 1273, 912: - / 1399 / 1296; records
+// 760: - / 1034 / 1097, 912: - / 1243 / 1121; Byte records 912: - / 787 / 809,
+// 1216: - / 995 / 822; text of 64 KiB blocks 608: - / 408 / 433, 912: - / 564 /
+// 494.  Where the device alone knows the blocks, it chooses between both
+// launches.  Blocks that are copied in meanwhile arrive in order, so that
+// finishing the first of them early counts (us, 8 warps / a pair): records from
+// host memory 1024: 1636 / 1825, 1368: 2166 / 2028; host to host 1824: 3522 /
+// 3923; Byte records 1824: 2047 / 2439 and 3688 / 3944.  A context whose
+// launches share the GPU takes CTAs only for the fewest blocks, since they cost
+// more SM time.  (The scratch has a slot per pair of c->shape's grid; a CTA
+// takes one.)
+static gmp::LaunchShape tile_shape(const gmp_context* c, uint64_t n_blocks, int byte_fmt, bool from_host = false,
+                                   bool to_host = false) {
   gmp::LaunchShape s = c->shape;
   const uint64_t slots = (uint64_t)c->shape.grid * (uint64_t)c->shape.warps_per_cta;
   const uint64_t g16 = std::min<uint64_t>(c->coop_ctas[0], slots), g8 = std::min<uint64_t>(c->coop_ctas[1], slots);
   if (!s.tile || !g16 || !g8) return s;
-  const uint64_t most = c->opts.concurrent ? g16 : from_host ? 3 * g8 : 2 * g8;
+  const uint64_t most = c->opts.concurrent              ? g16
+                        : !from_host                    ? 7 * g8 / 4
+                        : to_host || byte_fmt == 1      ? 4 * g8
+                                                        : 5 * g8 / 2;
+  const uint64_t most_byte = from_host ? most : most + most / 7;  // as takes_coop() in gmp_tile.cu
   if (n_blocks && n_blocks <= g16) {
     s.coop = 16;
     s.grid = (int)n_blocks;
-  } else if (n_blocks && n_blocks <= most * (byte_fmt == 1 ? 2u : 1u)) {
+  } else if (n_blocks && n_blocks <= (byte_fmt == 1 ? most_byte : most)) {
     s.coop = 8;
     s.grid = (int)std::min(n_blocks, g8);
-  } else if (!n_blocks || (byte_fmt < 0 && n_blocks <= 2 * most)) {
+  } else if (!n_blocks || (byte_fmt < 0 && n_blocks <= most_byte)) {
     s.coop_max = (uint32_t)most;
     s.coop_grid = (int)(n_blocks ? std::min(n_blocks, g8) : g8);
   }
@@ -781,7 +788,7 @@ static int decompress_from_host(gmp_context* c, size_t n_files, const void* cons
       int byte_fmt = -1;  // of all the streams
       for (size_t f = 0; f < n_files; f++)
         if (!files[f].idx.empty()) byte_fmt = (files[f].info.flags & 2u) || byte_fmt == 0 ? 0 : 1;
-      const gmp::LaunchShape shape = tile_shape(c, items, std::max(byte_fmt, 0), true);
+      const gmp::LaunchShape shape = tile_shape(c, items, std::max(byte_fmt, 0), true, !to_device);
       ce = gmp::launch_decode(shape, reinterpret_cast<const gmp_file_desc*>(c->h_meta + desc_off),
                               reinterpret_cast<const uint64_t*>(c->h_meta + pre_off), (uint32_t)n_pieces, nullptr,
                               c->h_status, counter, c->scratch, c->slot_bytes, c->shadow_off, c->max_seq, c->max_out,

@@ -30,7 +30,7 @@ constexpr int kWideWarpsPerSm = 16;
 size_t warp_smem_bytes(bool deep);
 cudaError_t configure_kernel(bool deep, size_t smem_bytes);
 cudaError_t occupancy(int warps_per_cta, size_t smem_bytes, bool deep, int* ctas_per_sm);
-// The default decode kernels (gmp_tile.cu): CTAs per SM, a warp per block at
+// The default decode kernels (gmp_tile.cu): CTAs per SM, a pair of warps per block at
 // this many warps per CTA, or a CTA of 8 or 16 warps per block; and the scratch
 // a block's slot needs for blocks of up to max_out bytes.
 cudaError_t tile_occupancy(int warps_per_cta, int* ctas_per_sm);

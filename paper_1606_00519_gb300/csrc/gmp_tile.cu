@@ -3,42 +3,47 @@
 // 32-sequence groups and resolution rounds the statistics and the ablation of
 // Sec. 5.1 are about.
 //
-// A warp decodes a block in two phases:
+// A pair of warps decodes a block in two phases:
 //
-//  Phase A, Huffman decoding (Sec. 3.2.1): lane j decodes sub-block j (lanes
-//  take j, j+32 for K > 32).  A lookup yields up to two literals and the
-//  match length after them when their codes fit the table's bits together,
-//  so that a sequence takes about one step.  Each sequence becomes an 8-byte
-//  record with its literals inside {literal bytes, distance | match length
-//  << 16 | literal count << 24}; a longer literal string takes further
-//  records of 3 or 4 literals without a match.  Records go to the warp's
-//  scratch slot.
+//  Phase A, Huffman decoding (Sec. 3.2.1), the first warp: lane j decodes
+//  sub-block j (lanes take j, j+32 for K > 32).  A lookup yields up to two
+//  literals and the match length after them when their codes fit the table's
+//  bits together, so that a sequence takes about one step.  Each sequence
+//  becomes an 8-byte record with its literals inside {literal bytes, distance
+//  | match length << 16 | literal count << 24}; a longer literal string takes
+//  further records of 3 or 4 literals without a match.  Records go to the
+//  pair's scratch slot.
 //
-//  Phase B, LZ77 decompression (Sec. 3.2.2): the warp takes 32 records per
-//  group and writes the group's output 32 bytes at a time, one byte per lane
-//  (a tile).  The group's literal strings and matches are segments; a bit
-//  per segment start and a population count give each byte its segment, and
-//  the segment's entry the shared-memory address its byte comes from: the
-//  output window, the literals, or the staging of sources older than the
-//  window.  Tiles run in output order, so that every byte below a tile is
-//  complete when the tile starts and no resolution rounds are needed;
-//  sources inside the tile itself (rare) are followed to the byte they
-//  repeat by pointer doubling over the warp's lanes.  So MRR and DE streams
-//  take the same path at the same speed.
+//  Phase B, LZ77 decompression (Sec. 3.2.2): the first warp lays out groups of
+//  64 records, two per lane, while the second writes the group before, 32
+//  bytes at a time, one byte per lane (a tile).  The group's literal strings
+//  and matches are segments; a bit per segment start and a population count
+//  give each byte its segment, and the segment's entry the shared-memory
+//  address its byte comes from: the output window, the literals, or the
+//  staging of sources older than the window.  Tiles run in output order, so
+//  that every byte below a tile is complete when the tile starts and no
+//  resolution rounds are needed; four tiles whose sources all lie below the
+//  first are written at once.  Sources inside the tile itself (rare) are
+//  followed to the byte they repeat by pointer doubling over the warp's lanes.
+//  So MRR and DE streams take the same path at the same speed.
 //
 //  Byte blocks (Gompresso/Byte, Sec. 3.1) run phase B on the stream's own
 //  records, with each group's records checked before it is staged.
 //
-//
-// What bounds it and what it measured (GB300, 152 SMs): with every SM full the
-// integer pipe and the load/store unit (32 lanes reading and writing 32
-// places), on small launches one warp's chain of dependent instructions.  The
-// Huffman step without branches, records of 8 bytes with their literals
-// inside and stored four at a time (single 8-byte stores cost 0.5 of 3.5 ms
-// on 2 x 512 MiB of records), and tiles in place of per-sequence copies with
-// resolution rounds: 2 x 512 MiB of records, MRR and DE in one launch, 4.53 ->
-// 3.48 ms; 2 x 256 MiB of text 2.66 -> 2.15; 107 files of 256 MiB together
-// 2.22 -> 1.73; one 64 MiB stream 1.95 -> 1.60 (before: gmp_decode.cu).
+// What bounds it and what it measured (GB300, 152 SMs): the number of
+// instructions with every SM full (2.4 warp instructions per byte of text,
+// 61 % of the issue slots), and a block's chain of dependent ones on small
+// launches.  The Huffman step without branches, records of 8 bytes with their
+// literals inside and stored four at a time (single 8-byte stores cost 0.5 of
+// 3.5 ms on 2 x 512 MiB of records), and tiles in place of per-sequence copies
+// with resolution rounds: 2 x 512 MiB of records, MRR and DE in one launch,
+// 4.53 -> 3.48 ms; 2 x 256 MiB of text 2.66 -> 2.15 (before: gmp_decode.cu).
+// A second warp for the writing, which doubles the warps on an SM in the same
+// shared memory (16 blocks), and groups of 64 records instead of 32, whose
+// layout and hand-over cost little more than one of 32: records 3.37 -> 2.90,
+// text 2.08 -> 1.76, 1 GiB of Byte records 3.17 -> 1.90 (the pair alone, with
+// groups of 32: 3.36, 2.08, 2.48).  64 registers a thread are what 32 warps
+// leave; phase A spills a few of them.
 // Every read of the compressed stream is bounds-checked; every loop over
 // input data is bounded by sizes checked against the block header; corrupt
 // input sets the caller's status word and abandons the block.
@@ -81,12 +86,12 @@ __device__ __forceinline__ uint32_t off_entry(uint32_t os, uint32_t len) {
 // Working space of the table build; overlaid by the bitstream ring.
 struct BuildSmem {
   Canon cll;
-  uint32_t run[16];
+  uint32_t run[2][16];
   uint16_t sorted_ll[N_LL + 1];
   uint8_t lens[N_LL + N_OFF + 3];
 };
 
-constexpr int kLLBits = 11, kOffBits = 9;  // a warp's tables
+constexpr int kLLBits = 11, kOffBits = 9;  // a pair's tables
 constexpr uint32_t kChunksAhead = 4;  // 16-byte bitstream chunks held per lane
 struct TileSmemA {
   uint32_t ll[1 << kLLBits];
@@ -103,19 +108,33 @@ struct TileSmemA {
 // Phase B.  The output window `buf` holds at least the last kHist output
 // bytes and the group being written: it slides down (by a multiple of 16)
 // when a group would not fit.
-constexpr uint32_t kHist = 4096;
-constexpr uint32_t kGroupMax = 32 * 68;  // 4 literals and a match of 64 per record
-constexpr uint32_t kBuf = kHist + 16 + kGroupMax;
+constexpr uint32_t kHist = 1024;
+constexpr uint32_t kGroupRecs = 64;          // records of a group: two per lane, or half of them if they
+constexpr uint32_t kGroupMax = 32 * 68;  // write more than this (4 literals and a match of 64 per record)
+constexpr uint32_t kBuf = 5840;
 constexpr uint32_t kFlush = 512;    // output bytes per flush (one 16-byte store per lane)
-constexpr uint32_t kFarSlot = 80;   // a 64-byte source spans at most 5 aligned 16-byte chunks
+constexpr uint32_t kFarChunks = 32 * 5;  // 16-byte chunks; a 64-byte source spans at most 5 aligned ones
 constexpr uint32_t kLitStage = 512; // a Byte group's literal run, with alignment
 constexpr uint32_t kMarkWords = (kGroupMax + 127) / 128 * 4;
 struct TileSmemB {
   uint8_t lit[2][kLitStage];
-  uint8_t far[2][32][kFarSlot];
-  uint32_t seg[2][64];
+  uint8_t far[2][16 * kFarChunks];
+  uint32_t seg[2][2 * kGroupRecs];
   uint32_t mark[2][kMarkWords];
   uint8_t buf[kBuf + 32];  // a last tile may write up to 31 bytes past its group
+};
+struct Window {
+  uint32_t g0;       // output position of the next byte
+  uint32_t cur;      // its place in buf
+  uint32_t base;     // output position of buf[0] (a multiple of 16): g0 - cur
+  uint32_t flushed;  // output bytes stored (a multiple of kFlush)
+};
+// What the first warp of a pair hands to the second: the block, and in phase B
+// group after group.
+enum Work : uint32_t { kEnd, kSkip, kByte, kHuffman };
+enum Step : uint32_t { kGroup, kSlow, kDone, kAbandon };
+struct StepMsg {
+  uint32_t what, total, shift;  // kGroup: its bytes, and what the window slides by before it
 };
 struct __align__(64) TileSmem {
   union {
@@ -124,9 +143,25 @@ struct __align__(64) TileSmem {
   } u;
   uint32_t sb_out[MAX_SUB];  // sub-block output start
   uint32_t sb_cnt[MAX_SUB];  // its records
+  BlockView view;
+  uint8_t* out;
+  uint32_t work, file;
+  int32_t result[3];  // of the parts of the table build
+  StepMsg step[2];
+  Window win;                  // after a slow group
+  uint32_t slow_t0, slow_t1;   // its records
+  const uint8_t* slow_lits;
 };
 static_assert(kBuf % 16 == 0 && sizeof(TileSmem) % 16 == 0, "16-byte copies");
-static_assert(sizeof(TileSmem) * 4 + 1024 <= 57 * 1024, "16 warps per SM in CTAs of 4");
+static_assert(kHist >= kFlush + 80, "what slow_group copies from the output is flushed");
+static_assert(kGroupMax + kFlush + 80 + 16 + kGroupMax <= kBuf, "two groups of the longest matches");
+static_assert(sizeof(TileSmem) * 4 + 1024 <= 57 * 1024, "16 pairs per SM in CTAs of 4");
+
+// Both warps of a pair: 64 threads at the pair's hardware barrier (the kernel
+// uses no __syncthreads).
+__device__ __forceinline__ void pair_sync() {
+  asm volatile("bar.sync %0, 64;" ::"r"(threadIdx.x >> 6) : "memory");
+}
 
 // First record of sub-block j, whose output starts at `out`: a record covers
 // at least 3 bytes of output but for a sub-block's last one, and a corrupt
@@ -503,59 +538,66 @@ __device__ __forceinline__ void unpack_lens(uint8_t* lens, const uint8_t* B, uin
   }
 }
 
-// Phase A of one block by one warp; false: the block's status is set.
-__device__ bool huffman_block(TileSmem& S, const BlockView& V, int32_t* status, uint2* rec) {
-  const uint32_t lane = lane_id();
+// Phase A of one block by the warp pair; false: the block's status is set.
+__device__ __forceinline__ bool huffman_block(TileSmem& S, const BlockView& V, int32_t* status, uint2* rec,
+                                              uint32_t half) {
+  const uint32_t lane = lane_id(), t = 32 * half + lane;
   TileSmemA& A = S.u.a;
-  const uint32_t bs_off = (192u + 12u * V.K + 15u) & ~15u;  // bitstream start within the block
-  int err = sub_block_table(V, (V.comp_bytes - bs_off) * 8ull, A.sb_bit, S.sb_out, A.sb_seq);
-  if (err) {
-    if (lane == 0) set_status(status, err);
-    return false;
-  }
-  unpack_lens(A.u.build.lens, V.B, lane, 32);
-  __syncwarp();
   BuildSmem& T = A.u.build;
-  const int n_ll = build_canon(T.cll, T.run, T.sorted_ll, T.lens, N_LL);
-  const int n_off = build_canon(A.coff, T.run, A.sorted_off, T.lens + N_LL, N_OFF);
-  if (n_ll < 0 || n_off < 0) {
-    if (lane == 0) set_status(status, GMP_STATUS_BAD_HEADER);
+  const uint32_t bs_off = (192u + 12u * V.K + 15u) & ~15u;  // bitstream start within the block
+  unpack_lens(T.lens, V.B, t, 64);
+  pair_sync();
+  if (half == 0) {
+    const int r = build_canon(T.cll, T.run[0], T.sorted_ll, T.lens, N_LL);
+    if (lane == 0) S.result[0] = r;
+  } else {
+    const int r = build_canon(A.coff, T.run[1], A.sorted_off, T.lens + N_LL, N_OFF);
+    const int e = sub_block_table(V, (V.comp_bytes - bs_off) * 8ull, A.sb_bit, S.sb_out, A.sb_seq);
+    if (lane == 0) {
+      S.result[1] = r;
+      S.result[2] = e;
+    }
+  }
+  pair_sync();
+  const int n_ll = S.result[0], n_off = S.result[1];
+  int err = S.result[2] ? S.result[2] : n_ll < 0 || n_off < 0 ? (int)GMP_STATUS_BAD_HEADER : 0;
+  if (err) {
+    if (t == 0) set_status(status, err);
     return false;
   }
-  fill_ll<kLLBits>(A.ll, T.cll, T.sorted_ll, n_ll == 0, V.max_match, lane, 32);
-  fill_off<kOffBits>(A.off, A.coff, A.sorted_off, n_off == 0, lane, 32);
-  __syncwarp();  // the ring takes the build's place
-  const uint8_t* bs = V.B + bs_off;
-  const uint32_t n_chunks = (uint32_t)min((uint64_t)0xffffffffu, (V.comp_bytes - bs_off) / 16);
-  for (uint32_t jb = 0; jb < V.K; jb += 32) {
-    const uint32_t j = jb + lane;
-    SubBlock sb{0, 0, 0, 0, 0, 0};
-    if (j < V.K) {
-      const uint8_t* e = V.B + 192 + 12 * j;
-      sb = SubBlock{A.sb_bit[j], ld_u32_nc(e), S.sb_out[j], ld_u32_nc(e + 4), A.sb_seq[j], ld_u32_nc(e + 8)};
+  fill_ll<kLLBits>(A.ll, T.cll, T.sorted_ll, n_ll == 0, V.max_match, t, 64);
+  fill_off<kOffBits>(A.off, A.coff, A.sorted_off, n_off == 0, t, 64);
+  pair_sync();  // the ring takes the build's place
+  if (half == 0) {
+    const uint8_t* bs = V.B + bs_off;
+    const uint32_t n_chunks = (uint32_t)min((uint64_t)0xffffffffu, (V.comp_bytes - bs_off) / 16);
+    for (uint32_t jb = 0; jb < V.K; jb += 32) {
+      const uint32_t j = jb + lane;
+      SubBlock sb{0, 0, 0, 0, 0, 0};
+      if (j < V.K) {
+        const uint8_t* e = V.B + 192 + 12 * j;
+        sb = SubBlock{A.sb_bit[j], ld_u32_nc(e), S.sb_out[j], ld_u32_nc(e + 4), A.sb_seq[j], ld_u32_nc(e + 8)};
+      }
+      const uint32_t cnt = huffman_lane<kLLBits, kOffBits, true>(
+          A.ll, A.off, A.coff, A.sorted_off, A.u.bits[lane], bs, n_chunks, j < V.K, n_ll == 0, sb, V.n_seq, V.window,
+          rec + rec_start(sb.out, j), err);
+      if (j < V.K) S.sb_cnt[j] = cnt;
     }
-    const uint32_t cnt = huffman_lane<kLLBits, kOffBits, true>(A.ll, A.off, A.coff, A.sorted_off, A.u.bits[lane], bs, n_chunks, j < V.K, n_ll == 0,
-                                      sb, V.n_seq, V.window, rec + rec_start(sb.out, j), err);
-    if (j < V.K) S.sb_cnt[j] = cnt;
+    if (err) set_status(status, err);
+    err = __any_sync(FULL, err != 0);
+    if (lane == 0) S.result[0] = err;
   }
-  if (err) set_status(status, err);
-  if (__any_sync(FULL, err != 0)) return false;
-  __syncwarp();  // the records are visible to the whole warp
-  return true;
+  pair_sync();  // the records are visible to the first warp, the tables' place is free
+  return S.result[0] == 0;
 }
 
 // ---------------------------------------------------------------------------
 // Phase B.
-struct Window {
-  uint32_t g0;       // output position of the next byte
-  uint32_t cur;      // its place in buf
-  uint32_t base;     // output position of buf[0] (a multiple of 16): g0 - cur
-  uint32_t flushed;  // output bytes stored (a multiple of kFlush)
-};
 struct Group {
   uint32_t total, lits, shift;
   int err;
-  bool slow;  // a Byte group too large for the window or the literal staging
+  uint32_t end;  // its last record, plus one
+  bool slow;  // a Byte group too large for the window or the literal staging, even half of it
 };
 
 __device__ __forceinline__ void slide(uint8_t* buf, Window& w, uint32_t shift) {
@@ -641,20 +683,21 @@ __device__ __noinline__ void slow_group(uint8_t* buf, uint32_t cap, uint32_t his
   }
 }
 
+// The first warp of a pair reads the records and lays out group after group;
+// the second writes them.
 template <bool BYTE>
-__device__ __forceinline__ void lz_block(TileSmem& SS, const BlockView& V, int32_t* status, const uint2* rec,
-                                         uint8_t* out_blk) {
+__device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, int32_t* status, const uint2* rec,
+                                              uint8_t* out_blk) {
   TileSmemB& S = SS.u.b;
-  const uint32_t lane = lane_id(), lt = (1u << lane) - 1u, le = lt | (1u << lane);
+  const uint32_t lane = lane_id();
   const bool vec_ok = (((uintptr_t)out_blk) & 15u) == 0;
   const uint8_t* recs = V.B + 16;           // Byte blocks: the stream's records
   const uint8_t* lits = V.B + V.lit_off;    // and literals
   const uint32_t buf_a = smem_addr(S.buf);
 
-  // records of the next group: Huffman blocks {literals, distance | match
-  // length << 16 | literal count << 24} of one sub-block, Byte blocks the
-  // stream's word; zero past the end
-  uint32_t i_grp = 0;
+  // the lane's two records of the group at i0: Huffman blocks {literals,
+  // distance | match length << 16 | literal count << 24} of one sub-block,
+  // Byte blocks {-, the stream's word}; zero past the end
   uint32_t j = 0, i0 = 0, n_j = 0;  // sub-block, record within it, its records (Byte: the block's)
   const uint2* rec_j = rec;
   if (BYTE) {
@@ -664,14 +707,25 @@ __device__ __forceinline__ void lz_block(TileSmem& SS, const BlockView& V, int32
     if (j < V.K) rec_j = rec + rec_start(SS.sb_out[j], j);
     else n_j = 0;
   }
-  auto load = [&]() -> uint2 {
-    const uint32_t i = i0 + lane;
-    if (i >= n_j) return make_uint2(0, 0);
-    if (BYTE) return make_uint2(0, ld_u32_nc(recs + 4ull * i));
-    return __ldcg(rec_j + i);
+  auto load = [&]() -> uint4 {
+    const uint32_t i = i0 + 2 * lane;
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (i < n_j) {
+      // whole pairs: Byte blocks' records are followed by padding when their
+      // number is odd, and a sub-block's have room for one more
+      if (BYTE) {
+        const uint2 u = __ldg(reinterpret_cast<const uint2*>(recs + 4ull * i));
+        v.y = u.x;
+        v.w = u.y;
+      } else {
+        v = __ldcg(reinterpret_cast<const uint4*>(rec_j + i));
+      }
+      if (i + 1u >= n_j) v.z = v.w = 0;
+    }
+    return v;
   };
-  auto step = [&]() {  // to the next group
-    i0 += 32;
+  auto step = [&](uint32_t n) {  // past n records
+    i0 += min(n, n_j - i0);
     if (i0 < n_j || BYTE) return;
     i0 = 0;
     n_j = 0;
@@ -679,102 +733,221 @@ __device__ __forceinline__ void lz_block(TileSmem& SS, const BlockView& V, int32
     if (j < V.K) rec_j = rec + rec_start(SS.sb_out[j], j);
   };
 
-  // Lays out the group of records r at window w (its state before the
-  // group): segment starts and entries, far sources and Byte literals staged
-  // by cp.async.
-  auto prep = [&](uint2 r, const Window& w, uint32_t litpos, int stage) -> Group {
-    Group G;
-    G.err = 0;
-    G.slow = false;
-    G.shift = 0;
-    uint32_t ll, ml, dist, dst;
-    if (BYTE) {
-      const uint32_t m = (r.y >> 10) & 63u;
-      ll = r.y & 1023u;
-      ml = m ? m + 2u : 0u;  // code 63 has no length; as 65 it fails the check below
-      dist = (r.y >> 16) + 1u;
-      const uint32_t packed = (ll << 16) | (ll + ml);  // a group's sums stay below 2^16
-      const uint32_t inc = warp_incl_scan(packed), sum = __shfl_sync(FULL, inc, 31);
-      G.total = sum & 0xffffu;
-      G.lits = sum >> 16;
-      dst = (inc & 0xffffu) - (ll + ml);
-      const uint32_t mst = w.g0 + dst + ll;
-      if (__any_sync(FULL, ml > V.max_match)) G.err = GMP_STATUS_CORRUPT_SYMBOL;
-      else if (__any_sync(FULL, ml > 0 && (dist > V.window || dist > mst))) G.err = GMP_STATUS_BAD_OFFSET;
-      else if ((uint64_t)w.g0 + G.total > V.out_bytes || (uint64_t)litpos + G.lits > V.n_lit)
-        G.err = GMP_STATUS_OUTPUT_OVERRUN;
-      if (G.err) return G;
-      const uint32_t l0 = litpos & ~15u, l1 = (litpos + G.lits + 15u) & ~15u;
-      if (G.total > kGroupMax || l1 - l0 > kLitStage) {
-        G.slow = true;
-        return G;
+  uint4 r = load();
+  // Lays out the next group (records r) at window w, its state before the
+  // group, which follows one of `prev` bytes: segment starts and entries, far
+  // sources and Byte literals staged by cp.async.
+  auto prep = [&](const Window& w, uint32_t prev, uint32_t litpos, uint32_t stage) -> Group {
+    Group G{0, 0, 0, 0, 0, false};
+    uint32_t ll[2], ml[2], dist[2], lit_x[2] = {r.x, r.z};
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+      const uint32_t y = k ? r.w : r.y;
+      if (BYTE) {
+        const uint32_t m = (y >> 10) & 63u;
+        ll[k] = y & 1023u;
+        ml[k] = m ? m + 2u : 0u;  // code 63 has no length; as 65 it fails the check below
+        dist[k] = (y >> 16) + 1u;
+      } else {
+        ll[k] = y >> 24;
+        ml[k] = (y >> 16) & 255u;
+        dist[k] = y & 0xffffu;
       }
-      if (16u * lane < l1 - l0) cp_async16(S.lit[stage] + 16u * lane, lits + l0 + 16u * lane);
-      // literal string's place in the staging
-      r.x = (litpos & 15u) + (inc >> 16) - ll;
-    } else {
-      ll = r.y >> 24;
-      ml = (r.y >> 16) & 255u;
-      dist = r.y & 0xffffu;
-      const uint32_t inc = warp_incl_scan(ll + ml);
-      G.total = __shfl_sync(FULL, inc, 31);
-      G.lits = 0;
-      dst = inc - (ll + ml);
-      *reinterpret_cast<uint32_t*>(S.lit[stage] + 4u * lane) = r.x;
-      r.x = 4u * lane;
     }
-    G.shift = w.cur + G.total > kBuf ? (w.cur - kHist) & ~15u : 0u;
+    // The second warp may still be writing the group before: everything up to
+    // that one's start is complete, and stored but for a flush row.  Sources
+    // older than the window must be stored, so this much stays in it.
+    const uint32_t hist = max(kHist, prev + kFlush + 80u), near = min(w.cur, hist);
+    uint32_t n = kGroupRecs, dst, segs, chunks, lit_at;
+    for (;;) {
+      // one scan gives output positions, segment numbers and places for the
+      // chunks of sources that may be older than the window (in Byte blocks,
+      // whose literal strings are longer, two scans)
+      uint32_t own = 0, own_l = 0;
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+        const uint32_t nc = ml[k] && dist[k] > near ? (ml[k] + 30u) >> 4 : 0u, ns = (ll[k] ? 1u : 0u) + (ml[k] ? 1u : 0u);
+        own += ll[k] + ml[k] + (BYTE ? ns << 20 : (ns << 13) + (nc << 21));
+        own_l += ll[k] + (nc << 16);
+      }
+      const uint32_t inc = warp_incl_scan(own), sum = __shfl_sync(FULL, inc, 31), ex = inc - own;
+      uint32_t n_chunks;
+      bool fits;
+      if (BYTE) {
+        const uint32_t inc_l = warp_incl_scan(own_l), sum_l = __shfl_sync(FULL, inc_l, 31), ex_l = inc_l - own_l;
+        G.total = sum & 0xfffffu;
+        G.lits = sum_l & 0xffffu;
+        n_chunks = sum_l >> 16;
+        dst = ex & 0xfffffu;
+        segs = ex >> 20;
+        chunks = ex_l >> 16;
+        lit_at = (litpos & 15u) + (ex_l & 0xffffu);
+        bool long_match = false, bad = false;
+        uint32_t at = w.g0 + dst;
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+          at += ll[k];
+          long_match = long_match || ml[k] > V.max_match;
+          bad = bad || (ml[k] > 0 && (dist[k] > V.window || dist[k] > at));
+          at += ml[k];
+        }
+        G.err = 0;
+        if (__any_sync(FULL, long_match)) G.err = GMP_STATUS_CORRUPT_SYMBOL;
+        else if (__any_sync(FULL, bad)) G.err = GMP_STATUS_BAD_OFFSET;
+        else if ((uint64_t)w.g0 + G.total > V.out_bytes || (uint64_t)litpos + G.lits > V.n_lit)
+          G.err = GMP_STATUS_OUTPUT_OVERRUN;
+        fits = !G.err && ((litpos + G.lits + 15u) & ~15u) - (litpos & ~15u) <= kLitStage;
+      } else {
+        G.total = sum & 0x1fffu;
+        n_chunks = sum >> 21;
+        dst = ex & 0x1fffu;
+        segs = (ex >> 13) & 255u;
+        chunks = ex >> 21;
+        lit_at = 8u * lane;
+        fits = true;
+      }
+      fits = fits && G.total <= kGroupMax && n_chunks <= kFarChunks;
+      if (fits) break;
+      if (n == 32u) {  // (Byte only)
+        if (G.err) return G;
+        G.slow = true;
+        break;
+      }
+      n = 32;
+      if (lane >= 16u) ll[0] = ll[1] = ml[0] = ml[1] = 0;
+    }
+    // the records after this group are on their way while it is laid out
+    G.end = min(i0 + n, n_j);
+    step(n);
+    r = load();
+    if (BYTE && G.slow) return G;
+    G.shift = w.cur + G.total > kBuf ? (w.cur - hist) & ~15u : 0u;
     const uint32_t cur = w.cur - G.shift, base = w.base + G.shift;
+    if (BYTE) {
+      const uint32_t l0 = litpos & ~15u, l1 = (litpos + G.lits + 15u) & ~15u;
+      if (16u * lane < l1 - l0) cp_async16(S.lit[stage] + 16u * lane, lits + l0 + 16u * lane);
+    } else {
+      *reinterpret_cast<uint2*>(S.lit[stage] + 8u * lane) = make_uint2(lit_x[0], lit_x[1]);
+    }
     // segment starts
     uint32_t* mark = S.mark[stage];
     for (uint32_t x = lane; x < ((G.total + 127u) >> 7) * 4u; x += 32) mark[x] = 0;
     __syncwarp();
-    const uint32_t mst = dst + ll, src = w.g0 + mst - dist;
-    const uint32_t b_l = __ballot_sync(FULL, ll > 0), b_m = __ballot_sync(FULL, ml > 0);
-    uint32_t k = __popc(b_l & lt) + __popc(b_m & lt);
     uint32_t* seg = S.seg[stage];
-    if (ll) {
-      atomicOr(mark + (dst >> 5), 1u << (dst & 31u));
-      seg[k++] = smem_addr(S.lit[stage]) + r.x - dst;
-    }
-    const bool is_far = ml > 0 && src < base;
-    if (ml) {
-      atomicOr(mark + (mst >> 5), 1u << (mst & 31u));
-      seg[k] = is_far ? smem_addr(S.far[stage][lane]) + (src & 15u) - mst : buf_a + cur - dist;
-    }
-    // sources older than the window: at least kHist - 64 bytes back, hence
-    // flushed (at most a group and a flush row are not)
-    uint8_t* slot = S.far[stage][lane];
-    if (vec_ok) {
-      const uint8_t* g = out_blk + (src & ~15u);
-      const uint32_t nc = is_far ? ((src & 15u) + ml + 15u) >> 4 : 0u;
-      if (nc > 0) cp_async16(slot, g);
-      if (nc > 1) cp_async16(slot + 16, g + 16);
-      if (__any_sync(FULL, nc > 2)) {
-        if (nc > 2) cp_async16(slot + 32, g + 32);
-        if (nc > 3) cp_async16(slot + 48, g + 48);
-        if (nc > 4) cp_async16(slot + 64, g + 64);
+    const uint32_t lit_a = smem_addr(S.lit[stage]);
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+      if (ll[k]) {
+        atomicOr(mark + (dst >> 5), 1u << (dst & 31u));
+        seg[segs++] = lit_a + lit_at - dst;
       }
-    } else if (is_far) {
-      for (uint32_t i = 0; i < ml; i++) slot[(src & 15u) + i] = (uint8_t)__ldcg(out_blk + src + i);
+      dst += ll[k];
+      lit_at += BYTE ? ll[k] : 4u;
+      if (ml[k]) {
+        const uint32_t src = w.g0 + dst - dist[k];
+        const bool is_far = src < base;
+        uint8_t* place = S.far[stage] + 16u * chunks;
+        atomicOr(mark + (dst >> 5), 1u << (dst & 31u));
+        seg[segs++] = is_far ? smem_addr(place) + (src & 15u) - dst : buf_a + cur - dist[k];
+        if (is_far) {
+          // sources older than the window
+          if (vec_ok) {
+            const uint8_t* g = out_blk + (src & ~15u);
+            const uint32_t nc = ((src & 15u) + ml[k] + 15u) >> 4;
+            cp_async16(place, g);
+            if (nc > 1) cp_async16(place + 16, g + 16);
+            for (uint32_t c = 2; c < nc; c++) cp_async16(place + 16u * c, g + 16u * c);
+          } else {
+            for (uint32_t i = 0; i < ml[k]; i++) place[(src & 15u) + i] = (uint8_t)__ldcg(out_blk + src + i);
+          }
+        }
+        chunks += dist[k] > near ? (ml[k] + 30u) >> 4 : 0u;
+      }
+      dst += ml[k];
     }
     return G;
   };
 
+  Window w{0, 0, 0, 0};
+  uint32_t litpos = 0, prev = 0, stage = 0;
+  auto tell = [&](uint32_t what, uint32_t total, uint32_t shift) {
+    if (lane == 0) SS.step[stage] = StepMsg{what, total, shift};
+    pair_sync();
+    stage ^= 1u;
+  };
+  while (i0 < n_j) {
+    const uint32_t t_cur = i0;
+    const Group G = prep(w, prev, litpos, stage);
+    if (BYTE && G.err) {
+      if (lane == 0) set_status(status, G.err);
+      tell(kAbandon, 0, 0);
+      return;
+    }
+    if (BYTE && G.slow) {
+      if (lane == 0) {
+        SS.slow_t0 = t_cur;
+        SS.slow_t1 = G.end;
+        SS.slow_lits = lits + litpos;
+      }
+      tell(kSlow, 0, 0);
+      pair_sync();  // it is written
+      stage ^= 1u;
+      w = SS.win;
+      prev = 0;
+    } else {
+      cp_async_commit();
+      cp_async_wait<0>();
+      tell(kGroup, G.total, G.shift);
+      w.g0 += G.total;
+      w.base += G.shift;
+      w.cur = w.g0 - w.base;
+      prev = G.total;
+    }
+    litpos += G.lits;
+  }
+  if ((w.g0 != V.out_bytes || (BYTE && litpos != V.n_lit)) && lane == 0) set_status(status, GMP_STATUS_OUTPUT_OVERRUN);
+  tell(kDone, 0, 0);
+}
+
+// The second warp writes the groups, slides the window and stores whole rows
+// of output.
+__device__ __forceinline__ void write_block(TileSmem& SS, uint8_t* out_blk) {
+  TileSmemB& S = SS.u.b;
+  const uint32_t lane = lane_id(), le = (2u << lane) - 1u;
+  const bool vec_ok = (((uintptr_t)out_blk) & 15u) == 0;
+  const uint32_t buf_a = smem_addr(S.buf);
+
   // Writes the group's bytes at buf + cur, tile by tile.
-  auto tiles = [&](const Group& G, uint32_t cur, int stage) {
+  auto tiles = [&](uint32_t total, uint32_t cur, uint32_t stage) {
     const uint32_t* mark = S.mark[stage];
     const uint32_t* seg = S.seg[stage];
     uint32_t tile_a = buf_a + cur;  // shared address of the tile's first byte
     uint32_t before = 0xffffffffu;  // segments started before the tile, less one
-    for (uint32_t t = 0; t < G.total; t += 128, tile_a += 128) {
+    // the addresses of 128 bytes, a byte of each of four tiles per lane
+    uint32_t a0, a1, a2, a3;
+    auto look = [&](uint32_t t) {
       const uint4 m = *reinterpret_cast<const uint4*>(mark + (t >> 5));
-      const uint32_t c0 = before + __popc(m.x), c1 = c0 + __popc(m.y), c2 = c1 + __popc(m.z);
-      const uint32_t o = t + lane;
-      uint32_t a0 = seg[before + __popc(m.x & le)] + o, a1 = seg[c0 + __popc(m.y & le)] + o + 32u;
-      uint32_t a2 = seg[c1 + __popc(m.z & le)] + o + 64u, a3 = seg[c2 + __popc(m.w & le)] + o + 96u;
+      const uint32_t c0 = before + __popc(m.x), c1 = c0 + __popc(m.y), c2 = c1 + __popc(m.z), o = t + lane;
+      a0 = seg[before + __popc(m.x & le)] + o;
+      a1 = seg[c0 + __popc(m.y & le)] + o + 32u;
+      a2 = seg[c1 + __popc(m.z & le)] + o + 64u;
+      a3 = seg[c2 + __popc(m.w & le)] + o + 96u;
       before = c2 + __popc(m.w);
-      const uint32_t n = G.total - t;
+    };
+    if (total) look(0);
+    for (uint32_t t = 0; t < total; t += 128, tile_a += 128) {
+      const uint32_t n = total - t;
+      if (!__any_sync(FULL, max(max(a0, a1), max(a2, a3)) >= tile_a)) {
+        // all 128 bytes at once; the next addresses are looked up meanwhile
+        const uint32_t v0 = lds_u8(a0), v1 = lds_u8(a1), v2 = lds_u8(a2), v3 = lds_u8(a3);
+        if (n > 128u) look(t + 128);
+        sts_u8(tile_a + lane, v0);
+        if (n > 32u) sts_u8(tile_a + 32u + lane, v1);
+        if (n > 64u) sts_u8(tile_a + 64u + lane, v2);
+        if (n > 96u) sts_u8(tile_a + 96u + lane, v3);
+        __syncwarp();
+        continue;
+      }
       // a source inside its own tile is not written yet: follow it (to a
       // lower lane each time) to the address its byte comes from
       auto resolve = [&](uint32_t& a, uint32_t tile) {
@@ -803,69 +976,29 @@ __device__ __forceinline__ void lz_block(TileSmem& SS, const BlockView& V, int32
         sts_u8(tile_a + 96u + lane, lds_u8(a3));
         __syncwarp();
       }
+      if (n > 128u) look(t + 128);
     }
   };
 
   Window w{0, 0, 0, 0};
-  uint32_t litpos = 0, t_cur = 0;  // Byte: the group's first literal and record
-  uint2 r = load();
-  Group G{0, 0, 0, 0, false};  // an empty group before the first
-  for (bool more = true; more;) {
-    if (BYTE && G.err) {
-      cp_async_wait<0>();
-      if (lane == 0) set_status(status, G.err);
+  for (uint32_t stage = 0;; stage ^= 1u) {
+    pair_sync();
+    const StepMsg m = SS.step[stage];
+    if (m.what == kGroup) {
+      if (m.shift) slide(S.buf, w, m.shift);
+      tiles(m.total, w.cur, stage);
+      w.g0 += m.total;
+      w.cur += m.total;
+      flush(S.buf, w, out_blk, vec_ok, lane, 32);
+    } else if (m.what == kSlow) {
+      slow_group(S.buf, kBuf, kHist, w, SS.view.B + 16, SS.slow_t0, SS.slow_t1, SS.slow_lits, out_blk, vec_ok);
+      if (lane == 0) SS.win = w;
+      pair_sync();
+      stage ^= 1u;
+    } else {
+      if (m.what == kDone) flush_rest(S.buf, w, out_blk, vec_ok, lane, 32);
       return;
     }
-    if (BYTE && G.slow) {
-      cp_async_wait<0>();
-      slow_group(S.buf, kBuf, kHist, w, recs, t_cur, min(t_cur + 32u, V.n_seq), lits + litpos, out_blk, vec_ok);
-      litpos += G.lits;
-      G = Group{0, 0, 0, 0, false};
-    }
-    // the next group is laid out, and its copies started, before this
-    // group's bytes are written
-    more = i0 < n_j;
-    const int stage = (int)((i_grp++) & 1u);
-    Window after = w;
-    after.g0 += G.total;
-    after.base += G.shift;
-    after.cur = after.g0 - after.base;
-    const Group N = prep(r, after, litpos + G.lits, stage);
-    t_cur = i0;
-    step();
-    r = load();
-    cp_async_commit();
-    cp_async_wait<1>();
-    __syncwarp();
-    if (G.shift) slide(S.buf, w, G.shift);
-    tiles(G, w.cur, stage ^ 1);
-    w.g0 += G.total;
-    w.cur += G.total;
-    litpos += G.lits;
-    flush(S.buf, w, out_blk, vec_ok, lane, 32);
-    G = N;
-  }
-  cp_async_wait<0>();
-  __syncwarp();
-  flush_rest(S.buf, w, out_blk, vec_ok, lane, 32);
-  if ((w.g0 != V.out_bytes || (BYTE && litpos != V.n_lit)) && lane == 0) set_status(status, GMP_STATUS_OUTPUT_OVERRUN);
-}
-
-__device__ __forceinline__ void tile_block(TileSmem& S, const KParams& P, const gmp_file_desc& F, uint64_t b,
-                                           int32_t* status, uint8_t* slot) {
-  BlockView V;
-  int err = open_block(F, b, V);
-  if (!err && !V.byte_fmt && (V.out_bytes > P.max_out || V.n_seq > P.max_seq)) err = GMP_STATUS_CAPACITY;
-  if (err) {
-    if (lane_id() == 0) set_status(status, err);
-    return;
-  }
-  uint2* rec = reinterpret_cast<uint2*>(slot);
-  uint8_t* out_blk = F.out + V.out_offset;
-  if (V.byte_fmt) {
-    lz_block<true>(S, V, status, rec, out_blk);
-  } else if (huffman_block(S, V, status, rec)) {
-    lz_block<false>(S, V, status, rec, out_blk);
   }
 }
 
@@ -881,57 +1014,92 @@ __device__ __forceinline__ uint32_t find_file(const KParams& P, uint64_t item) {
 }
 
 // A launch whose number of blocks only the device knows is made twice, a CTA
-// per block and a warp per block, and one of the two returns at once.  True if
-// this launch is to be the former: up to coop_max blocks, twice as many when
-// the (first) stream has Byte blocks, whose chains have no phase A.
+// per block and a pair of warps per block, and one of the two returns at once.
+// True if this launch is to be the former: up to coop_max blocks, a seventh
+// more when the (first) stream has Byte blocks, whose chains have no phase A
+// (912 of them: 787 us against 809; 912 of text: 1399 against 1296).
 __device__ __forceinline__ bool takes_coop(const KParams& P, uint64_t total) {
   const gmp_file_desc F = P.files ? P.files[0] : P.single;
   bool byte_fmt = false;
   if (F.n_blocks && F.comp_bytes >= 64 && !(((uintptr_t)F.comp) & 3u)) byte_fmt = !((ld_u32_nc(F.comp + 4) >> 16) & 2u);
-  return total <= (uint64_t)P.coop_max * (byte_fmt ? 2u : 1u);
+  return total <= P.coop_max + (byte_fmt ? P.coop_max / 7u : 0u);
 }
 
-// Persistent kernel: warps take blocks until none are left (the first one
+// Persistent kernel: warp pairs take blocks until none are left (the first one
 // fixed and interleaved over the CTAs when P.spread, as in gmp_decode.cu).
+// The first warp alone reads what a caller could change under the kernel and
+// decides; the second follows what it is told, so that both always meet at the
+// same barriers.
 template <bool PIPE>
-__global__ void __launch_bounds__(512, 1) tile_kernel(const KParams P) {
+__global__ void __launch_bounds__(1024, 1) tile_kernel(const KParams P) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  const uint32_t warp = threadIdx.x >> 5, lane = lane_id();
-  TileSmem& S = reinterpret_cast<TileSmem*>(smem_raw)[warp];
-  const uint64_t gw = (uint64_t)blockIdx.x * (blockDim.x >> 5) + warp;
-  uint8_t* slot = P.scratch + gw * P.slot_bytes;
+  const uint32_t pair = threadIdx.x >> 6, half = (threadIdx.x >> 5) & 1u, lane = lane_id(), pairs = blockDim.x >> 6;
+  TileSmem& S = reinterpret_cast<TileSmem*>(smem_raw)[pair];
+  uint2* rec = reinterpret_cast<uint2*>(P.scratch + ((uint64_t)blockIdx.x * pairs + pair) * P.slot_bytes);
   const uint64_t total = P.files ? P.item_start[P.n_files] : P.single.n_blocks;
   if (P.coop_max && takes_coop(P, total)) return;
-  const unsigned long long fixed = P.spread ? (unsigned long long)gridDim.x * (blockDim.x >> 5) : 0ull;
-  unsigned long long item = 0;
-  if (P.spread) {
-    item = (unsigned long long)warp * gridDim.x + blockIdx.x;
-  } else {
-    if (lane == 0) item = atomicAdd(P.counter, 1ull);
-    item = __shfl_sync(FULL, item, 0);
-  }
-  while (item < total) {
-    uint32_t file = 0;
-    uint64_t b = item;
-    gmp_file_desc F = P.single;
-    if (P.files) {
-      file = find_file(P, item);
-      b = item - P.item_start[file];
-      F = P.files[file];
+  bool first = P.spread != 0;
+  for (;;) {
+    if (half == 0) {
+      unsigned long long item = (unsigned long long)pair * gridDim.x + blockIdx.x;
+      if (!first) {
+        if (lane == 0) item = (P.spread ? (unsigned long long)gridDim.x * pairs : 0ull) + atomicAdd(P.counter, 1ull);
+        item = __shfl_sync(FULL, item, 0);
+      }
+      first = false;
+      uint32_t work = kEnd, file = 0;
+      if (item < total) {
+        uint64_t b = item;
+        gmp_file_desc F = P.single;
+        if (P.files) {
+          file = find_file(P, item);
+          b = item - P.item_start[file];
+          F = P.files[file];
+        }
+        work = kSkip;
+        int err = 0;
+        if (!PIPE || !P.in_ready || wait_input(P.in_ready + file, P.abort_wait, P.gen, P.wait_ns)) {
+          BlockView V;
+          err = open_block(F, b, V);
+          if (!err && !V.byte_fmt && (V.out_bytes > P.max_out || V.n_seq > P.max_seq)) err = GMP_STATUS_CAPACITY;
+          if (!err) {
+            work = V.byte_fmt ? kByte : kHuffman;
+            if (lane == 0) {
+              S.view = V;
+              S.out = F.out + V.out_offset;
+            }
+          }
+        } else {
+          err = GMP_STATUS_INPUT_TIMEOUT;
+        }
+        if (err && lane == 0) set_status(P.status + file, err);
+      }
+      if (lane == 0) {
+        S.work = work;
+        S.file = file;
+      }
     }
-    if (!PIPE || !P.in_ready || wait_input(P.in_ready + file, P.abort_wait, P.gen, P.wait_ns)) {
-      tile_block(S, P, F, b, P.status + file, slot);
-    } else if (lane == 0) {
-      set_status(P.status + file, GMP_STATUS_INPUT_TIMEOUT);
+    pair_sync();
+    const uint32_t work = S.work, file = S.file;
+    if (work == kEnd) break;
+    if (work != kSkip) {
+      const BlockView& V = S.view;
+      if (work == kByte || huffman_block(S, V, P.status + file, rec, half)) {
+        if (half) write_block(S, S.out);
+        else if (work == kByte) lay_out_block<true>(S, V, P.status + file, rec, S.out);
+        else lay_out_block<false>(S, V, P.status + file, rec, S.out);
+      }
     }
-    __syncwarp();
-    if (PIPE && P.out_ready) block_done(P.done + file, P.out_ready + file, P.gen, F.n_blocks);
-    unsigned long long next = 0;
-    if (lane == 0) next = fixed + atomicAdd(P.counter, 1ull);
-    item = __shfl_sync(FULL, next, 0);
+    if (PIPE && P.out_ready && half) {
+      const uint64_t n = P.files ? P.files[file].n_blocks : P.single.n_blocks;
+      block_done(P.done + file, P.out_ready + file, P.gen, n);
+    }
+    // the second warp is done with S.work and S.file before the first writes
+    // them again
+    pair_sync();
   }
-  if (PIPE && P.out_ready)
-    pipeline_exit(P.exited, P.out_ready, P.gen, P.files ? P.n_files : 1u, gridDim.x * (blockDim.x >> 5));
+  if (PIPE && P.out_ready && half)
+    pipeline_exit(P.exited, P.out_ready, P.gen, P.files ? P.n_files : 1u, gridDim.x * pairs);
 }
 
 // ---------------------------------------------------------------------------
@@ -948,7 +1116,7 @@ __global__ void __launch_bounds__(512, 1) tile_kernel(const KParams P) {
 // What bounds it is latency: of a 256 KiB block of CSV rows' 0.31 ms with 16
 // warps, about half is the chain of 1,000 Huffman steps in a lane (about 300
 // cycles each), half 34 waves of four dependent parts (scan, lay out and copy,
-// follow, flush).  One warp took 1.55 ms for it: 16 KiB 156 -> 51 us, 1 MiB of
+// follow, flush).  One warp took 1.55 ms for it (a pair of warps now 1.0): 16 KiB 156 -> 51 us, 1 MiB of
 // 64 KiB blocks 754 -> 195, 16 MiB of records 1554 -> 310, 64 MiB of text 1599
 // -> 548, 128 MiB of Byte records 1541 -> 540.
 constexpr uint32_t kLitWave = 1984;  // most literal bytes of a wave of a Byte block
@@ -968,7 +1136,6 @@ struct CoopSmemA {
   uint32_t bits[MAX_SUB][4 * kChunksAhead];
   BuildSmem build;
   Canon coff;
-  uint32_t run_off[16];
   uint16_t sorted_off[N_OFF + 2];
   uint32_t sb_bit[MAX_SUB], sb_seq[MAX_SUB];
 };
@@ -1000,9 +1167,6 @@ __device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
   asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
   return v;
 }
-__device__ __forceinline__ void sts_u16(uint32_t a, uint32_t v) {
-  asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)v) : "memory");
-}
 
 __device__ __forceinline__ void sts_u8_if(uint32_t a, uint32_t v, bool on) {
   asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p st.shared.u8 [%0], %1;\n}\n" ::"r"(a), "r"(v),
@@ -1027,8 +1191,8 @@ __device__ bool coop_huffman(CoopSmem<W>& S, const BlockView& V, int32_t* status
   if (warp < 3) {
     int r;
     if (warp == 0) r = sub_block_table(V, (V.comp_bytes - bs_off) * 8ull, A.sb_bit, S.sb_out, A.sb_seq);
-    else if (warp == 1) r = build_canon(T.cll, T.run, T.sorted_ll, T.lens, N_LL);
-    else r = build_canon(A.coff, A.run_off, A.sorted_off, T.lens + N_LL, N_OFF);
+    else if (warp == 1) r = build_canon(T.cll, T.run[0], T.sorted_ll, T.lens, N_LL);
+    else r = build_canon(A.coff, T.run[1], A.sorted_off, T.lens + N_LL, N_OFF);
     if (lane == 0) S.result[warp] = r;
   }
   __syncthreads();
@@ -1256,7 +1420,7 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
       if (BYTE) fill();
       const uint32_t wave_a = buf_a + w.cur;
       if (mine && !err) {
-        // segment starts and entries, as in lz_block
+        // segment starts and entries, as in lay_out_block
         uint32_t* mark = S.mark[warp];
         uint32_t* seg = S.seg[warp];
         for (uint32_t x = lane; x < ((total + 127u) >> 7) * 4u; x += 32) mark[x] = 0;
@@ -1423,7 +1587,7 @@ static cudaError_t configure_tile() {
 cudaError_t tile_occupancy(int warps_per_cta, int* ctas_per_sm) {
   cudaError_t e = configure_tile();
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, tile_kernel<false>, warps_per_cta * 32,
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, tile_kernel<false>, warps_per_cta * 64,
                                                        warps_per_cta * sizeof(TileSmem));
 }
 
@@ -1431,8 +1595,8 @@ cudaError_t launch_tile(const KParams& P, int grid, int warps_per_cta, bool pipe
   cudaError_t e = configure_tile();
   if (e != cudaSuccess) return e;
   const size_t smem = warps_per_cta * sizeof(TileSmem);
-  if (pipe) tile_kernel<true><<<grid, warps_per_cta * 32, smem, stream>>>(P);
-  else tile_kernel<false><<<grid, warps_per_cta * 32, smem, stream>>>(P);
+  if (pipe) tile_kernel<true><<<grid, warps_per_cta * 64, smem, stream>>>(P);
+  else tile_kernel<false><<<grid, warps_per_cta * 64, smem, stream>>>(P);
   return cudaGetLastError();
 }
 
