@@ -539,7 +539,9 @@ int gmp_compress_gpu(int device, const void* host_in, size_t n, const gmp_compre
     uint32_t* d_count = nullptr;
     unsigned long long* d_counter = nullptr;
     gmp::EncBlockPlan* d_plan = nullptr;
+    gmp::EncShare* d_share = nullptr;
     uint64_t* d_bytes = nullptr;
+    const uint32_t n_share = (uint32_t)std::min<uint64_t>(gmp::kEncShares, stride);
     if (check(cudaMalloc(&D.p[0], n + 16), "cudaMalloc") && check(cudaMalloc(&D.p[1], n), "cudaMalloc") &&
         check(cudaMalloc(&D.p[2], 2 * n), "cudaMalloc") &&
         check(cudaMalloc(&D.p[3], nb * stride * sizeof(gmp::ParseToken)), "cudaMalloc") &&
@@ -547,7 +549,8 @@ int gmp_compress_gpu(int device, const void* host_in, size_t n, const gmp_compre
         check(cudaMalloc(&D.p[5], nb * sizeof(uint32_t)), "cudaMalloc") &&
         check(cudaMalloc(&D.p[6], 2 * sizeof(unsigned long long)), "cudaMalloc") &&
         check(cudaMalloc(&D.p[7], nb * sizeof(gmp::EncBlockPlan)), "cudaMalloc") &&
-        check(cudaMalloc(&D.p[8], nb * sizeof(uint64_t)), "cudaMalloc")) {
+        check(cudaMalloc(&D.p[8], nb * sizeof(uint64_t)), "cudaMalloc") &&
+        check(cudaMalloc(&D.p[11], nb * n_share * sizeof(gmp::EncShare)), "cudaMalloc")) {
       d_in = static_cast<uint8_t*>(D.p[0]);
       d_len = static_cast<uint8_t*>(D.p[1]);
       d_dist = static_cast<uint16_t*>(D.p[2]);
@@ -557,6 +560,7 @@ int gmp_compress_gpu(int device, const void* host_in, size_t n, const gmp_compre
       d_counter = static_cast<unsigned long long*>(D.p[6]);
       d_plan = static_cast<gmp::EncBlockPlan*>(D.p[7]);
       d_bytes = static_cast<uint64_t*>(D.p[8]);
+      d_share = static_cast<gmp::EncShare*>(D.p[11]);
     }
     int* d_error = reinterpret_cast<int*>(d_counter + 1);
     if (rc == GMP_OK) {
@@ -595,7 +599,8 @@ int gmp_compress_gpu(int device, const void* host_in, size_t n, const gmp_compre
     // entropy coding on the GPU: plan every block (sizes), lay the blocks out
     // on the host, write them
     gmp::EncLaunch L{d_in, n, o.block_size, o.byte_mode ? 0u : o.n_sub, o.cwl, o.window, o.max_match,
-                     o.byte_mode ? 1 : 0, nb, d_tok, d_tpos, stride, d_count, d_plan, d_bytes, d_error,
+                     o.byte_mode ? 1 : 0, nb, d_tok, d_tpos, stride, d_count, d_plan, d_share, n_share, d_bytes,
+                     d_error,
                      (unsigned)std::min<uint64_t>(nb, (uint64_t)std::max(sms, 1) * 8), nullptr};
     if (rc == GMP_OK) {
       check(cudaEventRecord(ev[2]), "cudaEventRecord");

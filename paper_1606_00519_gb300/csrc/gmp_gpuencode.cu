@@ -23,11 +23,16 @@
 //     costs and, per sub-block, a search for the token where the running
 //     cost reaches (j + 1) / K of the total;
 //   - the bits of every sub-block, hence the block's encoded size, and of
-//     every share: the block's tokens in kEncThreads runs of equal work, each
+//     every share: the block's tokens in up to kEncThreads runs of equal work, each
 //     with its bit offset, since sub-blocks follow each other without gaps.
 //  Counting every byte and taking off those under back-references, and one
 //  thread per sub-block in write_kernel, took 4.0 ms for 64 MiB of text (256
 //  blocks of 32 sub-blocks); with literals counted and a thread per share 1.2.
+//  What bounds both kernels is a thread's chain of dependent reads (token,
+//  position, literals, their codes), so a CTA has as many threads as it can:
+//  1024 shares instead of 256 and prefix sums by all warps instead of one
+//  thread 1.22 -> 0.70 ms (512: 0.80; 1024 with one CTA on an SM instead of
+//  two: 0.89), 1 MiB of text 0.74 -> 0.42.
 //  write_kernel, one CTA per block at the offset the host computed from the
 //   sizes: the block header (code lengths, sub-block table), canonical codes
 //   (Sec. 3.1) from the lengths, then thread j packs share j's codes
@@ -63,8 +68,9 @@ struct TreeWS {
 
 struct PlanSmem {
   uint32_t h1[kNLL + 1], h2[kNOff + 2];
-  unsigned long long csum[kEncThreads];  // token cost per thread chunk, then its exclusive prefix
-  uint32_t lsum[kEncThreads];            // literal bytes per thread chunk, then prefix
+  unsigned long long csum[kEncThreads];  // exclusive prefix of the token cost per thread chunk
+  unsigned long long warp_cost[32];      // of cta_scan
+  uint32_t warp_sum[2][32];
   uint32_t g[kMaxSub], qs[kMaxSub + 1], so[kMaxSub + 1];
   unsigned long long sbits[kMaxSub];
   uint8_t lens[kNLL + kNOff + 1];
@@ -181,6 +187,30 @@ __device__ __forceinline__ uint32_t last_le(const T* a, uint32_t n, T x) {
   return lo;
 }
 
+// Exclusive prefix sum of v over the CTA's threads and their total (a barrier
+// inside; `sums` of an earlier call may not be in use any more).
+template <class T>
+__device__ __forceinline__ T cta_scan(T v, T* sums, T& total) {
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  T inc = v;
+#pragma unroll
+  for (uint32_t d = 1; d < 32; d <<= 1) {
+    const T y = __shfl_up_sync(0xffffffffu, inc, d);
+    if (lane >= d) inc += y;
+  }
+  if (lane == 31) sums[warp] = inc;
+  __syncthreads();
+  T all = lane < kEncThreads / 32 ? sums[lane] : (T)0;
+#pragma unroll
+  for (uint32_t d = 1; d < 32; d <<= 1) {
+    const T y = __shfl_up_sync(0xffffffffu, all, d);
+    if (lane >= d) all += y;
+  }
+  total = __shfl_sync(0xffffffffu, all, 31);
+  const T before = __shfl_sync(0xffffffffu, all, (warp + 31u) & 31u);
+  return (warp ? before : (T)0) + inc - v;
+}
+
 struct EncParams {
   const uint8_t* in;
   uint64_t n;
@@ -192,6 +222,8 @@ struct EncParams {
   uint64_t stride;
   const uint32_t* count;
   EncBlockPlan* plan;
+  EncShare* share;
+  uint32_t n_share;
   uint64_t* block_bytes;
   int* error;
 };
@@ -256,10 +288,11 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
         }
       }
     }
-    S.csum[tid] = cost;
-    S.lsum[tid] = lits;
     if (bad) atomicOr(&S.err, 1u);
-    __syncthreads();
+    unsigned long long all_cost;
+    uint32_t all_lits;
+    S.csum[tid] = cta_scan(cost, S.warp_cost, all_cost);
+    cta_scan(lits, S.warp_sum[0], all_lits);
     // (tokens that fail their checks may not lie in the block)
     if (!S.err) {
       for (uint32_t i = warp; i < S.n_long; i += kEncThreads / 32) {
@@ -267,20 +300,11 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
         for (uint32_t x = tid & 31u; x < ll; x += 32) atomicAdd(&S.h1[blk[p + x]], 1u);
       }
     }
+    __syncthreads();
     if (tid == 0) {
-      unsigned long long rc = 0;
-      uint32_t rl = 0;
-      for (int c = 0; c < kEncThreads; c++) {
-        const unsigned long long v = S.csum[c];
-        const uint32_t l = S.lsum[c];
-        S.csum[c] = rc;
-        S.lsum[c] = rl;
-        rc += v;
-        rl += l;
-      }
-      S.total_cost = rc;
-      S.n_lit = rl;
-      if (rc != (unsigned long long)nn + S.n_lit) S.err = 1;
+      S.total_cost = all_cost;
+      S.n_lit = all_lits;
+      if (all_cost != (unsigned long long)nn + all_lits) S.err = 1;
     }
     __syncthreads();
     EncBlockPlan& P = E.plan[b];
@@ -331,9 +355,9 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
       S.g[tid] = T > 0 ? g : 0xffffffffu;  // T = 0: the sub-block is empty
     }
     {
-      // shares, likewise: the first token whose running cost passes tid / 256
-      // of the total
-      const unsigned long long T = S.total_cost * tid / kEncThreads;
+      // shares, likewise: the first token whose running cost passes tid /
+      // n_share of the total
+      const unsigned long long T = S.total_cost * min(tid, E.n_share) / E.n_share;
       const uint32_t c = last_le<unsigned long long>(S.csum, kEncThreads, T);
       unsigned long long run = S.csum[c];
       uint32_t k = min(c * C, nn);
@@ -403,14 +427,10 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
       P.sub_bits[tid] = S.sbits[tid];
     }
     for (uint32_t i = tid; i < kNLL + kNOff; i += kEncThreads) P.lens[i] = S.lens[i];
-    P.share_first[tid] = S.share[tid];
+    uint32_t all_bits;
+    const uint32_t at_bit = cta_scan(S.share_bits[tid], S.warp_sum[1], all_bits);
+    if (tid < E.n_share) E.share[b * E.n_share + tid] = EncShare{S.share[tid], at_bit};
     if (tid == 0) {
-      P.share_first[kEncThreads] = nn;
-      uint32_t at = 0;
-      for (int c = 0; c < kEncThreads; c++) {
-        P.share_bit[c] = at;
-        at += S.share_bits[c];
-      }
       unsigned long long bits = 0;
       for (uint32_t j = 0; j < K; j++) bits += S.sbits[j];
       P.sub_first[K] = nn;
@@ -433,7 +453,7 @@ __device__ __forceinline__ void put_le32(uint8_t* p, uint32_t v) { *reinterpret_
 __global__ void __launch_bounds__(kEncThreads) write_kernel(const EncParams E, const uint64_t* offsets, uint8_t* out) {
   __shared__ uint16_t rc[kNLL + kNOff];  // canonical codes, bit-reversed for LSB-first output
   __shared__ uint8_t lens[kNLL + kNOff];
-  __shared__ uint32_t lsum[kEncThreads];
+  __shared__ uint32_t warp_sum[32];
   const uint32_t tid = threadIdx.x;
   for (uint64_t b = blockIdx.x; b < E.n_blocks; b += gridDim.x) {
     const EncBlockPlan& P = E.plan[b];
@@ -456,22 +476,15 @@ __global__ void __launch_bounds__(kEncThreads) write_kernel(const EncParams E, c
       const uint32_t k0 = min(tid * C, n), k1 = min(k0 + C, n);
       uint32_t l = 0;
       for (uint32_t k = k0; k < k1; k++) l += t[k].lit_len;
-      lsum[tid] = l;
-      __syncthreads();
+      uint32_t all;
+      uint32_t lo = cta_scan(l, warp_sum, all);
       if (tid == 0) {
-        uint32_t r = 0;
-        for (int c = 0; c < kEncThreads; c++) {
-          const uint32_t v = lsum[c];
-          lsum[c] = r;
-          r += v;
-        }
         put_le32(dst, n);
         put_le32(dst + 4, P.out_bytes);
         put_le32(dst + 8, P.n_lit);
       }
       __syncthreads();
       const uint64_t lit_sec = (16ull + 4ull * n + 15) & ~15ull;
-      uint32_t lo = lsum[tid];
       for (uint32_t k = k0; k < k1; k++) {
         const uint32_t ll = t[k].lit_len, ml = t[k].match & 0xffu, d = t[k].match >> 8;
         put_le32(dst + 16 + 4ull * k, ll | (ml ? ((ml - 2) << 10) | ((d - 1) << 16) : 0u));
@@ -516,10 +529,11 @@ __global__ void __launch_bounds__(kEncThreads) write_kernel(const EncParams E, c
       }
     }
     __syncthreads();
-    const uint32_t w0 = P.share_first[tid], w1 = P.share_first[tid + 1];
+    const EncShare* sh = E.share + b * E.n_share;
+    const uint32_t w0 = tid < E.n_share ? sh[tid].first : n, w1 = tid + 1 < E.n_share ? sh[tid + 1].first : n;
     if (w0 < w1) {
       // the share's bits, from its bit offset in the block's bitstream
-      const uint32_t start = P.share_bit[tid];
+      const uint32_t start = sh[tid].bit;
       uint32_t* W = reinterpret_cast<uint32_t*>(dst + hdr);
       uint32_t w = start >> 5;
       unsigned long long acc = 0;
@@ -564,14 +578,14 @@ __global__ void __launch_bounds__(kEncThreads) write_kernel(const EncParams E, c
 
 cudaError_t launch_encode_plan(const EncLaunch& L) {
   EncParams E{L.in, L.n, L.block_size, L.n_sub, L.cwl, L.window, L.max_match, L.byte_mode, L.n_blocks, L.tok,
-              L.tpos, L.stride, L.count, L.plan, L.block_bytes, L.error};
+              L.tpos, L.stride, L.count, L.plan, L.share, L.n_share, L.block_bytes, L.error};
   plan_kernel<<<L.grid, kEncThreads, 0, L.stream>>>(E);
   return cudaGetLastError();
 }
 
 cudaError_t launch_encode_write(const EncLaunch& L, const uint64_t* offsets, uint8_t* out) {
   EncParams E{L.in, L.n, L.block_size, L.n_sub, L.cwl, L.window, L.max_match, L.byte_mode, L.n_blocks, L.tok,
-              L.tpos, L.stride, L.count, L.plan, L.block_bytes, L.error};
+              L.tpos, L.stride, L.count, L.plan, L.share, L.n_share, L.block_bytes, L.error};
   write_kernel<<<L.grid, kEncThreads, 0, L.stream>>>(E, offsets, out);
   return cudaGetLastError();
 }

@@ -80,16 +80,18 @@ struct ParseToken {
 // GPU entropy coding of GPU parses (gmp_gpuencode.cu): per block, a plan
 // (token checks, code lengths, sub-block split and sizes), then the block's
 // bytes at an offset computed from the planned sizes.
-constexpr uint32_t kEncShares = 256;
+// Writing threads per block: its tokens in this many runs of about equal work,
+// or in fewer where a block has not as many tokens.
+constexpr uint32_t kEncShares = 1024;
+struct EncShare {
+  uint32_t first, bit;  // first token, its first bit
+};
 struct EncBlockPlan {
   uint64_t bytes, bits;  // encoded size (a multiple of 16), bitstream bits
   uint32_t n_seq, out_bytes, n_lit, err;
   uint32_t sub_first[kMaxSub + 1];  // first token of each sub-block; [K] = n_seq
   uint32_t sub_out[kMaxSub];        // output bytes of each sub-block
   uint64_t sub_bits[kMaxSub];       // bits of each sub-block
-  // the tokens in kEncShares runs of about equal work, a writing thread each:
-  // first token, first bit
-  uint32_t share_first[kEncShares + 1], share_bit[kEncShares];
   uint8_t lens[kLitLenSyms + kOffsetSyms];
 };
 struct EncLaunch {
@@ -103,6 +105,8 @@ struct EncLaunch {
   uint64_t stride;
   const uint32_t* count;  // tokens per block
   EncBlockPlan* plan;
+  EncShare* share;        // n_share per block
+  uint32_t n_share;       // at most kEncShares
   uint64_t* block_bytes;  // encoded size per block
   int* error;             // set to 1 if a token fails its checks
   unsigned grid;
