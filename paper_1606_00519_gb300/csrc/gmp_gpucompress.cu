@@ -486,8 +486,19 @@ __global__ void __launch_bounds__(kParseThreads) parse_kernel(const uint8_t* bes
 // Device times of the calling thread's last gmp_compress_gpu.
 thread_local gmp_gpu_compress_times g_times = {0, 0, 0, 0};
 
+// A call's device memory: one allocation for everything whose size is known
+// from the input's, and one for the stream's blocks when they do not fit where
+// the matches were.  Eleven buffers allocated and freed one by one took 0.5 ms
+// more: 64 MiB of text 8.30 -> 7.79 ms, 16 MiB of records (Byte) 4.81 -> 4.35,
+// 1 MiB of text 2.44 -> 2.17.
 struct DeviceBuffers {
-  void* p[12] = {};
+  void* p[2] = {};
+  uint64_t bytes = 0;
+  uint64_t place(uint64_t n) {  // its offset in the first allocation
+    const uint64_t at = bytes;
+    bytes += (n + 255u) & ~(uint64_t)255u;
+    return at;
+  }
   ~DeviceBuffers() {
     for (void* q : p)
       if (q) cudaFree(q);
@@ -542,25 +553,25 @@ int gmp_compress_gpu(int device, const void* host_in, size_t n, const gmp_compre
     gmp::EncShare* d_share = nullptr;
     uint64_t* d_bytes = nullptr;
     const uint32_t n_share = (uint32_t)std::min<uint64_t>(gmp::kEncShares, stride);
-    if (check(cudaMalloc(&D.p[0], n + 16), "cudaMalloc") && check(cudaMalloc(&D.p[1], n), "cudaMalloc") &&
-        check(cudaMalloc(&D.p[2], 2 * n), "cudaMalloc") &&
-        check(cudaMalloc(&D.p[3], nb * stride * sizeof(gmp::ParseToken)), "cudaMalloc") &&
-        check(cudaMalloc(&D.p[4], nb * stride * sizeof(uint32_t)), "cudaMalloc") &&
-        check(cudaMalloc(&D.p[5], nb * sizeof(uint32_t)), "cudaMalloc") &&
-        check(cudaMalloc(&D.p[6], 2 * sizeof(unsigned long long)), "cudaMalloc") &&
-        check(cudaMalloc(&D.p[7], nb * sizeof(gmp::EncBlockPlan)), "cudaMalloc") &&
-        check(cudaMalloc(&D.p[8], nb * sizeof(uint64_t)), "cudaMalloc") &&
-        check(cudaMalloc(&D.p[11], nb * n_share * sizeof(gmp::EncShare)), "cudaMalloc")) {
-      d_in = static_cast<uint8_t*>(D.p[0]);
-      d_len = static_cast<uint8_t*>(D.p[1]);
-      d_dist = static_cast<uint16_t*>(D.p[2]);
-      d_tok = static_cast<gmp::ParseToken*>(D.p[3]);
-      d_tpos = static_cast<uint32_t*>(D.p[4]);
-      d_count = static_cast<uint32_t*>(D.p[5]);
-      d_counter = static_cast<unsigned long long*>(D.p[6]);
-      d_plan = static_cast<gmp::EncBlockPlan*>(D.p[7]);
-      d_bytes = static_cast<uint64_t*>(D.p[8]);
-      d_share = static_cast<gmp::EncShare*>(D.p[11]);
+    uint64_t* d_off = nullptr;
+    const uint64_t at_in = D.place(n + 16), at_len = D.place(n), at_dist = D.place(2 * n), matches_end = D.bytes;
+    const uint64_t at_tok = D.place(nb * stride * sizeof(gmp::ParseToken)), at_tpos = D.place(nb * stride * sizeof(uint32_t));
+    const uint64_t at_count = D.place(nb * sizeof(uint32_t)), at_counter = D.place(2 * sizeof(unsigned long long));
+    const uint64_t at_plan = D.place(nb * sizeof(gmp::EncBlockPlan)), at_bytes = D.place(nb * sizeof(uint64_t));
+    const uint64_t at_share = D.place(nb * n_share * sizeof(gmp::EncShare)), at_off = D.place(nb * sizeof(uint64_t));
+    if (check(cudaMalloc(&D.p[0], D.bytes), "cudaMalloc")) {
+      uint8_t* m = static_cast<uint8_t*>(D.p[0]);
+      d_in = m + at_in;
+      d_len = m + at_len;
+      d_dist = reinterpret_cast<uint16_t*>(m + at_dist);
+      d_tok = reinterpret_cast<gmp::ParseToken*>(m + at_tok);
+      d_tpos = reinterpret_cast<uint32_t*>(m + at_tpos);
+      d_count = reinterpret_cast<uint32_t*>(m + at_count);
+      d_counter = reinterpret_cast<unsigned long long*>(m + at_counter);
+      d_plan = reinterpret_cast<gmp::EncBlockPlan*>(m + at_plan);
+      d_bytes = reinterpret_cast<uint64_t*>(m + at_bytes);
+      d_share = reinterpret_cast<gmp::EncShare*>(m + at_share);
+      d_off = reinterpret_cast<uint64_t*>(m + at_off);
     }
     int* d_error = reinterpret_cast<int*>(d_counter + 1);
     if (rc == GMP_OK) {
@@ -618,15 +629,17 @@ int gmp_compress_gpu(int device, const void* host_in, size_t n, const gmp_compre
       if (total > cap) rc = GMP_ERR_CAPACITY;
     }
     const uint64_t body = total - first - 16;  // the blocks, back to back
-    if (rc == GMP_OK && check(cudaMalloc(&D.p[9], std::max<uint64_t>(body, 16)), "cudaMalloc") &&
-        check(cudaMalloc(&D.p[10], nb * sizeof(uint64_t)), "cudaMalloc")) {
-      uint64_t* d_off = static_cast<uint64_t*>(D.p[10]);
+    // where the matches were, which the parse was the last to read
+    uint8_t* d_body = d_len;
+    if (rc == GMP_OK && body > matches_end - at_len && check(cudaMalloc(&D.p[1], body), "cudaMalloc"))
+      d_body = static_cast<uint8_t*>(D.p[1]);
+    if (rc == GMP_OK) {
       for (uint64_t b = 0; b < nb; b++) offsets[b] -= first;
       check(cudaMemcpy(d_off, offsets.data(), nb * sizeof(uint64_t), cudaMemcpyHostToDevice), "cudaMemcpy");
-      if (rc == GMP_OK) check(gmp::launch_encode_write(L, d_off, static_cast<uint8_t*>(D.p[9])), "write_kernel");
+      if (rc == GMP_OK) check(gmp::launch_encode_write(L, d_off, d_body), "write_kernel");
       if (rc == GMP_OK) check(cudaEventRecord(ev[3]), "cudaEventRecord");
       uint8_t* out = static_cast<uint8_t*>(host_out);
-      if (rc == GMP_OK) check(cudaMemcpy(out + first, D.p[9], body, cudaMemcpyDeviceToHost), "cudaMemcpy");
+      if (rc == GMP_OK) check(cudaMemcpy(out + first, d_body, body, cudaMemcpyDeviceToHost), "cudaMemcpy");
       if (rc == GMP_OK) {
         for (uint64_t b = 0; b < nb; b++) offsets[b] += first;
         gmp::write_stream_header(o, n, nb, offsets.data(), total, out);
