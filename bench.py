@@ -408,7 +408,7 @@ def measure_decode(args, w, data, streams, dev, dist=None, rank=0, clocks=False,
         "roofline": {"bound": "hbm", "achieved": round(achieved, 2), "peak": hbm_peak, "unit": "GB/s",
                      "frac": round(achieved / hbm_peak, 4), "peak_kind": peak_kind,
                      "traffic": (round(tpu * out_bytes) if tpu else None),
-                     "kernel": "gmp::decode_kernel (persistent; one launch per step)",
+                     "kernel": "gmp::tile_kernel (persistent; one launch per step)",
                      "algorithmic_bytes_per_launch": int(algo_bytes),
                      "launch_avg_ms": round(launch_avg_ms, 4),
                      "launch_median_ms": round(float(np.median(per_launch)), 4),
