@@ -185,6 +185,15 @@ __device__ __forceinline__ void cp_async16_if(uint32_t smem, const void* gmem, u
                "l"(gmem), "r"(n), "r"((uint32_t)on)
                : "memory");
 }
+// A segment that starts at output byte `at` of its group: its bit in the words
+// at `mark` and its entry; `on` only.
+__device__ __forceinline__ void segment_if(uint32_t mark, uint32_t at, uint32_t entry_a, uint32_t entry, bool on) {
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n@p red.shared.or.b32 [%0], %1;\n@p st.shared.u32 [%2], %3;\n}\n" ::"r"(
+          mark + ((at >> 3) & ~3u)),
+      "r"(1u << (at & 31u)), "r"(entry_a), "r"(entry), "r"((uint32_t)on)
+      : "memory");
+}
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
@@ -833,36 +842,36 @@ __device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, 
     uint32_t* mark = S.mark[stage];
     for (uint32_t x = lane; x < ((G.total + 127u) >> 7) * 4u; x += 32) mark[x] = 0;
     __syncwarp();
-    uint32_t* seg = S.seg[stage];
-    const uint32_t lit_a = smem_addr(S.lit[stage]);
+    // (predicated: with branches, of which every lane takes its own mix, 2 x 512
+    // MiB of records 2.90 ms against 2.86, files of 256 MiB 1.30 against 1.27)
+    const uint32_t lit_a = smem_addr(S.lit[stage]), mark_a = smem_addr(mark), far_a = smem_addr(S.far[stage]);
+    uint32_t seg_a = smem_addr(S.seg[stage]) + 4u * segs;
 #pragma unroll
     for (int k = 0; k < 2; k++) {
-      if (ll[k]) {
-        atomicOr(mark + (dst >> 5), 1u << (dst & 31u));
-        seg[segs++] = lit_a + lit_at - dst;
-      }
+      const bool has_l = ll[k] != 0, has_m = ml[k] != 0;
+      segment_if(mark_a, dst, seg_a, lit_a + lit_at - dst, has_l);
+      seg_a += has_l ? 4u : 0u;
       dst += ll[k];
       lit_at += BYTE ? ll[k] : 4u;
-      if (ml[k]) {
-        const uint32_t src = w.g0 + dst - dist[k];
-        const bool is_far = src < base;
-        uint8_t* place = S.far[stage] + 16u * chunks;
-        atomicOr(mark + (dst >> 5), 1u << (dst & 31u));
-        seg[segs++] = is_far ? smem_addr(place) + (src & 15u) - dst : buf_a + cur - dist[k];
-        if (is_far) {
-          // sources older than the window
-          if (vec_ok) {
-            const uint8_t* g = out_blk + (src & ~15u);
-            const uint32_t nc = ((src & 15u) + ml[k] + 15u) >> 4;
-            cp_async16(place, g);
-            if (nc > 1) cp_async16(place + 16, g + 16);
-            for (uint32_t c = 2; c < nc; c++) cp_async16(place + 16u * c, g + 16u * c);
-          } else {
-            for (uint32_t i = 0; i < ml[k]; i++) place[(src & 15u) + i] = (uint8_t)__ldcg(out_blk + src + i);
-          }
+      const uint32_t src = w.g0 + dst - dist[k], place = far_a + 16u * chunks;
+      const bool is_far = has_m && src < base;
+      segment_if(mark_a, dst, seg_a, is_far ? place + (src & 15u) - dst : buf_a + cur - dist[k], has_m);
+      seg_a += has_m ? 4u : 0u;
+      // sources older than the window
+      if (vec_ok) {
+        const uint8_t* g = out_blk + (src & ~15u);
+        const uint32_t nc = is_far ? ((src & 15u) + ml[k] + 15u) >> 4 : 0u;
+        cp_async16_if(place, g, 16, nc > 0);
+        cp_async16_if(place + 16, g + 16, 16, nc > 1);
+        if (__any_sync(FULL, nc > 2)) {
+          cp_async16_if(place + 32, g + 32, 16, nc > 2);
+          cp_async16_if(place + 48, g + 48, 16, nc > 3);
+          cp_async16_if(place + 64, g + 64, 16, nc > 4);
         }
-        chunks += dist[k] > near ? (ml[k] + 30u) >> 4 : 0u;
+      } else if (is_far) {
+        for (uint32_t i = 0; i < ml[k]; i++) sts_u8(place + (src & 15u) + i, __ldcg(out_blk + src + i));
       }
+      chunks += has_m && dist[k] > near ? (ml[k] + 30u) >> 4 : 0u;
       dst += ml[k];
     }
     return G;
