@@ -34,10 +34,12 @@
 // instructions with every SM full (2.4 warp instructions per byte of text,
 // 61 % of the issue slots), and a block's chain of dependent ones on small
 // launches.  The Huffman step without branches, records of 8 bytes with their
-// literals inside and stored four at a time (single 8-byte stores cost 0.5 of
-// 3.5 ms on 2 x 512 MiB of records), and tiles in place of per-sequence copies
-// with resolution rounds: 2 x 512 MiB of records, MRR and DE in one launch,
-// 4.53 -> 3.48 ms; 2 x 256 MiB of text 2.66 -> 2.15 (before: gmp_decode.cu).
+// literals inside and stored two at a time (single 8-byte stores cost 0.5 of
+// 3.5 ms on 2 x 512 MiB of records; four at a time, whose register moves cost
+// more than they save, 2 x 256 MiB of text 1.72 ms against 1.70), and tiles in
+// place of per-sequence copies with resolution rounds: 2 x 512 MiB of records,
+// MRR and DE in one launch, 4.53 -> 3.48 ms; 2 x 256 MiB of text 2.66 -> 2.15
+// (before: gmp_decode.cu).
 // A second warp for the writing, which doubles the warps on an SM in the same
 // shared memory (16 blocks), and groups of 64 records instead of 32, whose
 // layout and hand-over cost little more than one of 32: records 3.37 -> 2.90,
@@ -165,8 +167,8 @@ __device__ __forceinline__ void pair_sync() {
 
 // First record of sub-block j, whose output starts at `out`: a record covers
 // at least 3 bytes of output but for a sub-block's last one, and a corrupt
-// stream may write two more; a multiple of 4, so that four records are
-// 32-byte aligned.
+// stream may write two more; a multiple of 4, which keeps pairs of
+// records 16-byte aligned.
 __device__ __forceinline__ uint32_t rec_start(uint32_t out, uint32_t j) { return (out / 3 + 7 * j + 3) & ~3u; }
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -321,13 +323,10 @@ __device__ __forceinline__ void st_global_if(uint2* p, const uint2& v, bool on) 
                "r"(v.x), "r"(v.y), "r"((uint32_t)on)
                : "memory");
 }
-__device__ __forceinline__ void st_global_32B_if(uint2* p, const uint2& a, const uint2& b, const uint2& c,
-                                                 const uint2& d, bool on) {
-  asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.u32 p, %9, 0;\n@p st.global.v8.u32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n}\n" ::"l"(
-          p),
-      "r"(a.x), "r"(a.y), "r"(b.x), "r"(b.y), "r"(c.x), "r"(c.y), "r"(d.x), "r"(d.y), "r"((uint32_t)on)
-      : "memory");
+__device__ __forceinline__ void st_global_16B_if(uint2* p, const uint2& a, const uint2& b, bool on) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %5, 0;\n@p st.global.v4.u32 [%0], {%1, %2, %3, %4};\n}\n" ::"l"(p),
+               "r"(a.x), "r"(a.y), "r"(b.x), "r"(b.y), "r"((uint32_t)on)
+               : "memory");
 }
 __device__ __forceinline__ int byte1_signed(uint32_t v) {
   int r;
@@ -344,7 +343,7 @@ __device__ __forceinline__ uint32_t shr_clamp(uint32_t v, uint32_t n) {
   asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
   return r;
 }
-template <int LLB, int OFB, bool QUAD>
+template <int LLB, int OFB, bool PAIR>
 __device__ __forceinline__ uint32_t huffman_lane(const uint32_t* ll_lut, const uint32_t* off_lut, const Canon& coff,
                                                  const uint16_t* sorted_off, const uint32_t* ring, const uint8_t* bs,
                                                  uint32_t n_chunks, bool act, bool empty, const SubBlock& sb,
@@ -385,7 +384,7 @@ __device__ __forceinline__ uint32_t huffman_lane(const uint32_t* ll_lut, const u
     pos = np;
   };
   uint32_t lits = 0, ln8 = 0, cnt = 0;
-  uint2 q0 = make_uint2(0, 0), q1 = q0, q2 = q0, q3 = q0;  // QUAD: the last four records
+  uint2 q2 = make_uint2(0, 0), q3 = q2;  // PAIR: the last two records
   // the entry of a peek
   auto ll_of = [&](uint32_t pk) -> uint32_t {
     uint32_t e = ll_lut[pk & ((1u << LLB) - 1u)];
@@ -422,13 +421,11 @@ __device__ __forceinline__ uint32_t huffman_lane(const uint32_t* ll_lut, const u
     odd = odd || mc < 0 || dist > min(window, wpos);
     const bool emit = mc != 0 || ln8 >= 24u;
     const uint2 r = make_uint2(lits, dist | (ml << 16) | (ln8 << 21));
-    if (QUAD) {
-      q0 = emit ? q1 : q0;
-      q1 = emit ? q2 : q1;
+    if (PAIR) {
       q2 = emit ? q3 : q2;
       q3 = emit ? r : q3;
       cnt += emit ? 1u : 0u;
-      st_global_32B_if(rec + (cnt - 4u), q0, q1, q2, q3, emit && (cnt & 3u) == 0);
+      st_global_16B_if(rec + (cnt - 2u), q2, q3, emit && (cnt & 1u) == 0);
     } else {
       st_global_if(rec + cnt, r, emit);
       cnt += emit ? 1u : 0u;
@@ -487,11 +484,8 @@ __device__ __forceinline__ uint32_t huffman_lane(const uint32_t* ll_lut, const u
     cp_async_wait<2>();
   }
   cp_async_wait<0>();
-  if (QUAD && cnt <= rec_cap) {
-    const uint32_t n = cnt & 3u;  // records not stored yet
-    if (n > 2) rec[cnt - 3u] = q1;
-    if (n > 1) rec[cnt - 2u] = q2;
-    if (n > 0) rec[cnt - 1u] = q3;
+  if (PAIR && cnt <= rec_cap) {
+    if (cnt & 1u) rec[cnt - 1u] = q3;  // not stored yet
   }
   outp += ln8 >> 3;
   if (!err && pos != end) err = GMP_STATUS_BITSTREAM;
