@@ -1296,7 +1296,8 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
   Recs r = load();
 
   // Byte literals: a ring of kLitRing bytes filled at each wave's start for
-  // the waves after it
+  // the waves after it.  Each fill is a commit group of its own: the waits
+  // before the barriers below cover committed copies only.
   uint32_t litpos = 0, lit_asked = 0;
   auto fill = [&]() {
     const uint32_t upto = min((V.n_lit + 15u) & ~15u, (litpos & ~15u) + kLitRing);
@@ -1305,6 +1306,7 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
       cp_async16(S.blit + at, lits + c);
       if (at < kLitOver) cp_async16(S.blit + kLitRing + at, lits + c);
     }
+    cp_async_commit();
     lit_asked = max(lit_asked, upto);
   };
   if (t == 0) SS.bad = ~0u;

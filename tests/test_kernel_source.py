@@ -1,0 +1,36 @@
+"""CPU checks of the decode kernels' source, for rules that a run cannot show to
+hold: a broken one is a race that is usually won by time."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1606_00519_gb300", "csrc")
+
+
+def source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//.*", "", f.read())
+
+
+def functions(text):
+    """{name: body} of the definitions that start at the left margin."""
+    found = {}
+    for m in re.finditer(r"^(?:static |template <[^\n]*>\n)*[^\s#}/][^;{}]*?(\w+)\([^;{}]*\)\s*\{\n(.*?)^\}", text, re.M | re.S):
+        found[m.group(1)] = m.group(2)
+    return found
+
+
+@pytest.mark.parametrize("name", ["gmp_tile.cu", "gmp_decode.cu"])
+def test_waits_cover_the_copies(name):
+    # cp.async.wait_group waits for committed copies only: code that copies and
+    # waits by groups also commits what it copied
+    users = 0
+    for fn, body in functions(source(name)).items():
+        if "cp_async_wait" not in body:
+            continue
+        users += 1
+        copies = [m.start() for m in re.finditer(r"\bcp_async16(?:_if)?\(", body)]
+        commits = [m.start() for m in re.finditer(r"\bcp_async_commit\(", body)]
+        assert copies and commits and commits[-1] > copies[-1], fn
+    assert users >= 1
