@@ -42,7 +42,7 @@ struct KParams {
   unsigned long long* stats;  // [groups, rounds, de_fallback, blocks, max_rounds, cycles x3]
   int collect_stats;
   int resolve;  // 0: by the stream's DE flag, 1: MRR always, 2: sequential copying (SC)
-  uint32_t coop_max;  // 0, or: of a pair of launches the one that the number of blocks calls for runs
+  const uint32_t* route;  // null, or: of a pair of launches the one it names (a Route) runs
   int spread;   // 1: first items fixed and interleaved over the CTAs; 0: all from the counter
   // Host-to-host pipeline (all null otherwise): a file's input is complete
   // once in_ready[file] reaches gen (written by the copy stream after the

@@ -95,7 +95,8 @@ struct gmp_context {
   uint64_t slot_bytes = 0, shadow_off = 0;
   uint8_t* scratch = nullptr;
   size_t scratch_bytes = 0;
-  unsigned long long* counter = nullptr;  // 64 words: [0] work counter, [48, 56) pipeline partitions' counters
+  unsigned long long* counter = nullptr;  // 64 words: [0] work counter, [8] route, [48, 56) pipeline partitions' counters
+  uint32_t* route() const { return reinterpret_cast<uint32_t*>(counter + 8); }
   unsigned long long* stats = nullptr;    // counter + 16: 32 statistics words (gmp_stats_read)
   uint64_t* item_start = nullptr;         // batch prefix, max_files + 1
   // staging of gmp_decompress_host
@@ -297,7 +298,7 @@ static gmp::LaunchShape tile_shape(const gmp_context* c, uint64_t n_blocks, int 
                         : !from_host                    ? 7 * g8 / 4
                         : to_host || byte_fmt == 1      ? 4 * g8
                                                         : 5 * g8 / 2;
-  const uint64_t most_byte = from_host ? most : most + most / 7;  // as takes_coop() in gmp_tile.cu
+  const uint64_t most_byte = from_host ? most : most + most / 7;  // as route_of() in gmp_decode.cu
   if (n_blocks && n_blocks <= g16) {
     s.coop = 16;
     s.grid = (int)n_blocks;
@@ -306,6 +307,7 @@ static gmp::LaunchShape tile_shape(const gmp_context* c, uint64_t n_blocks, int 
     s.grid = (int)std::min(n_blocks, g8);
   } else if (!n_blocks || (byte_fmt < 0 && n_blocks <= most_byte)) {
     s.coop_max = (uint32_t)most;
+    s.route = c->route();
     s.coop_grid = (int)(n_blocks ? std::min(n_blocks, g8) : g8);
   }
   return s;
@@ -412,6 +414,7 @@ int gmp_decompress(gmp_context* c, const uint8_t* d_comp, size_t comp_bytes, con
     if ((uint64_t)shape.grid > wide_ctas) shape.grid = (int)wide_ctas;
   }
   if ((uint64_t)shape.grid > n_blocks) shape.grid = (int)n_blocks;
+  if (shape.coop_max) GMP_CUDA(gmp::launch_route(F, shape.coop_max, c->route(), s));
   GMP_CUDA(gmp::launch_decode(shape, nullptr, nullptr, 0, &F, d_status, c->counter, c->scratch, c->slot_bytes,
                               c->shadow_off, c->max_seq, c->max_out, c->stats, (int)c->opts.collect_stats,
                               (int)c->opts.resolve, s, c->opts.concurrent ? 0 : 1));
@@ -427,8 +430,9 @@ int gmp_decompress_batch(gmp_context* c, const gmp_file_desc* d_files, size_t n_
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   GMP_CUDA(cudaMemsetAsync(d_status, 0, n_files * sizeof(int32_t), s));
   GMP_CUDA(cudaMemsetAsync(c->counter, 0, sizeof(unsigned long long), s));
-  GMP_CUDA(gmp::launch_batch_prefix(d_files, (uint32_t)n_files, c->item_start, s));
-  GMP_CUDA(gmp::launch_decode(tile_shape(c, 0, -1), d_files, c->item_start, (uint32_t)n_files, nullptr, d_status, c->counter,
+  const gmp::LaunchShape shape = tile_shape(c, 0, -1);
+  GMP_CUDA(gmp::launch_batch_prefix(d_files, (uint32_t)n_files, c->item_start, shape.coop_max, c->route(), s));
+  GMP_CUDA(gmp::launch_decode(shape, d_files, c->item_start, (uint32_t)n_files, nullptr, d_status, c->counter,
                               c->scratch, c->slot_bytes, c->shadow_off, c->max_seq, c->max_out, c->stats,
                               (int)c->opts.collect_stats, (int)c->opts.resolve, s, c->opts.concurrent ? 0 : 1));
   return GMP_OK;

@@ -20,7 +20,10 @@ struct LaunchShape {
   int coop;           // with tile: 0, or the warps (8, 16) of a CTA that decodes a block together (grid CTAs)
   uint32_t coop_max;  // with coop = 0: 0, or launch coop_grid CTAs of 8 warps too, which take up to this many blocks
   int coop_grid;
+  const uint32_t* route;  // with coop_max: the device word that launch_route or launch_batch_prefix sets
 };
+// Which of a pair of launches runs: a CTA per block, or a pair of warps.
+enum Route : uint32_t { kRoutePair, kRouteCoop };
 
 // warps per SM that the 128-register kernel holds
 constexpr int kWideWarpsPerSm = 16;
@@ -59,8 +62,11 @@ cudaError_t launch_decode(const LaunchShape& shape, const gmp_file_desc* files, 
                           int resolve, cudaStream_t stream, int spread = 1, const PipeFlags* pipe = nullptr);
 // compiled architecture of decode_kernel (cudaFuncGetAttributes)
 cudaError_t kernel_arch(int* binary_version, int* ptx_version);
-cudaError_t launch_batch_prefix(const gmp_file_desc* files, uint32_t n_files, uint64_t* item_start,
-                                cudaStream_t stream);
+// The work-item prefix of a batch; with coop_max the route of its launches too.
+cudaError_t launch_batch_prefix(const gmp_file_desc* files, uint32_t n_files, uint64_t* item_start, uint32_t coop_max,
+                                uint32_t* route, cudaStream_t stream);
+// The route of one stream's launches.
+cudaError_t launch_route(const gmp_file_desc& file, uint32_t coop_max, uint32_t* route, cudaStream_t stream);
 
 // Stream-format constants (format version 1).
 constexpr uint32_t kHeaderBytes = 64;

@@ -138,6 +138,7 @@ int gmp_decompress_noalloc(const uint8_t* d_comp, size_t comp_bytes, const gmp_b
   shape.coop = 16;  // a CTA of 16 warps per block and slot
   shape.coop_max = 0;
   shape.coop_grid = 0;
+  shape.route = nullptr;
   shape.grid = (int)(n_blocks < kSlots ? n_blocks : kSlots);
   gmp_file_desc F{d_comp, comp_bytes, d_index, n_blocks, d_out, out_cap};
   unsigned long long* counter = reinterpret_cast<unsigned long long*>(scratch);

@@ -131,9 +131,16 @@ struct Window {
   uint32_t base;     // output position of buf[0] (a multiple of 16): g0 - cur
   uint32_t flushed;  // output bytes stored (a multiple of kFlush)
 };
-// What the first warp of a pair hands to the second: the block, and in phase B
-// group after group.
+// What one warp reads of the caller's descriptors, index and block header and
+// hands to the others that decode the block with it.
 enum Work : uint32_t { kEnd, kSkip, kByte, kHuffman };
+struct Job {
+  BlockView view;
+  uint8_t* out;
+  uint32_t work, file;
+};
+// What the first warp of a pair hands to the second in phase B, group after
+// group.
 enum Step : uint32_t { kGroup, kSlow, kDone, kAbandon };
 struct StepMsg {
   uint32_t what, total, shift;  // kGroup: its bytes, and what the window slides by before it
@@ -145,9 +152,7 @@ struct __align__(64) TileSmem {
   } u;
   uint32_t sb_out[MAX_SUB];  // sub-block output start
   uint32_t sb_cnt[MAX_SUB];  // its records
-  BlockView view;
-  uint8_t* out;
-  uint32_t work, file;
+  Job job;
   int32_t result[3];  // of the parts of the table build
   StepMsg step[2];
   Window win;                  // after a slow group
@@ -994,7 +999,7 @@ __device__ __forceinline__ void write_block(TileSmem& SS, uint8_t* out_blk) {
       w.cur += m.total;
       flush(S.buf, w, out_blk, vec_ok, lane, 32);
     } else if (m.what == kSlow) {
-      slow_group(S.buf, kBuf, kHist, w, SS.view.B + 16, SS.slow_t0, SS.slow_t1, SS.slow_lits, out_blk, vec_ok);
+      slow_group(S.buf, kBuf, kHist, w, SS.job.view.B + 16, SS.slow_t0, SS.slow_t1, SS.slow_lits, out_blk, vec_ok);
       if (lane == 0) SS.win = w;
       pair_sync();
       stage ^= 1u;
@@ -1016,23 +1021,52 @@ __device__ __forceinline__ uint32_t find_file(const KParams& P, uint64_t item) {
   return lo;
 }
 
-// A launch whose number of blocks only the device knows is made twice, a CTA
-// per block and a pair of warps per block, and one of the two returns at once.
-// True if this launch is to be the former: up to coop_max blocks, a seventh
-// more when the (first) stream has Byte blocks, whose chains have no phase A
-// (912 of them: 787 us against 809; 912 of text: 1399 against 1296).
-__device__ __forceinline__ bool takes_coop(const KParams& P, uint64_t total) {
-  const gmp_file_desc F = P.files ? P.files[0] : P.single;
-  bool byte_fmt = false;
-  if (F.n_blocks && F.comp_bytes >= 64 && !(((uintptr_t)F.comp) & 3u)) byte_fmt = !((ld_u32_nc(F.comp + 4) >> 16) & 2u);
-  return total <= P.coop_max + (byte_fmt ? P.coop_max / 7u : 0u);
+// One warp: work item `item` of `total`, opened and checked, into J.  The warps
+// that decode a block follow what it says and read none of this themselves: a
+// caller could change it under the kernel, and warps that saw different values
+// would miss each other at a barrier.
+template <bool PIPE>
+__device__ __forceinline__ void take_block(const KParams& P, uint64_t item, uint64_t total, Job& J) {
+  const uint32_t lane = lane_id();
+  uint32_t work = kEnd, file = 0;
+  if (item < total) {
+    uint64_t b = item;
+    gmp_file_desc F = P.single;
+    if (P.files) {
+      file = find_file(P, item);
+      b = item - P.item_start[file];
+      F = P.files[file];
+    }
+    work = kSkip;
+    int err = 0;
+    if (!PIPE || !P.in_ready || wait_input(P.in_ready + file, P.abort_wait, P.gen, P.wait_ns)) {
+      BlockView V;
+      err = open_block(F, b, V);
+      if (!err && !V.byte_fmt && (V.out_bytes > P.max_out || V.n_seq > P.max_seq)) err = GMP_STATUS_CAPACITY;
+      if (!err) {
+        work = V.byte_fmt ? kByte : kHuffman;
+        if (lane == 0) {
+          J.view = V;
+          J.out = F.out + V.out_offset;
+        }
+      }
+    } else {
+      err = GMP_STATUS_INPUT_TIMEOUT;
+    }
+    if (err && lane == 0) set_status(P.status + file, err);
+  }
+  if (lane == 0) {
+    J.work = work;
+    J.file = file;
+  }
 }
+
+// Of a pair of launches, a CTA per block and a pair of warps per block, the one
+// that the route does not name returns at once.
+__device__ __forceinline__ bool not_routed(const KParams& P, uint32_t mine) { return P.route && *P.route != mine; }
 
 // Persistent kernel: warp pairs take blocks until none are left (the first one
 // fixed and interleaved over the CTAs when P.spread, as in gmp_decode.cu).
-// The first warp alone reads what a caller could change under the kernel and
-// decides; the second follows what it is told, so that both always meet at the
-// same barriers.
 template <bool PIPE>
 __global__ void __launch_bounds__(1024, 1) tile_kernel(const KParams P) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -1040,7 +1074,7 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(const KParams P) {
   TileSmem& S = reinterpret_cast<TileSmem*>(smem_raw)[pair];
   uint2* rec = reinterpret_cast<uint2*>(P.scratch + ((uint64_t)blockIdx.x * pairs + pair) * P.slot_bytes);
   const uint64_t total = P.files ? P.item_start[P.n_files] : P.single.n_blocks;
-  if (P.coop_max && takes_coop(P, total)) return;
+  if (not_routed(P, kRoutePair)) return;
   bool first = P.spread != 0;
   for (;;) {
     if (half == 0) {
@@ -1050,55 +1084,24 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(const KParams P) {
         item = __shfl_sync(FULL, item, 0);
       }
       first = false;
-      uint32_t work = kEnd, file = 0;
-      if (item < total) {
-        uint64_t b = item;
-        gmp_file_desc F = P.single;
-        if (P.files) {
-          file = find_file(P, item);
-          b = item - P.item_start[file];
-          F = P.files[file];
-        }
-        work = kSkip;
-        int err = 0;
-        if (!PIPE || !P.in_ready || wait_input(P.in_ready + file, P.abort_wait, P.gen, P.wait_ns)) {
-          BlockView V;
-          err = open_block(F, b, V);
-          if (!err && !V.byte_fmt && (V.out_bytes > P.max_out || V.n_seq > P.max_seq)) err = GMP_STATUS_CAPACITY;
-          if (!err) {
-            work = V.byte_fmt ? kByte : kHuffman;
-            if (lane == 0) {
-              S.view = V;
-              S.out = F.out + V.out_offset;
-            }
-          }
-        } else {
-          err = GMP_STATUS_INPUT_TIMEOUT;
-        }
-        if (err && lane == 0) set_status(P.status + file, err);
-      }
-      if (lane == 0) {
-        S.work = work;
-        S.file = file;
-      }
+      take_block<PIPE>(P, item, total, S.job);
     }
     pair_sync();
-    const uint32_t work = S.work, file = S.file;
+    const uint32_t work = S.job.work, file = S.job.file;
     if (work == kEnd) break;
     if (work != kSkip) {
-      const BlockView& V = S.view;
+      const BlockView& V = S.job.view;
       if (work == kByte || huffman_block(S, V, P.status + file, rec, half)) {
-        if (half) write_block(S, S.out);
-        else if (work == kByte) lay_out_block<true>(S, V, P.status + file, rec, S.out);
-        else lay_out_block<false>(S, V, P.status + file, rec, S.out);
+        if (half) write_block(S, S.job.out);
+        else if (work == kByte) lay_out_block<true>(S, V, P.status + file, rec, S.job.out);
+        else lay_out_block<false>(S, V, P.status + file, rec, S.job.out);
       }
     }
     if (PIPE && P.out_ready && half) {
       const uint64_t n = P.files ? P.files[file].n_blocks : P.single.n_blocks;
       block_done(P.done + file, P.out_ready + file, P.gen, n);
     }
-    // the second warp is done with S.work and S.file before the first writes
-    // them again
+    // the second warp is done with S.job before the first writes it again
     pair_sync();
   }
   if (PIPE && P.out_ready && half)
@@ -1162,7 +1165,7 @@ struct __align__(64) CoopSmem {
   Window win;          // after a slow group
   int32_t result[3];   // of the parts of the table build
   uint32_t bad;        // Byte: lowest warp << 8 | status of a failed check, else ~0
-  unsigned long long item;
+  Job job;
 };
 
 __device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
@@ -1527,47 +1530,30 @@ __global__ void __launch_bounds__(32 * W, W == 16 ? 1 : 3) coop_kernel(const KPa
   const uint32_t t = threadIdx.x;
   uint2* rec = reinterpret_cast<uint2*>(P.scratch + blockIdx.x * P.slot_bytes);
   const uint64_t total = P.files ? P.item_start[P.n_files] : P.single.n_blocks;
-  if (P.coop_max && !takes_coop(P, total)) return;
-  unsigned long long item = blockIdx.x;
-  for (bool first = true;; first = false) {
-    if (!first || !P.spread) {
-      __syncthreads();
-      if (t == 0) S.item = (P.spread ? gridDim.x : 0u) + atomicAdd(P.counter, 1ull);
-      __syncthreads();
-      item = S.item;
-    }
-    if (item >= total) break;
-    uint32_t file = 0;
-    uint64_t b = item;
-    gmp_file_desc F = P.single;
-    if (P.files) {
-      file = find_file(P, item);
-      b = item - P.item_start[file];
-      F = P.files[file];
-    }
-    int32_t* status = P.status + file;
-    bool ok = true;
-    if (PIPE && P.in_ready) {
-      ok = wait_input(P.in_ready + file, P.abort_wait, P.gen, P.wait_ns);
-      ok = !__syncthreads_or(!ok);
-      if (!ok && t == 0) set_status(status, GMP_STATUS_INPUT_TIMEOUT);
-    }
-    if (ok) {
-      BlockView V;
-      int err = open_block(F, b, V);
-      if (!err && !V.byte_fmt && (V.out_bytes > P.max_out || V.n_seq > P.max_seq)) err = GMP_STATUS_CAPACITY;
-      if (err) {
-        if (t == 0) set_status(status, err);
-      } else if (V.byte_fmt) {
-        coop_lz<W, true>(S, V, status, rec, F.out + V.out_offset);
-      } else if (coop_huffman<W>(S, V, status, rec)) {
-        coop_lz<W, false>(S, V, status, rec, F.out + V.out_offset);
+  if (not_routed(P, kRouteCoop)) return;
+  for (bool first = P.spread != 0;; first = false) {
+    if (t < 32) {
+      unsigned long long item = blockIdx.x;
+      if (!first) {
+        if (t == 0) item = (P.spread ? gridDim.x : 0u) + atomicAdd(P.counter, 1ull);
+        item = __shfl_sync(FULL, item, 0);
       }
+      take_block<PIPE>(P, item, total, S.job);
     }
-    if (PIPE && P.out_ready) {
-      __threadfence();
-      __syncthreads();  // every thread's output is stored
-      if (t < 32) block_done(P.done + file, P.out_ready + file, P.gen, F.n_blocks);
+    __syncthreads();
+    const uint32_t work = S.job.work, file = S.job.file;
+    if (work == kEnd) break;
+    int32_t* status = P.status + file;
+    if (work != kSkip) {
+      const BlockView V = S.job.view;
+      if (work == kByte) coop_lz<W, true>(S, V, status, rec, S.job.out);
+      else if (coop_huffman<W>(S, V, status, rec)) coop_lz<W, false>(S, V, status, rec, S.job.out);
+    }
+    if (PIPE && P.out_ready) __threadfence();
+    __syncthreads();  // every thread's output is stored, and S.job free
+    if (PIPE && P.out_ready && t < 32) {
+      const uint64_t n = P.files ? P.files[file].n_blocks : P.single.n_blocks;
+      block_done(P.done + file, P.out_ready + file, P.gen, n);
     }
   }
   if (PIPE && P.out_ready) pipeline_exit(P.exited, P.out_ready, P.gen, P.files ? P.n_files : 1u, gridDim.x * W);

@@ -34,3 +34,20 @@ def test_waits_cover_the_copies(name):
         commits = [m.start() for m in re.finditer(r"\bcp_async_commit\(", body)]
         assert copies and commits and commits[-1] > copies[-1], fn
     assert users >= 1
+
+
+def test_one_warp_reads_what_a_caller_can_change():
+    # warps that share a block's barriers take the block's header, descriptor
+    # and index entry from the one warp that read them, and the choice between
+    # two launches is read from a device word, not worked out by each CTA
+    text = source("gmp_tile.cu")
+    text = re.sub(r"__launch_bounds__\([^)]*\)+ ", "", text)
+    found = functions(text)
+    kernels = {k: v for k, v in found.items() if k in ("coop_kernel", "tile_kernel")}
+    assert len(kernels) == 2 and [k for k, v in found.items() if "open_block(" in v] == ["take_block"]
+    for body in kernels.values():
+        assert not re.search(r"gmp_file_desc|find_file|wait_input|ld_u32_nc|->comp|\.comp\b", body)
+        assert len(re.findall(r"\btake_block<", body)) == 1
+        guard = body[:body.index("take_block<")]
+        assert re.search(r"if \((half == 0|t < 32)\) \{(?:[^{}]|\{[^{}]*\})*$", guard)
+    assert "takes_coop" not in text and "route_of" not in text
