@@ -104,7 +104,7 @@ struct TileSmemA {
   } u;
   Canon coff;
   uint16_t sorted_off[N_OFF + 2];
-  uint32_t sb_bit[MAX_SUB], sb_seq[MAX_SUB];
+  uint32_t sb_bit[MAX_SUB + 1], sb_seq[MAX_SUB];
 };
 
 // Phase B.  The output window `buf` holds at least the last kHist output
@@ -500,7 +500,9 @@ __device__ __forceinline__ uint32_t huffman_lane(const uint32_t* ll_lut, const u
 
 // Sub-block table: prefix sums of bit sizes, output sizes and sequences over
 // the K sub-blocks (one warp), with the totals checked in 64 bits, so that
-// no wrapped 32-bit sum passes.  Returns a gmp_status.
+// no wrapped 32-bit sum passes; sb_bit[K] is the last one's end.  The stream's
+// table is read here only: sub_block() has the sizes that were checked, whatever
+// a caller writes there meanwhile.  Returns a gmp_status.
 __device__ int sub_block_table(const BlockView& V, uint64_t bits_avail, uint32_t* sb_bit, uint32_t* sb_out,
                                uint32_t* sb_seq) {
   const uint32_t lane = lane_id();
@@ -534,8 +536,16 @@ __device__ int sub_block_table(const BlockView& V, uint64_t bits_avail, uint32_t
     to += __shfl_xor_sync(FULL, to, d);
     ts += __shfl_xor_sync(FULL, ts, d);
   }
+  if (lane == 0) sb_bit[V.K] = carry_bit;
   if (ts != V.n_seq || to != V.out_bytes) return GMP_STATUS_BAD_HEADER;
   return tb > bits_avail ? (int)GMP_STATUS_BITSTREAM : 0;
+}
+__device__ __forceinline__ SubBlock sub_block(const BlockView& V, const uint32_t* sb_bit, const uint32_t* sb_out,
+                                              const uint32_t* sb_seq, uint32_t j) {
+  if (j >= V.K) return SubBlock{0, 0, 0, 0, 0, 0};
+  const bool last = j + 1 == V.K;
+  return SubBlock{sb_bit[j], sb_bit[j + 1] - sb_bit[j], sb_out[j], (last ? V.out_bytes : sb_out[j + 1]) - sb_out[j],
+                  sb_seq[j], (last ? V.n_seq : sb_seq[j + 1]) - sb_seq[j]};
 }
 
 __device__ __forceinline__ void unpack_lens(uint8_t* lens, const uint8_t* B, uint32_t t, uint32_t n) {
@@ -581,11 +591,7 @@ __device__ __forceinline__ bool huffman_block(TileSmem& S, const BlockView& V, i
     const uint32_t n_chunks = (uint32_t)min((uint64_t)0xffffffffu, (V.comp_bytes - bs_off) / 16);
     for (uint32_t jb = 0; jb < V.K; jb += 32) {
       const uint32_t j = jb + lane;
-      SubBlock sb{0, 0, 0, 0, 0, 0};
-      if (j < V.K) {
-        const uint8_t* e = V.B + 192 + 12 * j;
-        sb = SubBlock{A.sb_bit[j], ld_u32_nc(e), S.sb_out[j], ld_u32_nc(e + 4), A.sb_seq[j], ld_u32_nc(e + 8)};
-      }
+      const SubBlock sb = sub_block(V, A.sb_bit, S.sb_out, A.sb_seq, j);
       const uint32_t cnt = huffman_lane<kLLBits, kOffBits, true>(
           A.ll, A.off, A.coff, A.sorted_off, A.u.bits[lane], bs, n_chunks, j < V.K, n_ll == 0, sb, V.n_seq, V.window,
           rec + rec_start(sb.out, j), err);
@@ -654,17 +660,20 @@ __device__ __forceinline__ void flush_rest(const uint8_t* buf, const Window& w, 
 
 // A Byte group that does not fit the fast path: record after record, one
 // warp copying each literal string and each match (window of `cap` bytes,
-// `hist` of them kept).
+// `hist` of them kept).  The records, which were checked as a group, are read
+// again here: every length is cut to what is left of the output and of the
+// literals (up to lits_end), so that a record changed meanwhile stays in them.
 __device__ __noinline__ void slow_group(uint8_t* buf, uint32_t cap, uint32_t hist, Window& w, const uint8_t* recs,
-                                        uint32_t t0, uint32_t t1, const uint8_t* lits, uint8_t* out_blk, bool vec_ok) {
+                                        uint32_t t0, uint32_t t1, const uint8_t* lits, const uint8_t* lits_end,
+                                        uint8_t* out_blk, uint32_t out_bytes, bool vec_ok) {
   const uint32_t lane = lane_id();
   auto room = [&](uint32_t n) {
     if (w.cur + n > cap) slide(buf, w, (w.cur - hist) & ~15u);
   };
   for (uint32_t t = t0; t < t1; t++) {
-    const uint32_t r = ld_u32_nc(recs + 4ull * t), m = (r >> 10) & 63u, dist = (r >> 16) + 1u;
-    uint32_t left = r & 1023u;
-    const uint32_t ml = m ? m + 2u : 0u;
+    const uint32_t r = __shfl_sync(FULL, ld_u32_nc(recs + 4ull * t), 0), m = (r >> 10) & 63u, dist = (r >> 16) + 1u;
+    uint32_t left = min(min(r & 1023u, out_bytes - w.g0), (uint32_t)min((uint64_t)1023u, (uint64_t)(lits_end - lits)));
+    const uint32_t ml = m && dist <= w.g0 + left ? min(m + 2u, out_bytes - w.g0 - left) : 0u;
     while (left) {
       const uint32_t n = min(left, kFlush);
       room(n);
@@ -999,7 +1008,8 @@ __device__ __forceinline__ void write_block(TileSmem& SS, uint8_t* out_blk) {
       w.cur += m.total;
       flush(S.buf, w, out_blk, vec_ok, lane, 32);
     } else if (m.what == kSlow) {
-      slow_group(S.buf, kBuf, kHist, w, SS.job.view.B + 16, SS.slow_t0, SS.slow_t1, SS.slow_lits, out_blk, vec_ok);
+      slow_group(S.buf, kBuf, kHist, w, SS.job.view.B + 16, SS.slow_t0, SS.slow_t1, SS.slow_lits,
+                 SS.job.view.B + SS.job.view.lit_off + SS.job.view.n_lit, out_blk, SS.job.view.out_bytes, vec_ok);
       if (lane == 0) SS.win = w;
       pair_sync();
       stage ^= 1u;
@@ -1143,7 +1153,7 @@ struct CoopSmemA {
   BuildSmem build;
   Canon coff;
   uint16_t sorted_off[N_OFF + 2];
-  uint32_t sb_bit[MAX_SUB], sb_seq[MAX_SUB];
+  uint32_t sb_bit[MAX_SUB + 1], sb_seq[MAX_SUB];
 };
 template <int W>
 struct CoopSmemB {
@@ -1218,11 +1228,7 @@ __device__ bool coop_huffman(CoopSmem<W>& S, const BlockView& V, int32_t* status
   // count (64 MiB of text, 8 warps: 0.92 ms with 8 of them, 0.60 with 4)
   constexpr uint32_t HW = W == 16 ? 8 : 4;
   const uint32_t j = warp < HW ? lane * HW + warp : MAX_SUB;
-  SubBlock sb{0, 0, 0, 0, 0, 0};
-  if (j < V.K) {
-    const uint8_t* e = V.B + 192 + 12 * j;
-    sb = SubBlock{A.sb_bit[j], ld_u32_nc(e), S.sb_out[j], ld_u32_nc(e + 4), A.sb_seq[j], ld_u32_nc(e + 8)};
-  }
+  const SubBlock sb = sub_block(V, A.sb_bit, S.sb_out, A.sb_seq, j);
   const uint32_t cnt = huffman_lane<LUT_BITS, LUT_BITS, false>(
       A.ll, A.off, A.coff, A.sorted_off, A.bits[min(j, (uint32_t)MAX_SUB - 1u)], bs, n_chunks, j < V.K, n_ll == 0,
       sb, V.n_seq, V.window, rec + rec_start(sb.out, j), err);
@@ -1414,7 +1420,8 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
         if (SS.bad != ~0u) break;
         if (warp == lo) {
           Window x = w;
-          slow_group(S.buf, CB, hist, x, recs, t_cur, min(t_cur + GR, V.n_seq), lits + litpos, out_blk, vec_ok);
+          slow_group(S.buf, CB, hist, x, recs, t_cur, min(t_cur + GR, V.n_seq), lits + litpos, lits + V.n_lit, out_blk,
+                     V.out_bytes, vec_ok);
           if (lane == 0) SS.win = x;
         }
         __syncthreads();

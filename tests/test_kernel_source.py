@@ -51,3 +51,12 @@ def test_one_warp_reads_what_a_caller_can_change():
         guard = body[:body.index("take_block<")]
         assert re.search(r"if \((half == 0|t < 32)\) \{(?:[^{}]|\{[^{}]*\})*$", guard)
     assert "takes_coop" not in text and "route_of" not in text
+
+
+def test_sizes_read_twice_are_bounded():
+    # the sub-block table is read once, where its totals are checked; records
+    # written one by one are read a second time, and cut to what is left
+    found = functions(source("gmp_tile.cu"))
+    assert [k for k, v in found.items() if re.search(r"192u? \+ 12u? \* j", v)] == ["sub_block_table"]
+    body = found["slow_group"]
+    assert "out_bytes - w.g0" in body and "lits_end - lits" in body and "dist <= w.g0" in body
