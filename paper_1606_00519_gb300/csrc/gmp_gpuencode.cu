@@ -70,7 +70,7 @@ struct PlanSmem {
   uint32_t h1[kNLL + 1], h2[kNOff + 2];
   unsigned long long csum[kEncThreads];  // exclusive prefix of the token cost per thread chunk
   unsigned long long warp_cost[32];      // of cta_scan
-  uint32_t warp_sum[2][32];
+  uint32_t warp_sum[32];
   uint32_t g[kMaxSub], qs[kMaxSub + 1], so[kMaxSub + 1];
   unsigned long long sbits[kMaxSub];
   uint8_t lens[kNLL + kNOff + 1];
@@ -78,7 +78,7 @@ struct PlanSmem {
   unsigned long long total_cost;
   uint32_t n_lit, err;
   uint32_t share[kEncThreads + 1];  // first token of each share
-  uint32_t share_bits[kEncThreads];
+  unsigned long long share_bits[kEncThreads];
   uint32_t longs[kMaxLong], n_long;
 };
 
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
     unsigned long long all_cost;
     uint32_t all_lits;
     S.csum[tid] = cta_scan(cost, S.warp_cost, all_cost);
-    cta_scan(lits, S.warp_sum[0], all_lits);
+    cta_scan(lits, S.warp_sum, all_lits);
     // (tokens that fail their checks may not lie in the block)
     if (!S.err) {
       for (uint32_t i = warp; i < S.n_long; i += kEncThreads / 32) {
@@ -386,11 +386,12 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
     // each, then each thread's share
     for (uint32_t i = warp; i < S.n_long; i += kEncThreads / 32) {
       const uint32_t k = S.longs[i], ll = t[k].lit_len, p = tp[k];
-      uint32_t bits = 0;
-      for (uint32_t x = tid & 31u; x < ll; x += 32) bits += S.lens[blk[p + x]];
-      bits = __reduce_add_sync(0xffffffffu, bits);
+      uint32_t mine = 0;
+      for (uint32_t x = tid & 31u; x < ll; x += 32) mine += S.lens[blk[p + x]];
+      unsigned long long bits = mine;
+      for (int d = 16; d >= 1; d >>= 1) bits += __shfl_xor_sync(0xffffffffu, bits, d);
       if ((tid & 31u) == 0) {
-        atomicAdd(&S.sbits[last_le<uint32_t>(S.qs, K, k)], (unsigned long long)bits);
+        atomicAdd(&S.sbits[last_le<uint32_t>(S.qs, K, k)], bits);
         atomicAdd(&S.share_bits[last_le<uint32_t>(S.share, kEncThreads, k)], bits);
       }
     }
@@ -418,7 +419,7 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
         }
       }
       atomicAdd(&S.sbits[j], (unsigned long long)acc);
-      atomicAdd(&S.share_bits[tid], all + acc);
+      atomicAdd(&S.share_bits[tid], (unsigned long long)all + acc);
     }
     __syncthreads();
     if (tid < K) {
@@ -427,9 +428,10 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
       P.sub_bits[tid] = S.sbits[tid];
     }
     for (uint32_t i = tid; i < kNLL + kNOff; i += kEncThreads) P.lens[i] = S.lens[i];
-    uint32_t all_bits;
-    const uint32_t at_bit = cta_scan(S.share_bits[tid], S.warp_sum[1], all_bits);
-    if (tid < E.n_share) E.share[b * E.n_share + tid] = EncShare{S.share[tid], at_bit};
+    unsigned long long all_bits;
+    const unsigned long long at_bit = cta_scan(S.share_bits[tid], S.warp_cost, all_bits);
+    if (tid < E.n_share)
+      E.share[b * E.n_share + tid] = EncShare{S.share[tid], (uint32_t)at_bit, (uint32_t)(at_bit >> 32)};
     if (tid == 0) {
       unsigned long long bits = 0;
       for (uint32_t j = 0; j < K; j++) bits += S.sbits[j];
@@ -533,11 +535,11 @@ __global__ void __launch_bounds__(kEncThreads) write_kernel(const EncParams E, c
     const uint32_t w0 = tid < E.n_share ? sh[tid].first : n, w1 = tid + 1 < E.n_share ? sh[tid + 1].first : n;
     if (w0 < w1) {
       // the share's bits, from its bit offset in the block's bitstream
-      const uint32_t start = sh[tid].bit;
+      const uint64_t start = sh[tid].bit_lo | ((uint64_t)sh[tid].bit_hi << 32);
       uint32_t* W = reinterpret_cast<uint32_t*>(dst + hdr);
-      uint32_t w = start >> 5;
+      uint32_t w = (uint32_t)(start >> 5);
       unsigned long long acc = 0;
-      uint32_t na = start & 31u;
+      uint32_t na = (uint32_t)start & 31u;
       bool first = true;
       auto put = [&](uint32_t bits, uint32_t nb) {
         acc |= (unsigned long long)bits << na;

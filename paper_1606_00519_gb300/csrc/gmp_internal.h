@@ -90,7 +90,7 @@ struct ParseToken {
 // or in fewer where a block has not as many tokens.
 constexpr uint32_t kEncShares = 1024;
 struct EncShare {
-  uint32_t first, bit;  // first token, its first bit
+  uint32_t first, bit_lo, bit_hi;  // first token, its first bit (a block may have 2^32 and more)
 };
 struct EncBlockPlan {
   uint64_t bytes, bits;  // encoded size (a multiple of 16), bitstream bits
