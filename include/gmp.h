@@ -258,7 +258,10 @@ void gmp_context_opts_default(gmp_context_opts* o);
    stream, as the serving loop's lanes do). */
 int gmp_context_create(gmp_context** ctx, int device, const gmp_context_opts* opts);
 void gmp_context_destroy(gmp_context* ctx);
-/* Change launch shape (an autotuner result); reallocates scratch if needed. */
+/* Change launch shape (an autotuner result); reallocates scratch if needed.
+   The shape is that of launches that give a pair of warps to each block; a
+   launch of few blocks gives each a CTA of 8 or 16 warps of its own, of which
+   the shape only bounds the number (a scratch slot each). */
 int gmp_context_set_launch(gmp_context* ctx, uint32_t warps_per_cta, uint32_t ctas_per_sm);
 /* Bytes of device scratch the context holds. */
 size_t gmp_context_scratch_bytes(const gmp_context* ctx);
@@ -320,13 +323,16 @@ void gmp_graph_destroy(gmp_graph* g);
 /* ------------------------------------------------------------------------ */
 /* Launch-shape autotuner: times the batched decode of a sample (device file
    descriptors, as for gmp_decompress_batch) under several shapes (warps per
-   CTA 1, 2, 4, 8, 16; CTAs per SM as many as fit and half of that), keeps
-   the fastest in the context and reports it.  Each shape is run once to
-   warm up and three times timed with CUDA events on `stream`; the context's
-   scratch is reallocated when a shape needs more.  Synchronous. */
+   CTA 1, 2, 4, 8, 16; CTAs per SM as many as fit and, for batches of more
+   blocks than run at once, half of that), keeps the fastest in the context and
+   reports it; the default shape (4 warps, as many CTAs as fit) unless another
+   is more than 2 % faster.  Each shape is run
+   once to warm up and three times timed with CUDA events on `stream`, with the
+   launches it governs (a pair of warps per block), however small the batch;
+   the context's scratch is reallocated when a shape needs more.  Synchronous. */
 typedef struct {
   uint32_t warps_per_cta, ctas_per_sm; /* the chosen shape */
-  double best_ms;                      /* its mean time per batched launch */
+  double best_ms;                      /* mean time of the batch's launch with it */
   uint32_t shapes_tried;
 } gmp_tuning;
 int gmp_autotune(gmp_context* ctx, const gmp_file_desc* d_files, size_t n_files, int32_t* d_status, void* stream,

@@ -91,6 +91,7 @@ struct gmp_context {
   gmp::LaunchShape shape{};
   int occ_wide = 0, occ_deep = 0;  // CTAs per SM of the two kernels at this shape's warps per CTA
   int coop_ctas[2] = {0, 0};       // resident CTAs of 16 and of 8 warps, a block each
+  bool pair_only = false;          // launches of the default kernels take a pair of warps per block (gmp_autotune)
   uint32_t max_seq = 0, max_out = 0;
   uint64_t slot_bytes = 0, shadow_off = 0;
   uint8_t* scratch = nullptr;
@@ -293,7 +294,7 @@ static gmp::LaunchShape tile_shape(const gmp_context* c, uint64_t n_blocks, int 
   gmp::LaunchShape s = c->shape;
   const uint64_t slots = (uint64_t)c->shape.grid * (uint64_t)c->shape.warps_per_cta;
   const uint64_t g16 = std::min<uint64_t>(c->coop_ctas[0], slots), g8 = std::min<uint64_t>(c->coop_ctas[1], slots);
-  if (!s.tile || !g16 || !g8) return s;
+  if (!s.tile || c->pair_only || !g16 || !g8) return s;
   const uint64_t most = c->opts.concurrent              ? g16
                         : !from_host                    ? 7 * g8 / 4
                         : to_host || byte_fmt == 1      ? 4 * g8
@@ -495,10 +496,37 @@ int gmp_autotune(gmp_context* c, const gmp_file_desc* d_files, size_t n_files, i
   GMP_CUDA(cudaEventCreate(&e0));
   GMP_CUDA(cudaEventCreate(&e1));
   const gmp_context_opts saved = c->opts;
-  double best = 1e300;
   uint32_t best_w = 0, best_c = 0, tried = 0;
   int rc = GMP_OK;
-  for (uint32_t w : {1u, 2u, 4u, 8u, 16u}) {
+  // the batch once to warm up, then three times: least and mean ms
+  auto time_batch = [&](double* least, double* mean) -> int {
+    *least = 1e300;
+    *mean = 0;
+    int r = gmp_decompress_batch(c, d_files, n_files, d_status, s);
+    for (int k = 0; k < 3 && r == GMP_OK; k++) {
+      float ms = 0;
+      cudaEventRecord(e0, s);
+      r = gmp_decompress_batch(c, d_files, n_files, d_status, s);
+      cudaEventRecord(e1, s);
+      if (r == GMP_OK && (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
+        r = cuda_fail(cudaGetLastError(), "gmp_autotune");
+      *least = std::min(*least, (double)ms);
+      *mean += ms / 3.0;
+    }
+    return r;
+  };
+  // A small batch is decoded by a CTA per block whatever the shape is; the
+  // shapes are compared by the launches they govern, a pair of warps per block,
+  // since the one that is kept governs the context's larger batches.  A batch
+  // whose blocks all run at once cannot tell a half-full SM from a full one
+  // (with 24 blocks of 64 KiB half-full shapes won now and then, by the time it
+  // takes to launch fewer CTAs), so that half-full shapes are for batches of more
+  // blocks; and the first shape, the default, stays unless another is faster by
+  // more than 2 %.
+  c->pair_only = true;
+  double best = 1e300, least, mean;
+  uint64_t n_blocks = 0;
+  for (uint32_t w : {4u, 1u, 2u, 8u, 16u}) {
     int occ_wide = 0, occ_deep = 0;
     if (c->shape.tile) {
       if (gmp::tile_occupancy((int)w, &occ_wide) != cudaSuccess) continue;
@@ -517,44 +545,46 @@ int gmp_autotune(gmp_context* c, const gmp_file_desc* d_files, size_t n_files, i
     const int cands[3] = {occ_deep > occ_wide ? occ_deep : 0, occ_wide, occ_wide / 2};
     for (int cps : cands) {
       if (cps < 1 || (cps == occ_wide / 2 && occ_wide / 2 == occ_wide)) continue;
+      const uint64_t slots = (uint64_t)std::max(occ_wide, occ_deep) * w * (uint64_t)c->sm_count;
+      if (cps == occ_wide / 2 && n_blocks <= slots) continue;
       c->opts.warps_per_cta = w;
       c->opts.ctas_per_sm = (uint32_t)cps;
       if ((rc = context_alloc_scratch(c)) != GMP_OK) break;
-      if ((rc = gmp_decompress_batch(c, d_files, n_files, d_status, s)) != GMP_OK) break;
-      cudaEventRecord(e0, s);
-      for (int r = 0; r < 3 && rc == GMP_OK; r++) rc = gmp_decompress_batch(c, d_files, n_files, d_status, s);
-      cudaEventRecord(e1, s);
-      if (rc) break;
-      if (cudaEventSynchronize(e1) != cudaSuccess) {
-        rc = cuda_fail(cudaGetLastError(), "gmp_autotune");
-        break;
+      if ((rc = time_batch(&least, &mean)) != GMP_OK) break;
+      if (!tried++) {
+        uint64_t total = 0;
+        const cudaError_t e = cudaMemcpyAsync(&total, c->item_start + n_files, sizeof(total), cudaMemcpyDeviceToHost, s);
+        if (e != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) {
+          rc = cuda_fail(e != cudaSuccess ? e : cudaGetLastError(), "gmp_autotune");
+          break;
+        }
+        n_blocks = total;
       }
-      float ms = 0;
-      cudaEventElapsedTime(&ms, e0, e1);
-      tried++;
-      if (ms / 3.0 < best) {
-        best = ms / 3.0;
+      if (least < 0.98 * best) {
+        best = least;
         best_w = w;
         best_c = (uint32_t)cps;
       }
     }
     if (rc) break;
   }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
+  c->pair_only = false;
   if (rc == GMP_OK && tried) {
     c->opts.warps_per_cta = best_w;
     c->opts.ctas_per_sm = best_c;
     rc = context_alloc_scratch(c);
+    if (rc == GMP_OK) rc = time_batch(&least, &mean);  // as the batch is launched from now on
     out->warps_per_cta = best_w;
     out->ctas_per_sm = best_c;
-    out->best_ms = best;
+    out->best_ms = mean;
     out->shapes_tried = tried;
   } else {
     c->opts = saved;
     int rc2 = context_alloc_scratch(c);
     if (rc == GMP_OK) rc = tried ? rc2 : GMP_ERR_CUDA;
   }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
   return rc;
 }
 
