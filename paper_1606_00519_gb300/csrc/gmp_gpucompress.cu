@@ -573,13 +573,25 @@ int gmp_compress_gpu(int device, const void* host_in, size_t n, const gmp_compre
     gmp::EncBlockPlan* d_plan = nullptr;
     gmp::EncShare* d_share = nullptr;
     uint64_t* d_bytes = nullptr;
-    const uint32_t n_share = (uint32_t)std::min<uint64_t>(gmp::kEncShares, stride);
+    gmp::EncLaunch L{};
+    L.n = n;
+    L.block_size = o.block_size;
+    L.n_sub = o.byte_mode ? 0u : o.n_sub;
+    L.cwl = o.cwl;
+    L.window = o.window;
+    L.max_match = o.max_match;
+    L.byte_mode = o.byte_mode ? 1 : 0;
+    L.n_blocks = nb;
+    L.stride = stride;
+    L.threads = gmp::encode_threads(L, (uint32_t)std::max(sms, 1));
+    L.n_share = (uint32_t)std::min<uint64_t>(L.threads, stride);
+    L.grid = (unsigned)std::min<uint64_t>(nb, (uint64_t)std::max(sms, 1) * 16);
     uint64_t* d_off = nullptr;
     const uint64_t at_in = D.place(n + 16), at_len = D.place(n), at_dist = D.place(2 * n), matches_end = D.bytes;
     const uint64_t at_tok = D.place(nb * stride * sizeof(gmp::ParseToken)), at_tpos = D.place(nb * stride * sizeof(uint32_t));
     const uint64_t at_count = D.place(nb * sizeof(uint32_t)), at_counter = D.place(2 * sizeof(unsigned long long));
     const uint64_t at_plan = D.place(nb * sizeof(gmp::EncBlockPlan)), at_bytes = D.place(nb * sizeof(uint64_t));
-    const uint64_t at_share = D.place(nb * n_share * sizeof(gmp::EncShare)), at_off = D.place(nb * sizeof(uint64_t));
+    const uint64_t at_share = D.place(nb * L.n_share * sizeof(gmp::EncShare)), at_off = D.place(nb * sizeof(uint64_t));
     if (check(cudaMalloc(&D.p[0], D.bytes), "cudaMalloc")) {
       uint8_t* m = static_cast<uint8_t*>(D.p[0]);
       d_in = m + at_in;
@@ -630,10 +642,14 @@ int gmp_compress_gpu(int device, const void* host_in, size_t n, const gmp_compre
     }
     // entropy coding on the GPU: plan every block (sizes), lay the blocks out
     // on the host, write them
-    gmp::EncLaunch L{d_in, n, o.block_size, o.byte_mode ? 0u : o.n_sub, o.cwl, o.window, o.max_match,
-                     o.byte_mode ? 1 : 0, nb, d_tok, d_tpos, stride, d_count, d_plan, d_share, n_share, d_bytes,
-                     d_error,
-                     (unsigned)std::min<uint64_t>(nb, (uint64_t)std::max(sms, 1) * 8), nullptr};
+    L.in = d_in;
+    L.tok = d_tok;
+    L.tpos = d_tpos;
+    L.count = d_count;
+    L.plan = d_plan;
+    L.share = d_share;
+    L.block_bytes = d_bytes;
+    L.error = d_error;
     if (rc == GMP_OK) {
       check(cudaEventRecord(ev[2]), "cudaEventRecord");
       check(gmp::launch_encode_plan(L), "plan_kernel");

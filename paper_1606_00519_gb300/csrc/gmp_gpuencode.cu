@@ -23,16 +23,23 @@
 //     costs and, per sub-block, a search for the token where the running
 //     cost reaches (j + 1) / K of the total;
 //   - the bits of every sub-block, hence the block's encoded size, and of
-//     every share: the block's tokens in up to kEncThreads runs of equal work, each
+//     every share: the block's tokens in up to a run per thread of equal work, each
 //     with its bit offset, since sub-blocks follow each other without gaps.
 //  Counting every byte and taking off those under back-references, and one
 //  thread per sub-block in write_kernel, took 4.0 ms for 64 MiB of text (256
 //  blocks of 32 sub-blocks); with literals counted and a thread per share 1.2.
 //  What bounds both kernels is a thread's chain of dependent reads (token,
-//  position, literals, their codes), so a CTA has as many threads as it can:
-//  1024 shares instead of 256 and prefix sums by all warps instead of one
-//  thread 1.22 -> 0.70 ms (512: 0.80; 1024 with one CTA on an SM instead of
-//  two: 0.89), 1 MiB of text 0.74 -> 0.42.
+//  position, literals, their codes) and one warp's chain that builds a tree,
+//  which takes as long for a block of 1 KiB.  So a block gets as many threads
+//  (NT, a CTA) as leave all blocks on the GPU at once, 1024 to 128: the planning
+//  kernel's 64 registers fit 1024 threads on an SM, the writing one's 32 twice
+//  as many.  Both, 1024 / 512 / 256 / 128 threads per block, ms: 64 MiB of text
+//  in 256 blocks 0.73 / 0.73 / 1.14 / 1.99 (256 threads and prefix sums by one
+//  of them 1.22); 16 MiB in 512 blocks 0.69 / 0.42 / 0.33 / 0.41, in 4096 3.72 /
+//  1.94 / 1.05 / 0.70, in 16384 12.4 / 6.3 / 3.2 / 1.8; 1 MiB in 4 blocks 0.41 /
+//  0.51 / 0.74 / 1.24.  Byte blocks, which have no trees, of more than 16 KiB
+//  always take 1024 (64 MiB of text in 1024 blocks 0.33, 128 threads 0.45; 16 MiB
+//  in 4096 blocks 0.33 and 0.14).
 //  write_kernel, one CTA per block at the offset the host computed from the
 //   sizes: the block header (code lengths, sub-block table), canonical codes
 //   (Sec. 3.1) from the lengths, then thread j packs share j's codes
@@ -49,7 +56,6 @@
 namespace gmp {
 namespace {
 
-constexpr int kEncThreads = kEncShares;
 constexpr uint32_t kMaxLong = 1024;  // literal strings of a block that are counted by a warp each
 constexpr int kMaxDepth = 64;
 constexpr uint32_t kNLL = kLitLenSyms, kNOff = kOffsetSyms;
@@ -66,9 +72,10 @@ struct TreeWS {
   uint32_t m;                          // used symbols
 };
 
+template <int NT>
 struct PlanSmem {
   uint32_t h1[kNLL + 1], h2[kNOff + 2];
-  unsigned long long csum[kEncThreads];  // exclusive prefix of the token cost per thread chunk
+  unsigned long long csum[NT];  // exclusive prefix of the token cost per thread chunk
   unsigned long long warp_cost[32];      // of cta_scan
   uint32_t warp_sum[32];
   uint32_t g[kMaxSub], qs[kMaxSub + 1], so[kMaxSub + 1];
@@ -77,8 +84,8 @@ struct PlanSmem {
   TreeWS ws[2];
   unsigned long long total_cost;
   uint32_t n_lit, err;
-  uint32_t share[kEncThreads + 1];  // first token of each share
-  unsigned long long share_bits[kEncThreads];
+  uint32_t share[NT + 1];  // first token of each share
+  unsigned long long share_bits[NT];
   uint32_t longs[kMaxLong], n_long;
 };
 
@@ -189,26 +196,26 @@ __device__ __forceinline__ uint32_t last_le(const T* a, uint32_t n, T x) {
 
 // Exclusive prefix sum of v over the CTA's threads and their total (a barrier
 // inside; `sums` of an earlier call may not be in use any more).
-template <class T>
-__device__ __forceinline__ T cta_scan(T v, T* sums, T& total) {
+template <int NT, class V>
+__device__ __forceinline__ V cta_scan(V v, V* sums, V& total) {
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  T inc = v;
+  V inc = v;
 #pragma unroll
   for (uint32_t d = 1; d < 32; d <<= 1) {
-    const T y = __shfl_up_sync(0xffffffffu, inc, d);
+    const V y = __shfl_up_sync(0xffffffffu, inc, d);
     if (lane >= d) inc += y;
   }
   if (lane == 31) sums[warp] = inc;
   __syncthreads();
-  T all = lane < kEncThreads / 32 ? sums[lane] : (T)0;
+  V all = lane < NT / 32 ? sums[lane] : (V)0;
 #pragma unroll
   for (uint32_t d = 1; d < 32; d <<= 1) {
-    const T y = __shfl_up_sync(0xffffffffu, all, d);
+    const V y = __shfl_up_sync(0xffffffffu, all, d);
     if (lane >= d) all += y;
   }
   total = __shfl_sync(0xffffffffu, all, 31);
-  const T before = __shfl_sync(0xffffffffu, all, (warp + 31u) & 31u);
-  return (warp ? before : (T)0) + inc - v;
+  const V before = __shfl_sync(0xffffffffu, all, (warp + 31u) & 31u);
+  return (warp ? before : (V)0) + inc - v;
 }
 
 struct EncParams {
@@ -228,8 +235,9 @@ struct EncParams {
   int* error;
 };
 
-__global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
-  __shared__ PlanSmem S;
+template <int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) plan_kernel(const EncParams E) {
+  __shared__ PlanSmem<NT> S;
   const uint32_t tid = threadIdx.x, warp = tid >> 5;
   for (uint64_t b = blockIdx.x; b < E.n_blocks; b += gridDim.x) {
     const uint64_t base = b * (uint64_t)E.block_size;
@@ -239,7 +247,7 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
     const ParseToken* t = E.tok + b * E.stride;
     const uint32_t* tp = E.tpos + b * E.stride;
     const uint32_t K = E.byte_mode ? 0u : E.n_sub;
-    for (uint32_t i = tid; i < kNLL + 1; i += kEncThreads) S.h1[i] = 0;
+    for (uint32_t i = tid; i < kNLL + 1; i += NT) S.h1[i] = 0;
     if (tid < kNOff + 2) S.h2[tid] = 0;
     if (tid == 0) {
       S.err = (n == 0 || n > E.stride) ? 1u : 0u;
@@ -248,7 +256,7 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
     S.share_bits[tid] = 0;
     __syncthreads();
     const uint32_t nn = min(n, (uint32_t)E.stride);
-    const uint32_t C = (nn + kEncThreads - 1) / kEncThreads;
+    const uint32_t C = (nn + NT - 1) / NT;
     const uint32_t k0 = min(tid * C, nn), k1 = min(k0 + C, nn);
     // literal strings from this length on are left to the warps (there are at
     // most kMaxLong of them)
@@ -291,11 +299,11 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
     if (bad) atomicOr(&S.err, 1u);
     unsigned long long all_cost;
     uint32_t all_lits;
-    S.csum[tid] = cta_scan(cost, S.warp_cost, all_cost);
-    cta_scan(lits, S.warp_sum, all_lits);
+    S.csum[tid] = cta_scan<NT>(cost, S.warp_cost, all_cost);
+    cta_scan<NT>(lits, S.warp_sum, all_lits);
     // (tokens that fail their checks may not lie in the block)
     if (!S.err) {
-      for (uint32_t i = warp; i < S.n_long; i += kEncThreads / 32) {
+      for (uint32_t i = warp; i < S.n_long; i += NT / 32) {
         const uint32_t k = S.longs[i], ll = t[k].lit_len, p = tp[k];
         for (uint32_t x = tid & 31u; x < ll; x += 32) atomicAdd(&S.h1[blk[p + x]], 1u);
       }
@@ -340,7 +348,7 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
       const unsigned long long T = S.total_cost * (tid + 1) / K;
       uint32_t g = 0;
       if (T > 0) {
-        const uint32_t c = last_le<unsigned long long>(S.csum, kEncThreads, T - 1);  // last chunk starting below T
+        const uint32_t c = last_le<unsigned long long>(S.csum, NT, T - 1);  // last chunk starting below T
         unsigned long long run = S.csum[c];
         const uint32_t c0 = min(c * C, nn), c1 = min(c0 + C, nn);
         g = c1;
@@ -358,12 +366,12 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
       // shares, likewise: the first token whose running cost passes tid /
       // n_share of the total
       const unsigned long long T = S.total_cost * min(tid, E.n_share) / E.n_share;
-      const uint32_t c = last_le<unsigned long long>(S.csum, kEncThreads, T);
+      const uint32_t c = last_le<unsigned long long>(S.csum, NT, T);
       unsigned long long run = S.csum[c];
       uint32_t k = min(c * C, nn);
       for (const uint32_t c1 = min(k + C, nn); k < c1 && run < T; k++) run += t[k].lit_len + 1ull;
       S.share[tid] = k;
-      if (tid == 0) S.share[kEncThreads] = nn;
+      if (tid == 0) S.share[NT] = nn;
     }
     __syncthreads();
     if (tid == 0) {
@@ -384,7 +392,7 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
     __syncthreads();
     // bits of each sub-block and each share: the long literal strings, a warp
     // each, then each thread's share
-    for (uint32_t i = warp; i < S.n_long; i += kEncThreads / 32) {
+    for (uint32_t i = warp; i < S.n_long; i += NT / 32) {
       const uint32_t k = S.longs[i], ll = t[k].lit_len, p = tp[k];
       uint32_t mine = 0;
       for (uint32_t x = tid & 31u; x < ll; x += 32) mine += S.lens[blk[p + x]];
@@ -392,7 +400,7 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
       for (int d = 16; d >= 1; d >>= 1) bits += __shfl_xor_sync(0xffffffffu, bits, d);
       if ((tid & 31u) == 0) {
         atomicAdd(&S.sbits[last_le<uint32_t>(S.qs, K, k)], bits);
-        atomicAdd(&S.share_bits[last_le<uint32_t>(S.share, kEncThreads, k)], bits);
+        atomicAdd(&S.share_bits[last_le<uint32_t>(S.share, NT, k)], bits);
       }
     }
     const uint32_t w0 = S.share[tid], w1 = S.share[tid + 1];
@@ -427,9 +435,9 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
       P.sub_out[tid] = S.so[tid + 1] - S.so[tid];
       P.sub_bits[tid] = S.sbits[tid];
     }
-    for (uint32_t i = tid; i < kNLL + kNOff; i += kEncThreads) P.lens[i] = S.lens[i];
+    for (uint32_t i = tid; i < kNLL + kNOff; i += NT) P.lens[i] = S.lens[i];
     unsigned long long all_bits;
-    const unsigned long long at_bit = cta_scan(S.share_bits[tid], S.warp_cost, all_bits);
+    const unsigned long long at_bit = cta_scan<NT>(S.share_bits[tid], S.warp_cost, all_bits);
     if (tid < E.n_share)
       E.share[b * E.n_share + tid] = EncShare{S.share[tid], (uint32_t)at_bit, (uint32_t)(at_bit >> 32)};
     if (tid == 0) {
@@ -452,7 +460,8 @@ __global__ void __launch_bounds__(kEncThreads) plan_kernel(const EncParams E) {
 
 __device__ __forceinline__ void put_le32(uint8_t* p, uint32_t v) { *reinterpret_cast<uint32_t*>(p) = v; }
 
-__global__ void __launch_bounds__(kEncThreads) write_kernel(const EncParams E, const uint64_t* offsets, uint8_t* out) {
+template <int NT>
+__global__ void __launch_bounds__(NT, 2048 / NT) write_kernel(const EncParams E, const uint64_t* offsets, uint8_t* out) {
   __shared__ uint16_t rc[kNLL + kNOff];  // canonical codes, bit-reversed for LSB-first output
   __shared__ uint8_t lens[kNLL + kNOff];
   __shared__ uint32_t warp_sum[32];
@@ -466,20 +475,20 @@ __global__ void __launch_bounds__(kEncThreads) write_kernel(const EncParams E, c
     const ParseToken* t = E.tok + b * E.stride;
     const uint32_t* tp = E.tpos + b * E.stride;
     // zero the block (P.bytes is a multiple of 16, dst 16-byte aligned)
-    for (uint64_t i = 16ull * tid; i < P.bytes; i += 16ull * kEncThreads)
+    for (uint64_t i = 16ull * tid; i < P.bytes; i += 16ull * NT)
       *reinterpret_cast<uint4*>(dst + i) = make_uint4(0, 0, 0, 0);
     if (!E.byte_mode) {
-      for (uint32_t i = tid; i < kNLL + kNOff; i += kEncThreads) lens[i] = P.lens[i];
+      for (uint32_t i = tid; i < kNLL + kNOff; i += NT) lens[i] = P.lens[i];
     }
     __syncthreads();
     if (E.byte_mode) {
       // {n_seq, out_bytes, n_lit, 0}, one record per sequence, the literals
-      const uint32_t C = (n + kEncThreads - 1) / kEncThreads;
+      const uint32_t C = (n + NT - 1) / NT;
       const uint32_t k0 = min(tid * C, n), k1 = min(k0 + C, n);
       uint32_t l = 0;
       for (uint32_t k = k0; k < k1; k++) l += t[k].lit_len;
       uint32_t all;
-      uint32_t lo = cta_scan(l, warp_sum, all);
+      uint32_t lo = cta_scan<NT>(l, warp_sum, all);
       if (tid == 0) {
         put_le32(dst, n);
         put_le32(dst + 4, P.out_bytes);
@@ -504,9 +513,9 @@ __global__ void __launch_bounds__(kEncThreads) write_kernel(const EncParams E, c
       put_le32(dst, n);
       put_le32(dst + 4, P.out_bytes);
     }
-    if (tid < (kNLL + 1) / 2) {
-      const uint32_t s = 2 * tid;
-      dst[8 + tid] = (uint8_t)(lens[s] | ((s + 1 < kNLL ? lens[s + 1] : 0u) << 4));
+    for (uint32_t i = tid; i < (kNLL + 1) / 2; i += NT) {
+      const uint32_t s = 2 * i;
+      dst[8 + i] = (uint8_t)(lens[s] | ((s + 1 < kNLL ? lens[s + 1] : 0u) << 4));
     }
     if (tid < kNOff / 2) dst[168 + tid] = (uint8_t)(lens[kNLL + 2 * tid] | (lens[kNLL + 2 * tid + 1] << 4));
     if (tid < K) {
@@ -578,17 +587,37 @@ __global__ void __launch_bounds__(kEncThreads) write_kernel(const EncParams E, c
 
 }  // namespace
 
+uint32_t encode_threads(const EncLaunch& L, uint32_t sms) {
+  if (L.byte_mode && L.block_size > 16384) return 1024;
+  for (uint32_t threads = 1024; threads > 128; threads /= 2)
+    if (L.n_blocks <= (uint64_t)sms * (1024 / threads)) return threads;
+  return 128;
+}
+
+static EncParams params(const EncLaunch& L) {
+  return EncParams{L.in, L.n, L.block_size, L.n_sub, L.cwl, L.window, L.max_match, L.byte_mode, L.n_blocks, L.tok,
+                   L.tpos, L.stride, L.count, L.plan, L.share, L.n_share, L.block_bytes, L.error};
+}
+
 cudaError_t launch_encode_plan(const EncLaunch& L) {
-  EncParams E{L.in, L.n, L.block_size, L.n_sub, L.cwl, L.window, L.max_match, L.byte_mode, L.n_blocks, L.tok,
-              L.tpos, L.stride, L.count, L.plan, L.share, L.n_share, L.block_bytes, L.error};
-  plan_kernel<<<L.grid, kEncThreads, 0, L.stream>>>(E);
+  const EncParams E = params(L);
+  switch (L.threads) {
+    case 128: plan_kernel<128><<<L.grid, 128, 0, L.stream>>>(E); break;
+    case 256: plan_kernel<256><<<L.grid, 256, 0, L.stream>>>(E); break;
+    case 512: plan_kernel<512><<<L.grid, 512, 0, L.stream>>>(E); break;
+    default: plan_kernel<1024><<<L.grid, 1024, 0, L.stream>>>(E);
+  }
   return cudaGetLastError();
 }
 
 cudaError_t launch_encode_write(const EncLaunch& L, const uint64_t* offsets, uint8_t* out) {
-  EncParams E{L.in, L.n, L.block_size, L.n_sub, L.cwl, L.window, L.max_match, L.byte_mode, L.n_blocks, L.tok,
-              L.tpos, L.stride, L.count, L.plan, L.share, L.n_share, L.block_bytes, L.error};
-  write_kernel<<<L.grid, kEncThreads, 0, L.stream>>>(E, offsets, out);
+  const EncParams E = params(L);
+  switch (L.threads) {
+    case 128: write_kernel<128><<<L.grid, 128, 0, L.stream>>>(E, offsets, out); break;
+    case 256: write_kernel<256><<<L.grid, 256, 0, L.stream>>>(E, offsets, out); break;
+    case 512: write_kernel<512><<<L.grid, 512, 0, L.stream>>>(E, offsets, out); break;
+    default: write_kernel<1024><<<L.grid, 1024, 0, L.stream>>>(E, offsets, out);
+  }
   return cudaGetLastError();
 }
 

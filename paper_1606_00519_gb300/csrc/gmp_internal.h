@@ -86,9 +86,6 @@ struct ParseToken {
 // GPU entropy coding of GPU parses (gmp_gpuencode.cu): per block, a plan
 // (token checks, code lengths, sub-block split and sizes), then the block's
 // bytes at an offset computed from the planned sizes.
-// Writing threads per block: its tokens in this many runs of about equal work,
-// or in fewer where a block has not as many tokens.
-constexpr uint32_t kEncShares = 1024;
 struct EncShare {
   uint32_t first, bit_lo, bit_hi;  // first token, its first bit (a block may have 2^32 and more)
 };
@@ -112,12 +109,14 @@ struct EncLaunch {
   const uint32_t* count;  // tokens per block
   EncBlockPlan* plan;
   EncShare* share;        // n_share per block
-  uint32_t n_share;       // at most kEncShares
+  uint32_t threads;       // per block (a CTA): encode_threads()
+  uint32_t n_share;       // runs of about equal work for writing: `threads`, or fewer with fewer tokens
   uint64_t* block_bytes;  // encoded size per block
   int* error;             // set to 1 if a token fails its checks
   unsigned grid;
   cudaStream_t stream;
 };
+uint32_t encode_threads(const EncLaunch& L, uint32_t sms);
 cudaError_t launch_encode_plan(const EncLaunch& L);
 cudaError_t launch_encode_write(const EncLaunch& L, const uint64_t* offsets, uint8_t* out);
 // Stream layout (gmp_compress.cpp): block offsets (absolute, 16-byte
