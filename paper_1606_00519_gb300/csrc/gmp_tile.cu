@@ -28,7 +28,8 @@
 //  So MRR and DE streams take the same path at the same speed.
 //
 //  Byte blocks (Gompresso/Byte, Sec. 3.1) run phase B on the stream's own
-//  records, with each group's records checked before it is staged.
+//  records, with each group's records checked before it is staged, in groups of
+//  fewer records where they write more.
 //
 // What bounds it and what it measured (GB300, 152 SMs): the number of
 // instructions with every SM full (2.4 warp instructions per byte of text,
@@ -111,16 +112,18 @@ struct TileSmemA {
 // bytes and the group being written: it slides down (by a multiple of 16)
 // when a group would not fit.
 constexpr uint32_t kHist = 1024;
-constexpr uint32_t kGroupRecs = 64;          // records of a group: two per lane, or half of them if they
-constexpr uint32_t kGroupMax = 32 * 68;  // write more than this (4 literals and a match of 64 per record)
+constexpr uint32_t kGroupRecs = 64;          // records of a group: two per lane, or half of them (Byte blocks: or
+constexpr uint32_t kGroupMax = 32 * 68;  // fewer) if they write more than this (4 literals and a match of 64 per record)
 constexpr uint32_t kBuf = 5840;
 constexpr uint32_t kFlush = 512;    // output bytes per flush (one 16-byte store per lane)
 constexpr uint32_t kFarChunks = 32 * 5;  // 16-byte chunks; a 64-byte source spans at most 5 aligned ones
-constexpr uint32_t kLitStage = 512; // a Byte group's literal run, with alignment
+constexpr uint32_t kLitStage = 8 * kGroupRecs;  // literals of Huffman records
+// A group's staging: its literals, then its far chunks.  Byte groups share it as
+// they need: a group is halved until both fit.
+constexpr uint32_t kStage = kLitStage + 16 * kFarChunks;
 constexpr uint32_t kMarkWords = (kGroupMax + 127) / 128 * 4;
 struct TileSmemB {
-  uint8_t lit[2][kLitStage];
-  uint8_t far[2][16 * kFarChunks];
+  uint8_t stage[2][kStage];
   uint32_t seg[2][2 * kGroupRecs];
   uint32_t mark[2][kMarkWords];
   uint8_t buf[kBuf + 32];  // a last tile may write up to 31 bytes past its group
@@ -141,9 +144,9 @@ struct Job {
 };
 // What the first warp of a pair hands to the second in phase B, group after
 // group.
-enum Step : uint32_t { kGroup, kSlow, kDone, kAbandon };
+enum Step : uint32_t { kGroup, kDone, kAbandon };
 struct StepMsg {
-  uint32_t what, total, shift;  // kGroup: its bytes, and what the window slides by before it
+  uint32_t what, total, shift;  // of a group: its bytes, and what the window slides by before it
 };
 struct __align__(64) TileSmem {
   union {
@@ -155,12 +158,10 @@ struct __align__(64) TileSmem {
   Job job;
   int32_t result[3];  // of the parts of the table build
   StepMsg step[2];
-  Window win;                  // after a slow group
-  uint32_t slow_t0, slow_t1;   // its records
-  const uint8_t* slow_lits;
 };
 static_assert(kBuf % 16 == 0 && sizeof(TileSmem) % 16 == 0, "16-byte copies");
-static_assert(kHist >= kFlush + 80, "what slow_group copies from the output is flushed");
+static_assert(2 * (1023 + 65) <= kGroupMax && 2 * 1023 + 30 + 16 * 2 * 5 <= kStage, "any two records of a Byte block");
+static_assert(kFarChunks >= 32 * 5, "any 32 records of a Huffman block");
 static_assert(kGroupMax + kFlush + 80 + 16 + kGroupMax <= kBuf, "two groups of the longest matches");
 static_assert(sizeof(TileSmem) * 4 + 1024 <= 57 * 1024, "16 pairs per SM in CTAs of 4");
 
@@ -610,8 +611,6 @@ __device__ __forceinline__ bool huffman_block(TileSmem& S, const BlockView& V, i
 struct Group {
   uint32_t total, lits, shift;
   int err;
-  uint32_t end;  // its last record, plus one
-  bool slow;  // a Byte group too large for the window or the literal staging, even half of it
 };
 
 __device__ __forceinline__ void slide(uint8_t* buf, Window& w, uint32_t shift) {
@@ -750,12 +749,21 @@ __device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, 
     if (j < V.K) rec_j = rec + rec_start(SS.sb_out[j], j);
   };
 
+  // records of a group: as many as a group holds of the block's mean ones (16 KiB
+  // blocks, 31 literals and a match of 9 per record, 1100 of them: 51 us; with the
+  // groups that do not fit written record after record 362; gmp_decode.cu 86)
+  uint32_t most = kGroupRecs;
+  if (BYTE) {
+    const uint32_t mean = V.out_bytes / max(V.n_seq, 1u);
+    while (most > 2u && (uint64_t)most * mean > kGroupMax) most /= 2u;
+  }
   uint4 r = load();
   // Lays out the next group (records r) at window w, its state before the
   // group, which follows one of `prev` bytes: segment starts and entries, far
   // sources and Byte literals staged by cp.async.
   auto prep = [&](const Window& w, uint32_t prev, uint32_t litpos, uint32_t stage) -> Group {
-    Group G{0, 0, 0, 0, 0, false};
+    Group G{0, 0, 0, 0};
+    uint32_t lit_span = kLitStage;
     uint32_t ll[2], ml[2], dist[2], lit_x[2] = {r.x, r.z};
 #pragma unroll
     for (int k = 0; k < 2; k++) {
@@ -775,7 +783,8 @@ __device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, 
     // that one's start is complete, and stored but for a flush row.  Sources
     // older than the window must be stored, so this much stays in it.
     const uint32_t hist = max(kHist, prev + kFlush + 80u), near = min(w.cur, hist);
-    uint32_t n = kGroupRecs, dst, segs, chunks, lit_at;
+    uint32_t n = most, dst, segs, chunks, lit_at;
+    if (BYTE && lane >= n / 2u) ll[0] = ll[1] = ml[0] = ml[1] = 0;
     for (;;) {
       // one scan gives output positions, segment numbers and places for the
       // chunks of sources that may be older than the window (in Byte blocks,
@@ -813,7 +822,8 @@ __device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, 
         else if (__any_sync(FULL, bad)) G.err = GMP_STATUS_BAD_OFFSET;
         else if ((uint64_t)w.g0 + G.total > V.out_bytes || (uint64_t)litpos + G.lits > V.n_lit)
           G.err = GMP_STATUS_OUTPUT_OVERRUN;
-        fits = !G.err && ((litpos + G.lits + 15u) & ~15u) - (litpos & ~15u) <= kLitStage;
+        lit_span = ((litpos + G.lits + 15u) & ~15u) - (litpos & ~15u);
+        fits = !G.err;
       } else {
         G.total = sum & 0x1fffu;
         n_chunks = sum >> 21;
@@ -823,28 +833,21 @@ __device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, 
         lit_at = 8u * lane;
         fits = true;
       }
-      fits = fits && G.total <= kGroupMax && n_chunks <= kFarChunks;
+      fits = fits && G.total <= kGroupMax && lit_span + 16u * n_chunks <= kStage;
       if (fits) break;
-      if (n == 32u) {  // (Byte only)
-        if (G.err) return G;
-        G.slow = true;
-        break;
-      }
-      n = 32;
-      if (lane >= 16u) ll[0] = ll[1] = ml[0] = ml[1] = 0;
+      if (n == 2u) return G;  // (Byte blocks, a failed check: any two records fit)
+      n /= 2u;
+      if (lane >= n / 2u) ll[0] = ll[1] = ml[0] = ml[1] = 0;
     }
     // the records after this group are on their way while it is laid out
-    G.end = min(i0 + n, n_j);
     step(n);
     r = load();
-    if (BYTE && G.slow) return G;
     G.shift = w.cur + G.total > kBuf ? (w.cur - hist) & ~15u : 0u;
     const uint32_t cur = w.cur - G.shift, base = w.base + G.shift;
     if (BYTE) {
-      const uint32_t l0 = litpos & ~15u, l1 = (litpos + G.lits + 15u) & ~15u;
-      if (16u * lane < l1 - l0) cp_async16(S.lit[stage] + 16u * lane, lits + l0 + 16u * lane);
+      for (uint32_t c = 16u * lane; c < lit_span; c += 512u) cp_async16(S.stage[stage] + c, lits + (litpos & ~15u) + c);
     } else {
-      *reinterpret_cast<uint2*>(S.lit[stage] + 8u * lane) = make_uint2(lit_x[0], lit_x[1]);
+      *reinterpret_cast<uint2*>(S.stage[stage] + 8u * lane) = make_uint2(lit_x[0], lit_x[1]);
     }
     // segment starts
     uint32_t* mark = S.mark[stage];
@@ -852,7 +855,7 @@ __device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, 
     __syncwarp();
     // (predicated: with branches, of which every lane takes its own mix, 2 x 512
     // MiB of records 2.90 ms against 2.86, files of 256 MiB 1.30 against 1.27)
-    const uint32_t lit_a = smem_addr(S.lit[stage]), mark_a = smem_addr(mark), far_a = smem_addr(S.far[stage]);
+    const uint32_t lit_a = smem_addr(S.stage[stage]), mark_a = smem_addr(mark), far_a = lit_a + lit_span;
     uint32_t seg_a = smem_addr(S.seg[stage]) + 4u * segs;
 #pragma unroll
     for (int k = 0; k < 2; k++) {
@@ -893,33 +896,19 @@ __device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, 
     stage ^= 1u;
   };
   while (i0 < n_j) {
-    const uint32_t t_cur = i0;
     const Group G = prep(w, prev, litpos, stage);
     if (BYTE && G.err) {
       if (lane == 0) set_status(status, G.err);
       tell(kAbandon, 0, 0);
       return;
     }
-    if (BYTE && G.slow) {
-      if (lane == 0) {
-        SS.slow_t0 = t_cur;
-        SS.slow_t1 = G.end;
-        SS.slow_lits = lits + litpos;
-      }
-      tell(kSlow, 0, 0);
-      pair_sync();  // it is written
-      stage ^= 1u;
-      w = SS.win;
-      prev = 0;
-    } else {
-      cp_async_commit();
-      cp_async_wait<0>();
-      tell(kGroup, G.total, G.shift);
-      w.g0 += G.total;
-      w.base += G.shift;
-      w.cur = w.g0 - w.base;
-      prev = G.total;
-    }
+    cp_async_commit();
+    cp_async_wait<0>();
+    tell(kGroup, G.total, G.shift);
+    w.g0 += G.total;
+    w.base += G.shift;
+    w.cur = w.g0 - w.base;
+    prev = G.total;
     litpos += G.lits;
   }
   if ((w.g0 != V.out_bytes || (BYTE && litpos != V.n_lit)) && lane == 0) set_status(status, GMP_STATUS_OUTPUT_OVERRUN);
@@ -1007,12 +996,6 @@ __device__ __forceinline__ void write_block(TileSmem& SS, uint8_t* out_blk) {
       w.g0 += m.total;
       w.cur += m.total;
       flush(S.buf, w, out_blk, vec_ok, lane, 32);
-    } else if (m.what == kSlow) {
-      slow_group(S.buf, kBuf, kHist, w, SS.job.view.B + 16, SS.slow_t0, SS.slow_t1, SS.slow_lits,
-                 SS.job.view.B + SS.job.view.lit_off + SS.job.view.n_lit, out_blk, SS.job.view.out_bytes, vec_ok);
-      if (lane == 0) SS.win = w;
-      pair_sync();
-      stage ^= 1u;
     } else {
       if (m.what == kDone) flush_rest(S.buf, w, out_blk, vec_ok, lane, 32);
       return;
@@ -1135,17 +1118,21 @@ __global__ void __launch_bounds__(1024, 1) tile_kernel(const KParams P) {
 // follow, flush).  One warp took 1.55 ms for it (a pair of warps now 1.0): 16 KiB 156 -> 51 us, 1 MiB of
 // 64 KiB blocks 754 -> 195, 16 MiB of records 1554 -> 310, 64 MiB of text 1599
 // -> 548, 128 MiB of Byte records 1541 -> 540.
-constexpr uint32_t kLitWave = 1984;  // most literal bytes of a wave of a Byte block
-constexpr uint32_t kLitRing = 4096;  // literal bytes of a Byte block held; the first kLitOver again at the end
+// Literal bytes of a Byte block held: what 227 KB leave a CTA; the first kLitOver
+// again at the end.  A wave's and the next one's fit.
+__host__ __device__ constexpr uint32_t lit_ring(int W) { return W <= 8 ? 8192 : 32768; }
 constexpr uint32_t kLitOver = 1024;
 constexpr uint32_t kCoopRecs = 2;  // a lane's records of a group
 constexpr uint32_t kCoopGroupMax = kCoopRecs * kGroupMax;
 // most output bytes of a wave (a group of text or of CSV rows is about 520)
 __host__ __device__ constexpr uint32_t wave_bytes(int W) { return 768 * W; }
+__host__ __device__ constexpr uint32_t wave_lits(int W) {  // most literal bytes of a wave (Byte blocks)
+  return lit_ring(W) / 2 - 16 < wave_bytes(W) ? lit_ring(W) / 2 - 16 : wave_bytes(W);
+}
 __host__ __device__ constexpr uint32_t coop_buf(int W) { return 32768 + 16 + wave_bytes(W) + (W <= 8 ? 4096 : 32768); }
 constexpr uint32_t kFollow = 12;  // tiles followed at once
 constexpr uint32_t kValue = 0x8000;  // note: bits 0-7 are the byte; else its source's place in the wave
-static_assert(kCoopGroupMax <= wave_bytes(8) && wave_bytes(16) < kValue && 2 * kLitWave + 16 <= kLitRing, "wave sizes");
+static_assert(kCoopGroupMax <= wave_bytes(8) && wave_bytes(16) < kValue, "wave sizes");
 
 struct CoopSmemA {
   uint32_t ll[LUT_SIZE], off[LUT_SIZE];
@@ -1160,7 +1147,7 @@ struct CoopSmemB {
   uint8_t lit[W][128 * kCoopRecs];
   uint32_t seg[W][64 * kCoopRecs];
   uint32_t mark[W][(kCoopGroupMax + 127) / 128 * 4];
-  uint8_t blit[kLitRing + kLitOver];
+  uint8_t blit[lit_ring(W) + kLitOver];
   uint16_t note[wave_bytes(W)];
   uint8_t buf[coop_buf(W) + 160];  // a last batch of tiles may read up to 127 bytes past the wave
 };
@@ -1242,6 +1229,7 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
                                         uint8_t* out_blk) {
   CoopSmemB<W>& S = SS.u.b;
   constexpr uint32_t NT = 32 * W, CB = coop_buf(W), kWave = wave_bytes(W), R = kCoopRecs, GR = 32 * R;
+  constexpr uint32_t kLitRing = lit_ring(W), kLitWave = wave_lits(W);
   const uint32_t t = threadIdx.x, warp = t >> 5, lane = lane_id();
   const uint32_t le = (2u << lane) - 1u;
   const bool vec_ok = (((uintptr_t)out_blk) & 15u) == 0;
@@ -1251,17 +1239,26 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
   // kept below a wave: what a match reaches, and what is not flushed
   const uint32_t hist = max((V.window + 15u) & ~15u, kFlush);
 
-  // groups of GR records: the block's for Byte blocks, else each sub-block's
-  uint32_t n_groups;
+  // groups of GR records of a sub-block; Byte blocks: of as many, a power of two,
+  // as let every warp have its share of a wave (64 KiB blocks, 31 literals and a
+  // match of 9 per record, groups of 64 and a ring of 4 KiB: one block 229 us, 700
+  // of them 482; so 50 and 166; gmp_decode.cu 198 and 224).
+  // i0: the warp's first record of sub-block j; Byte blocks: the lane's, past
+  // every block for a lane without any.
+  uint32_t n_groups, i0 = GR * warp, next = GR * W;
   if (BYTE) {
-    n_groups = V.n_seq / GR + (V.n_seq % GR ? 1u : 0u);
+    const uint32_t mean = V.out_bytes / max(V.n_seq, 1u);
+    uint32_t gr = GR;
+    while (gr > 2u && (uint64_t)gr * mean > kWave / W) gr /= 2u;
+    n_groups = V.n_seq / gr + (V.n_seq % gr ? 1u : 0u);
+    i0 = R * lane < gr ? gr * warp + R * lane : 1u << 31;
+    next = gr * W;
   } else {
     uint32_t g = 0;
     for (uint32_t j = lane; j < V.K; j += 32) g += (SS.sb_cnt[j] + GR - 1u) / GR;
     n_groups = __reduce_add_sync(FULL, g);
   }
-  // the warp's group: record i0 of sub-block j (whose records start at rec_j)
-  uint32_t j = 0, i0 = GR * warp, n_j = BYTE ? V.n_seq : SS.sb_cnt[0];
+  uint32_t j = 0, n_j = BYTE ? V.n_seq : SS.sb_cnt[0];
   const uint2* rec_j = rec;
   auto settle = [&]() {
     if constexpr (!BYTE) {
@@ -1282,7 +1279,7 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
     uint2 r[R];
   };
   auto load = [&]() -> Recs {
-    const uint32_t i = i0 + R * lane;
+    const uint32_t i = BYTE ? i0 : i0 + R * lane;
     Recs x;
 #pragma unroll
     for (uint32_t k = 0; k < R; k++) x.r[k] = make_uint2(0, 0);
@@ -1351,8 +1348,8 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
       inc_l = warp_incl_scan(own_l);
       if (lane == 31) SS.tot_l[it & 1u][warp] = inc_l;
     }
-    const uint32_t t_cur = i0;  // the group's first record
-    i0 += GR * W;
+    const uint32_t t_cur = i0;  // the group's (Byte blocks: the lane's) first record
+    i0 += next;
     settle();
     r = load();
     if (BYTE) cp_async_wait<0>();
@@ -1420,7 +1417,8 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
         if (SS.bad != ~0u) break;
         if (warp == lo) {
           Window x = w;
-          slow_group(S.buf, CB, hist, x, recs, t_cur, min(t_cur + GR, V.n_seq), lits + litpos, lits + V.n_lit, out_blk,
+          const uint32_t t0 = __shfl_sync(FULL, t_cur, 0);
+          slow_group(S.buf, CB, hist, x, recs, t0, min(t0 + next / W, V.n_seq), lits + litpos, lits + V.n_lit, out_blk,
                      V.out_bytes, vec_ok);
           if (lane == 0) SS.win = x;
         }
