@@ -11,7 +11,9 @@
 //  bits together, so that a sequence takes about one step.  Each sequence
 //  becomes an 8-byte record with its literals inside {literal bytes, distance
 //  | match length << 16 | literal count << 24}; a longer literal string takes
-//  further records of 3 or 4 literals without a match.  Records go to the
+//  further records of 3 or 4 literals without a match.  In blocks of long
+//  literal strings a step looks up to three times, and such records have 5 to 7
+//  literals, in their first seven bytes.  Records go to the
 //  pair's scratch slot.
 //
 //  Phase B, LZ77 decompression (Sec. 3.2.2): the first warp lays out groups of
@@ -53,6 +55,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
+
+#include <type_traits>
 
 #include "gmp.h"
 #include "gmp_decode_common.h"
@@ -117,7 +121,7 @@ constexpr uint32_t kGroupMax = 32 * 68;  // fewer) if they write more than this 
 constexpr uint32_t kBuf = 5840;
 constexpr uint32_t kFlush = 512;    // output bytes per flush (one 16-byte store per lane)
 constexpr uint32_t kFarChunks = 32 * 5;  // 16-byte chunks; a 64-byte source spans at most 5 aligned ones
-constexpr uint32_t kLitStage = 8 * kGroupRecs;  // literals of Huffman records
+constexpr uint32_t kLitStage = 8 * kGroupRecs;  // Huffman records, with their literals
 // A group's staging: its literals, then its far chunks.  Byte groups share it as
 // they need: a group is halved until both fit.
 constexpr uint32_t kStage = kLitStage + 16 * kFarChunks;
@@ -313,12 +317,13 @@ __device__ __forceinline__ void fill_off(uint32_t* lut, const Canon& C, const ui
 
 // Phase A of one lane's sub-block (whole warp calls; `act`: the lane has
 // one).  The step is straight-line code: a lane that is done takes empty
-// entries, and literal and match work run under selects, so that the compiler
+// entries, and literal and match work run under selects (DENSE: the match's
+// lookup is left out when no lane has one), so that the compiler
 // can overlap a step's two table latencies with the record's arithmetic.  The
 // lane's 16-byte bitstream chunks pass through a ring of four in shared
 // memory, copied there by cp.async: asked for every second step, and at most
-// 74 bits are taken in two steps, so that a chunk is not read before the
-// third wait after it was asked for.
+// 74 bits are taken in two steps (DENSE: every step, 61 bits), so that a chunk
+// is not read before the third wait after it was asked for.
 struct SubBlock {
   uint32_t pos, bits;      // first bit, size in bits
   uint32_t out, out_n;     // output start and size
@@ -349,7 +354,7 @@ __device__ __forceinline__ uint32_t shr_clamp(uint32_t v, uint32_t n) {
   asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(n));
   return r;
 }
-template <int LLB, int OFB, bool PAIR>
+template <int LLB, int OFB, bool PAIR, bool DENSE>
 __device__ __forceinline__ uint32_t huffman_lane(const uint32_t* ll_lut, const uint32_t* off_lut, const Canon& coff,
                                                  const uint16_t* sorted_off, const uint32_t* ring, const uint8_t* bs,
                                                  uint32_t n_chunks, bool act, bool empty, const SubBlock& sb,
@@ -389,7 +394,8 @@ __device__ __forceinline__ uint32_t huffman_lane(const uint32_t* ll_lut, const u
     if (next) w2 = ring[(np >> 5) & 15u];
     pos = np;
   };
-  uint32_t lits = 0, ln8 = 0, cnt = 0;
+  std::conditional_t<DENSE, uint64_t, uint32_t> lits = 0;  // pending literals, ln8 bits
+  uint32_t ln8 = 0, cnt = 0;
   uint2 q2 = make_uint2(0, 0), q3 = q2;  // PAIR: the last two records
   // the entry of a peek
   auto ll_of = [&](uint32_t pk) -> uint32_t {
@@ -407,51 +413,73 @@ __device__ __forceinline__ uint32_t huffman_lane(const uint32_t* ll_lut, const u
   };
   bool odd = false;  // what the checks after a pair of steps look at
   auto one = [&]() {
-    const uint32_t pk = __funnelshift_r(w0, w1, pos);
-    uint32_t e = ll_of(pk);
-    e = rem ? e : 0u;
-    const int mc = byte1_signed(e);
-    advance(e & 15u);
-    lits |= (e >> 16) << ln8;
-    ln8 += (e >> 1) & 24u;
+    // a lookup, or up to three while they give literals alone and fewer than
+    // six of them are pending
+    int mc = 0;
+#pragma unroll
+    for (int k = 0; k < (DENSE ? 3 : 1); k++) {
+      uint32_t e = ll_of(__funnelshift_r(w0, w1, pos));
+      e = (k == 0 ? rem != 0 : mc == 0 && ln8 < 48u && rem != 0) ? e : 0u;
+      mc = k == 0 ? byte1_signed(e) : mc + byte1_signed(e);
+      advance(e & 15u);
+      lits |= (decltype(lits))(e >> 16) << ln8;
+      ln8 += (e >> 1) & 24u;
+    }
     const uint32_t pk2 = __funnelshift_r(w0, w1, pos);
-    uint32_t e2 = off_lut[pk2 & ((1u << OFB) - 1u)];
-    e2 = mc > 0 ? e2 : kNoMatch;
-    if (OFB < LUT_BITS && __any_sync(FULL, e2 == kLongOff)) {
-      if (e2 == kLongOff) e2 = off_long(pk2);
+    uint32_t e2 = kNoMatch;
+    if (!DENSE || __any_sync(FULL, mc > 0)) {
+      e2 = off_lut[pk2 & ((1u << OFB) - 1u)];
+      e2 = mc > 0 ? e2 : kNoMatch;
+      if (OFB < LUT_BITS && __any_sync(FULL, e2 == kLongOff)) {
+        if (e2 == kLongOff) e2 = off_long(pk2);
+      }
     }
     const uint32_t s1 = e2 & 63u, s2 = __byte_perm(e2, 0, 0x4441);
     const uint32_t dist = (e2 >> 16) + shr_clamp(shl_clamp(pk2, s1), s2);
     advance(32u - s1);
     const uint32_t ml = (uint32_t)max(mc, 0), wpos = outp + (ln8 >> 3);
     odd = odd || mc < 0 || dist > min(window, wpos);
-    const bool emit = mc != 0 || ln8 >= 24u;
-    const uint2 r = make_uint2(lits, dist | (ml << 16) | (ln8 << 21));
-    if (PAIR) {
-      q2 = emit ? q3 : q2;
-      q3 = emit ? r : q3;
-      cnt += emit ? 1u : 0u;
-      st_global_16B_if(rec + (cnt - 2u), q2, q3, emit && (cnt & 1u) == 0);
+    if (DENSE) {
+      // more literals than a match's record takes go out by themselves
+      const bool wide = ln8 > 32u, match = mc != 0;
+      st_global_if(rec + cnt, make_uint2((uint32_t)lits, (uint32_t)((uint64_t)lits >> 32) | (ln8 << 21)), wide);
+      cnt += wide ? 1u : 0u;
+      lits = wide ? 0u : lits;
+      ln8 = wide ? 0u : ln8;
+      st_global_if(rec + cnt, make_uint2((uint32_t)lits, dist | (ml << 16) | (ln8 << 21)), match);
+      cnt += match ? 1u : 0u;
+      outp = wide || match ? wpos + ml : outp;
+      lits = match ? 0u : lits;
+      ln8 = match ? 0u : ln8;
     } else {
-      st_global_if(rec + cnt, r, emit);
-      cnt += emit ? 1u : 0u;
+      const bool emit = mc != 0 || ln8 >= 24u;
+      const uint2 r = make_uint2((uint32_t)lits, dist | (ml << 16) | (ln8 << 21));
+      if (PAIR) {
+        q2 = emit ? q3 : q2;
+        q3 = emit ? r : q3;
+        cnt += emit ? 1u : 0u;
+        st_global_16B_if(rec + (cnt - 2u), q2, q3, emit && (cnt & 1u) == 0);
+      } else {
+        st_global_if(rec + cnt, r, emit);
+        cnt += emit ? 1u : 0u;
+      }
+      outp = emit ? wpos + ml : outp;
+      lits = emit ? 0u : lits;
+      ln8 = emit ? 0u : ln8;
     }
-    outp = emit ? wpos + ml : outp;
-    lits = emit ? 0u : lits;
-    ln8 = emit ? 0u : ln8;
     rem -= mc != 0 ? 1u : 0u;
   };
   while (__any_sync(FULL, rem != 0)) {
     const uint32_t pos0 = pos, out0 = outp + (ln8 >> 3), rem0 = rem;
     odd = false;
     one();
-    one();
+    if (!DENSE) one();
     if (__any_sync(FULL, odd || pos > end || outp > out_end)) {
-      // an end symbol or a corrupt stream: the pair of steps again, with every
-      // check.  A lane that runs past its sub-block stops here, which bounds
+      // an end symbol or a corrupt stream: the step or pair of steps again, with
+      // every check.  A lane that runs past its sub-block stops here, which bounds
       // the loop; literals past the sub-block's output are noticed when it ends.
       uint32_t p = pos0, o = out0, left = rem0;
-      for (int k = 0; k < 2 && left && !err; k++) {
+      for (int k = 0; k < (DENSE ? 3 : 2) && left && !err && (!DENSE || p < pos); k++) {
         auto peek = [&]() {
           return __funnelshift_r(ring[((p >> 5) - 2u) & 15u], ring[((p >> 5) - 1u) & 15u], p);
         };
@@ -490,13 +518,23 @@ __device__ __forceinline__ uint32_t huffman_lane(const uint32_t* ll_lut, const u
     cp_async_wait<2>();
   }
   cp_async_wait<0>();
-  if (PAIR && cnt <= rec_cap) {
+  if (PAIR && !DENSE && cnt <= rec_cap) {
     if (cnt & 1u) rec[cnt - 1u] = q3;  // not stored yet
   }
   outp += ln8 >> 3;
   if (!err && pos != end) err = GMP_STATUS_BITSTREAM;
   if (!err && outp != out_end) err = GMP_STATUS_OUTPUT_OVERRUN;
   return cnt;
+}
+
+// Whether a block's sequences are long strings of literals: more than 40 bits
+// each, of which a match takes about 17 (text and CSV rows: 24 to 26 in all).  A
+// step with one lookup decodes a literal or two in what a match takes too (1100
+// blocks, us, step of one lookup / of three / gmp_decode.cu: 16 KiB of random
+// bytes 3383 / 2010 / 2386; 64 KiB, 12 literals and a match of 9 per sequence
+// 693 / 525 / 659, 31 literals 824 / 554 / 751).
+__device__ __forceinline__ bool dense(const BlockView& V, uint32_t bs_off) {
+  return (V.comp_bytes - bs_off) / 5u > V.n_seq;
 }
 
 // Sub-block table: prefix sums of bit sizes, output sizes and sequences over
@@ -593,9 +631,12 @@ __device__ __forceinline__ bool huffman_block(TileSmem& S, const BlockView& V, i
     for (uint32_t jb = 0; jb < V.K; jb += 32) {
       const uint32_t j = jb + lane;
       const SubBlock sb = sub_block(V, A.sb_bit, S.sb_out, A.sb_seq, j);
-      const uint32_t cnt = huffman_lane<kLLBits, kOffBits, true>(
-          A.ll, A.off, A.coff, A.sorted_off, A.u.bits[lane], bs, n_chunks, j < V.K, n_ll == 0, sb, V.n_seq, V.window,
-          rec + rec_start(sb.out, j), err);
+      auto decode = [&](auto is_dense) {
+        return huffman_lane<kLLBits, kOffBits, true, decltype(is_dense)::value>(
+            A.ll, A.off, A.coff, A.sorted_off, A.u.bits[lane], bs, n_chunks, j < V.K, n_ll == 0, sb, V.n_seq, V.window,
+            rec + rec_start(sb.out, j), err);
+      };
+      const uint32_t cnt = dense(V, bs_off) ? decode(std::true_type()) : decode(std::false_type());
       if (j < V.K) S.sb_cnt[j] = cnt;
     }
     if (err) set_status(status, err);
@@ -764,7 +805,8 @@ __device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, 
   auto prep = [&](const Window& w, uint32_t prev, uint32_t litpos, uint32_t stage) -> Group {
     Group G{0, 0, 0, 0};
     uint32_t lit_span = kLitStage;
-    uint32_t ll[2], ml[2], dist[2], lit_x[2] = {r.x, r.z};
+    uint32_t ll[2], ml[2], dist[2];
+    const uint4 own_recs = r;
 #pragma unroll
     for (int k = 0; k < 2; k++) {
       const uint32_t y = k ? r.w : r.y;
@@ -775,7 +817,7 @@ __device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, 
         dist[k] = (y >> 16) + 1u;
       } else {
         ll[k] = y >> 24;
-        ml[k] = (y >> 16) & 255u;
+        ml[k] = ll[k] > 4u ? 0u : (y >> 16) & 255u;
         dist[k] = y & 0xffffu;
       }
     }
@@ -830,7 +872,7 @@ __device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, 
         dst = ex & 0x1fffu;
         segs = (ex >> 13) & 255u;
         chunks = ex >> 21;
-        lit_at = 8u * lane;
+        lit_at = 16u * lane;
         fits = true;
       }
       fits = fits && G.total <= kGroupMax && lit_span + 16u * n_chunks <= kStage;
@@ -847,7 +889,7 @@ __device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, 
     if (BYTE) {
       for (uint32_t c = 16u * lane; c < lit_span; c += 512u) cp_async16(S.stage[stage] + c, lits + (litpos & ~15u) + c);
     } else {
-      *reinterpret_cast<uint2*>(S.stage[stage] + 8u * lane) = make_uint2(lit_x[0], lit_x[1]);
+      *reinterpret_cast<uint4*>(S.stage[stage] + 16u * lane) = own_recs;
     }
     // segment starts
     uint32_t* mark = S.mark[stage];
@@ -863,7 +905,7 @@ __device__ __forceinline__ void lay_out_block(TileSmem& SS, const BlockView& V, 
       segment_if(mark_a, dst, seg_a, lit_a + lit_at - dst, has_l);
       seg_a += has_l ? 4u : 0u;
       dst += ll[k];
-      lit_at += BYTE ? ll[k] : 4u;
+      lit_at += BYTE ? ll[k] : 8u;
       const uint32_t src = w.g0 + dst - dist[k], place = far_a + 16u * chunks;
       const bool is_far = has_m && src < base;
       segment_if(mark_a, dst, seg_a, is_far ? place + (src & 15u) - dst : buf_a + cur - dist[k], has_m);
@@ -1144,10 +1186,12 @@ struct CoopSmemA {
 };
 template <int W>
 struct CoopSmemB {
-  uint8_t lit[W][128 * kCoopRecs];
   uint32_t seg[W][64 * kCoopRecs];
   uint32_t mark[W][(kCoopGroupMax + 127) / 128 * 4];
-  uint8_t blit[lit_ring(W) + kLitOver];
+  union {
+    uint8_t huffman[W][256 * kCoopRecs];    // the records
+    uint8_t ring[lit_ring(W) + kLitOver];  // Byte blocks
+  } lits;
   uint16_t note[wave_bytes(W)];
   uint8_t buf[coop_buf(W) + 160];  // a last batch of tiles may read up to 127 bytes past the wave
 };
@@ -1216,9 +1260,12 @@ __device__ bool coop_huffman(CoopSmem<W>& S, const BlockView& V, int32_t* status
   constexpr uint32_t HW = W == 16 ? 8 : 4;
   const uint32_t j = warp < HW ? lane * HW + warp : MAX_SUB;
   const SubBlock sb = sub_block(V, A.sb_bit, S.sb_out, A.sb_seq, j);
-  const uint32_t cnt = huffman_lane<LUT_BITS, LUT_BITS, false>(
-      A.ll, A.off, A.coff, A.sorted_off, A.bits[min(j, (uint32_t)MAX_SUB - 1u)], bs, n_chunks, j < V.K, n_ll == 0,
-      sb, V.n_seq, V.window, rec + rec_start(sb.out, j), err);
+  auto decode = [&](auto is_dense) {
+    return huffman_lane<LUT_BITS, LUT_BITS, false, decltype(is_dense)::value>(
+        A.ll, A.off, A.coff, A.sorted_off, A.bits[min(j, (uint32_t)MAX_SUB - 1u)], bs, n_chunks, j < V.K, n_ll == 0,
+        sb, V.n_seq, V.window, rec + rec_start(sb.out, j), err);
+  };
+  const uint32_t cnt = dense(V, bs_off) ? decode(std::true_type()) : decode(std::false_type());
   if (j < V.K) S.sb_cnt[j] = cnt;
   if (err) set_status(status, err);
   return !__syncthreads_or(err != 0);  // the records are visible to the whole CTA
@@ -1309,8 +1356,8 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
     const uint32_t upto = min((V.n_lit + 15u) & ~15u, (litpos & ~15u) + kLitRing);
     for (uint32_t c = lit_asked + 16u * t; c < upto; c += 16u * NT) {
       const uint32_t at = c & (kLitRing - 1u);
-      cp_async16(S.blit + at, lits + c);
-      if (at < kLitOver) cp_async16(S.blit + kLitRing + at, lits + c);
+      cp_async16(S.lits.ring + at, lits + c);
+      if (at < kLitOver) cp_async16(S.lits.ring + kLitRing + at, lits + c);
     }
     cp_async_commit();
     lit_asked = max(lit_asked, upto);
@@ -1323,6 +1370,9 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
     // lengths of the lane's records; one scan gives output positions and (from
     // bit 20) the number of the segments before
     uint32_t ll[R], ml[R], dist[R], own = 0, own_l = 0, inc_l = 0;
+    if (!BYTE)
+      *reinterpret_cast<uint4*>(S.lits.huffman[warp] + 8u * R * lane) =
+          make_uint4(r.r[0].x, r.r[0].y, r.r[R - 1].x, r.r[R - 1].y);
 #pragma unroll
     for (uint32_t k = 0; k < R; k++) {
       const uint32_t y = r.r[k].y;
@@ -1333,9 +1383,8 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
         dist[k] = (y >> 16) + 1u;
       } else {
         ll[k] = y >> 24;
-        ml[k] = (y >> 16) & 255u;
+        ml[k] = ll[k] > 4u ? 0u : (y >> 16) & 255u;
         dist[k] = y & 0xffffu;
-        *reinterpret_cast<uint32_t*>(S.lit[warp] + 4u * (R * lane + k)) = r.r[k].x;
       }
       own += ll[k] + ml[k] + (ll[k] ? 1u << 20 : 0u) + (ml[k] ? 1u << 20 : 0u);
       own_l += ll[k];
@@ -1443,8 +1492,8 @@ __device__ __forceinline__ void coop_lz(CoopSmem<W>& SS, const BlockView& V, int
         for (uint32_t k = 0; k < R; k++) {
           if (ll[k]) {
             atomicOr(mark + (at >> 5), 1u << (at & 31u));
-            seg[n++] = (BYTE ? smem_addr(S.blit) + (lit_at & (kLitRing - 1u))
-                             : smem_addr(S.lit[warp]) + 4u * (R * lane + k)) -
+            seg[n++] = (BYTE ? smem_addr(S.lits.ring) + (lit_at & (kLitRing - 1u))
+                             : smem_addr(S.lits.huffman[warp]) + 8u * (R * lane + k)) -
                        at;
           }
           at += ll[k];

@@ -1,8 +1,8 @@
-"""GPU tests of Byte blocks whose literal strings outgrow the staging of a group
-or a wave and are read from the stream: the oracle's bytes for records of every
-kind of literal length and distance, decoded by a CTA per block and (more
-blocks) by a pair of warps per block, at aligned and unaligned outputs, and
-damaged records among them."""
+"""GPU tests of blocks of long literal strings, which take groups of fewer records
+(Byte blocks) or records of up to seven literals (Huffman blocks): the oracle's
+bytes for every kind of literal length and distance, decoded by a CTA per block
+and (more blocks) by a pair of warps per block, at aligned and unaligned
+outputs, damaged blocks among them, and the time beside that of text."""
 import numpy as np
 import pytest
 
@@ -83,14 +83,62 @@ def test_damaged_records(gmp, ctx, kind, copies):  # noqa: F811
     assert failed > 5
 
 
+HUFFMAN = {"3 to 9": [3, 4, 5, 6, 7, 8, 9], "around 14": [12, 13, 14, 15, 16], "mean 31": [15, 16, 31, 32, 63],
+           "long": [255, 256, 257, 1023, 5000], "some": [0, 1, 2, 3, 4, 5, 6, 1000]}
+
+
+def huffman_stream(gmp, kind, seed, n, n_sub):  # noqa: F811
+    ll, ml, dist, lits = tokens(seed, n, HUFFMAN[kind], [1, 2, 31, 33, 1000, 2500, 30_000])
+    ml = np.maximum(ml, 3)  # every sequence but the last has a match
+    ml[-1] = 0
+    at = np.cumsum(ll.astype(np.int64)) + np.concatenate([[0], np.cumsum(ml.astype(np.int64))[:-1]])
+    dist = np.where(ml > 0, np.clip(dist, 1, np.minimum(at, 32768)), 0).astype(np.uint32)
+    if seed % 2:
+        lits = np.minimum(lits, 40 + lits % 30)  # shorter codes: lookups of two literals
+    return gmp.encode_tokens(ll, ml, dist, lits, n_sub=n_sub), oracle.lz77_decode(ll, ml, dist, lits)
+
+
+@pytest.mark.parametrize("copies", [1, 200, PAIRS])
+@pytest.mark.parametrize("kind", list(HUFFMAN))
+def test_huffman_literal_lengths(gmp, ctx, kind, copies):  # noqa: F811
+    for seed, n, n_sub in ((1, 2, 1), (2, 40, 3), (3, 65, 33), (4, 700, 64), (5, 900, 32), (6, 30, 16)):
+        s, data = huffman_stream(gmp, kind, seed, n, n_sub)
+        if data.size > 256 * KiB:  # what the context's blocks may hold
+            continue
+        for offset in (0, 16, 3):
+            st, same, guard = decode(gmp, ctx, s, data, copies, offset)
+            assert not st.any() and same and guard, (seed, offset)
+
+
+@pytest.mark.parametrize("copies", [1, PAIRS])
+@pytest.mark.parametrize("kind", ["3 to 9", "mean 31", "some"])
+def test_damaged_huffman_blocks(gmp, ctx, kind, copies):  # noqa: F811
+    s, data = huffman_stream(gmp, kind, 7, 300, 16)
+    lo = int(s[64:72].view(np.uint64)[0])
+    rng = np.random.default_rng(4)
+    failed = 0
+    for k in range(40):
+        bad = s.copy()
+        bad[int(rng.integers(lo, lo + 400 if k % 3 == 0 else s.size - 17))] ^= np.uint8(1 << int(rng.integers(0, 8)))
+        want = oracle.decompress_status(bad)
+        try:
+            st, same, guard = decode(gmp, ctx, bad, data if want else oracle.decompress(bad), copies, 0)
+        except gmp.GmpError:
+            continue
+        assert ((st != 0) == (want != 0)).all() and guard and (want != 0 or same)
+        failed += want != 0
+    assert failed > 5
+
+
+@pytest.mark.parametrize("byte_mode", [False, True])
 @pytest.mark.parametrize("block,n_blocks", [(16 * KiB, 1100), (64 * KiB, 700)])  # a pair of warps, a CTA per block
-def test_long_literals_take_no_longer_than_text(gmp, ctx, block, n_blocks):  # noqa: F811
+def test_time_beside_text(gmp, ctx, block, n_blocks, byte_mode):  # noqa: F811
     import torch
 
     import datagen
 
     def microseconds(data):
-        ds = gmp.DeviceStream(gmp.compress(np.resize(data, n_blocks * block), block, byte_mode=True, chain_depth=16))
+        ds = gmp.DeviceStream(gmp.compress(np.resize(data, n_blocks * block), block, byte_mode=byte_mode, chain_depth=16))
         out = torch.zeros(n_blocks * block, dtype=torch.uint8, device="cuda")
         st = torch.zeros(1, dtype=torch.int32, device="cuda")
         times = []
@@ -108,5 +156,6 @@ def test_long_literals_take_no_longer_than_text(gmp, ctx, block, n_blocks):  # n
     rows = rng.integers(0, 256, (8 << 10, 40)).astype(np.uint8)  # 31 literals, a copy of 9 bytes from 20 rows back
     for i in range(20, len(rows)):
         rows[i, 31:] = rows[i - 20, 3:12]
-    # 2.6 and 4 times as long when such groups were written record after record
-    assert microseconds(rows.reshape(-1)) < 1.5 * microseconds(datagen.markov_text(1 << 20, seed=2, order=3))
+    # Byte blocks: 2.6 and 4 times as long when such groups were written record after
+    # record.  Huffman blocks have three times as many codes per byte.
+    assert microseconds(rows.reshape(-1)) < (1.5 if byte_mode else 2.5) * microseconds(datagen.markov_text(1 << 20, seed=2, order=3))
