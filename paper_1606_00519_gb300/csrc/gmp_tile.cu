@@ -638,9 +638,14 @@ __device__ __forceinline__ bool huffman_block(TileSmem& S, const BlockView& V, i
       };
       const uint32_t cnt = dense(V, bs_off) ? decode(std::true_type()) : decode(std::false_type());
       if (j < V.K) S.sb_cnt[j] = cnt;
+      // the status is the first damaged sub-block's
+      const uint32_t bad = __ballot_sync(FULL, err != 0);
+      if (bad) {
+        if (lane == (uint32_t)__ffs(bad) - 1u) set_status(status, err);
+        err = 1;
+        break;
+      }
     }
-    if (err) set_status(status, err);
-    err = __any_sync(FULL, err != 0);
     if (lane == 0) S.result[0] = err;
   }
   pair_sync();  // the records are visible to the first warp, the tables' place is free
@@ -1205,7 +1210,7 @@ struct __align__(64) CoopSmem {
   uint32_t tot[2][W], tot_l[2][W];  // each group's output bytes; literal bytes of Byte blocks
   Window win;          // after a slow group
   int32_t result[3];   // of the parts of the table build
-  uint32_t bad;        // Byte: lowest warp << 8 | status of a failed check, else ~0
+  uint32_t bad;        // lowest warp (Huffman: sub-block) << 8 | status of a failed check, else ~0
   Job job;
 };
 
@@ -1233,6 +1238,7 @@ __device__ bool coop_huffman(CoopSmem<W>& S, const BlockView& V, int32_t* status
   CoopSmemA& A = S.u.a;
   BuildSmem& T = A.build;
   const uint32_t bs_off = (192u + 12u * V.K + 15u) & ~15u;  // bitstream start within the block
+  if (t == 0) S.bad = ~0u;
   unpack_lens(T.lens, V.B, t, 32 * W);
   __syncthreads();
   if (warp < 3) {
@@ -1267,8 +1273,10 @@ __device__ bool coop_huffman(CoopSmem<W>& S, const BlockView& V, int32_t* status
   };
   const uint32_t cnt = dense(V, bs_off) ? decode(std::true_type()) : decode(std::false_type());
   if (j < V.K) S.sb_cnt[j] = cnt;
-  if (err) set_status(status, err);
-  return !__syncthreads_or(err != 0);  // the records are visible to the whole CTA
+  if (err) atomicMin(&S.bad, (j << 8) | (uint32_t)err);
+  const bool bad = __syncthreads_or(err != 0);  // the records are visible to the whole CTA
+  if (bad && t == 0) set_status(status, (int)(S.bad & 255u));  // the first damaged sub-block's
+  return !bad;
 }
 
 template <int W, bool BYTE>
