@@ -432,8 +432,9 @@ def measure_decode(args, w, data, streams, dev, dist=None, rank=0, clocks=False,
             torch.cuda.synchronize()
             per_mode[m] = round(data.size * reps / (a.elapsed_time(b) / 1e3) / 1e9, 2)
         res["per_mode_gbs"] = per_mode
-        # where the decode kernel spends its cycles (one extra launch with the
-        # per-phase clock counters on, outside the timed region)
+        # where the kernel that keeps statistics spends its cycles, and its
+        # resolution rounds (one extra launch outside the timed region, whose
+        # kernel has neither)
         sctx = gmp.Context(device=local, max_block_out=w.block_size, warps_per_cta=shape["warps_per_cta"],
                            ctas_per_sm=shape["ctas_per_sm"], collect_stats=True)
         sctx.stats_reset(stream)
@@ -443,6 +444,7 @@ def measure_decode(args, w, data, streams, dev, dist=None, rank=0, clocks=False,
         sctx.close()
         cyc = phase["cycles_tables"] + phase["cycles_huffman"] + phase["cycles_lz77"]
         res["decode_kernel_cycles"] = {
+            "kernel": "gmp::decode_kernel (the one that keeps statistics, not the timed one)",
             "tables": round(phase["cycles_tables"] / max(cyc, 1), 4),
             "huffman": round(phase["cycles_huffman"] / max(cyc, 1), 4),
             "lz77": round(phase["cycles_lz77"] / max(cyc, 1), 4),
@@ -527,7 +529,9 @@ def run_gmp(args):
                 "input_only": {"value": round(in_val, 3), "unit": "GB/s", "h2d_bytes_per_step": int(comp_bytes),
                                "d2h_bytes_per_step": 0,
                                "call": "decompress_from_host_batch (output left in device memory)"}},
-        "gpu_launches": 2 * args.steps,
+        # a batch's prefix kernel and a launch of each default kernel, one of
+        # which decodes
+        "gpu_launches": 3 * args.steps,
         "clocks": res["clocks"],
     }
     if rank == 0 and not args.no_cpu_baseline:

@@ -5,14 +5,15 @@
  * Kaldewey, Lohman, Ross; arXiv:1606.00519).  A stream is cut into blocks that
  * are compressed independently (Sec. 3.1).  Decompression of a block
  * Huffman-decodes its sub-blocks in parallel, one lane per sub-block, with
- * lookup tables of both trees in on-chip memory (Sec. 3.2.1), then resolves
- * the block's LZ77 sequences 32 at a time in one warp: two exclusive prefix
- * sums by shuffle, literal copy, then back-reference copy (Sec. 3.2.2), either
- * by Multi-Round Resolution (Fig. 5, Sec. 4.1) or, for streams written with
- * Dependency Elimination, in a single pass (Fig. 7, Sec. 4.2).  Streams in
- * the byte-level format (Gompresso/Byte, Sec. 3.1) skip the Huffman phase:
- * the warp reads the block's fixed-size sequence records and literal bytes
- * directly and resolves them the same way.
+ * lookup tables of both trees in on-chip memory (Sec. 3.2.1), then writes the
+ * block's LZ77 sequences, many at a time: prefix sums by shuffle place them
+ * (Sec. 3.2.2), and every output byte is copied from its literal or source, by
+ * the default kernels in output order, by the kernel that keeps statistics as
+ * the paper does it: 32 sequences in a warp, back-references by Multi-Round
+ * Resolution (Fig. 5, Sec. 4.1) or, for streams written with Dependency
+ * Elimination, in a single pass (Fig. 7, Sec. 4.2).  Streams in the byte-level
+ * format (Gompresso/Byte, Sec. 3.1) skip the Huffman phase: the block's
+ * fixed-size sequence records and literal bytes are read directly.
  *
  * Conventions for every function:
  *   - Return value: GMP_OK (0) or a negative gmp_error.  No exception crosses
@@ -176,15 +177,16 @@ int gmp_compress(const void* host_in, size_t n, const gmp_compress_opts* o, void
 
 /* Compression on the GPU `device`, every step of it (Sec. 3.1: blocks are
    compressed independently, so all of them at once; Sec. 4.2 for DE).
-   Match search: a CTA per block finds, for 512 positions at a time, the
-   longest match among up to min(o->chain_depth, 64) earlier positions with
-   the same 3-byte prefix hash (input window, chain heads and links in shared
-   memory).  Parse: a warp per block (lazy evaluation, the DE rule when
-   o->de, 1023-byte literal runs for Byte blocks).  Entropy coding: a CTA
-   per block counts both alphabets, builds code lengths limited to o->cwl
-   bits (two-queue Huffman, then the bit-length adjustment of ITU-T T.81
-   Annex K.3), canonical codes, the sub-block split (equal decoding work) and
-   sizes, then packs each sub-block's codes at its bit offset; Byte blocks
+   Match search: a CTA per block links every position to the latest earlier
+   one with the same 3-byte prefix hash, 512 positions at a time; CTAs of up to
+   32 Ki positions then find each one's longest match among up to
+   min(o->chain_depth, 64) linked positions (window and links in shared
+   memory).  Parse: a CTA per block (lazy evaluation, the DE rule when o->de,
+   1023-byte literal runs for Byte blocks).  Entropy coding: a CTA per block
+   counts both alphabets, builds code lengths limited to o->cwl bits (two-queue
+   Huffman, then the bit-length adjustment of ITU-T T.81 Annex K.3), canonical
+   codes, the sub-block split (equal decoding work) and sizes, then packs the
+   codes, a share of the tokens per thread, at their bit offsets; Byte blocks
    get their records and literals.  The host lays the blocks out from their
    sizes and writes the file header and block offset table; the stream
    format is gmp_compress's.  Positions of one step do not see each other
@@ -235,23 +237,28 @@ typedef struct {
   uint32_t max_files;       /* largest n_files of gmp_decompress_batch (default 65536) */
   uint32_t resolve;         /* back-reference resolution, a gmp_resolve (default GMP_RESOLVE_AUTO) */
   uint32_t concurrent;      /* 1: launches run beside other kernels (a serving loop's overlapping
-                               batches): every warp takes its blocks from the work counter as it
-                               arrives; 0 (default): a warp's first block is fixed, interleaved
-                               over the CTAs, which spreads a launch's blocks evenly over the SMs
-                               when all its CTAs are resident at once */
+                               batches): every block is taken from the work counter as a decoder
+                               (a pair of warps, or a CTA) arrives; 0 (default): a decoder's first
+                               block is fixed, interleaved over the CTAs, which spreads a launch's
+                               blocks evenly over the SMs when all its CTAs are resident at once */
 } gmp_context_opts;
 
-/* How a context resolves each 32-sequence group's back-references.  AUTO:
-   streams with the DE flag in one pass (groups that break the DE property by
-   MRR), others by Multi-Round Resolution (Fig. 5, Sec. 4.1).  MRR: MRR even
-   for DE streams.  SC: Sequential Copying, one back-reference at a time in
-   sequence order, the paper's baseline (Sec. 5.1).  All give the same bytes;
-   MRR and SC exist to measure the strategies against each other. */
+/* How a context resolves back-references.  AUTO: by the default kernels, which
+   write the output in order, many bytes at a time, and follow a byte whose
+   source is not written yet to the byte it repeats; streams with and without
+   the DE flag alike.  A context that keeps statistics resolves the groups of 32
+   sequences of the paper instead: streams with the DE flag in one pass (groups
+   that break the DE property by MRR), others by Multi-Round Resolution (Fig. 5,
+   Sec. 4.1).  MRR: MRR even for DE streams.  SC: Sequential Copying, one
+   back-reference at a time in sequence order, the paper's baseline (Sec. 5.1).
+   All give the same bytes; MRR and SC exist to measure the strategies against
+   each other. */
 typedef enum { GMP_RESOLVE_AUTO = 0, GMP_RESOLVE_MRR = 1, GMP_RESOLVE_SC = 2 } gmp_resolve;
 
 void gmp_context_opts_default(gmp_context_opts* o);
 /* Creates a context on `device`: allocates the scratch of one persistent
-   launch (one slot per resident warp) and a small device work counter.
+   launch (a slot per block that is decoded at once) and a small device work
+   counter.
    opts may be NULL.  A context is not thread-safe, and its launches share
    the scratch: calls on one context must not run at the same time, from
    several host threads or on streams whose work overlaps (use a context per
@@ -277,8 +284,9 @@ int gmp_context_set_input_wait(gmp_context* ctx, uint32_t ms);
 int gmp_context_debug_drop_input_flag(gmp_context* ctx, int64_t piece);
 
 /* ------------------------------------------------------------------------ */
-/* Decompression of one stream (Sec. 3.2): one persistent launch, a warp per
-   block taken from a work counter.
+/* Decompression of one stream (Sec. 3.2): one persistent launch; a CTA per block
+   for few blocks, a pair of warps per block for more, taken from a work counter
+   (with statistics or a forced resolution, a warp per block).
    d_comp: device, the whole stream (16-byte aligned); comp_bytes its size.
    d_index: device array of n_blocks gmp_block_ref (from gmp_index_build).
    d_out: device output buffer of out_cap bytes (16-byte aligned for the
@@ -291,7 +299,7 @@ int gmp_decompress(gmp_context* ctx, const uint8_t* d_comp, size_t comp_bytes, c
 
 /* ------------------------------------------------------------------------ */
 /* Batched decompression: many independent streams in ONE persistent launch.
-   Every (file, block) pair is a work item; warps take items from a device
+   Every (file, block) pair is a work item; items are taken from a device
    counter, so files of uneven sizes share the GPU.                         */
 typedef struct {
   const uint8_t* comp;          /* device, 16-byte aligned stream */
@@ -306,8 +314,10 @@ typedef struct {
    n_files int32, each zeroed by this call and then set to the file's first
    error.  A small single-CTA kernel first forms the work-item prefix over the
    files' block counts in context scratch (n_files <= max_files of the
-   context, else GMP_ERR_CAPACITY); the persistent kernel then maps each item
-   to its (file, block) by binary search.  Asynchronous; no allocation;
+   context, else GMP_ERR_CAPACITY) and chooses between a CTA and a pair of warps
+   per block, for each of which there is a launch (the other one returns at
+   once); the persistent kernel then maps each item to its (file, block) by
+   binary search.  Asynchronous; no allocation;
    capturable in a CUDA graph (gmp_batch_graph_create does that). */
 int gmp_decompress_batch(gmp_context* ctx, const gmp_file_desc* d_files, size_t n_files, int32_t* d_status,
                          void* stream);
@@ -363,7 +373,7 @@ int gmp_stats_read(gmp_context* ctx, gmp_stats* out); /* synchronises the device
    decodes all the streams' blocks, which are cut into pieces of consecutive
    blocks (about 32 pieces, 8 to 256 blocks each).  The pieces are copied in,
    in order, on one copy stream, which sets a device flag after each piece;
-   a warp waits for its piece's flag before reading it, so decoding starts
+   a block's decoder waits for its piece's flag before reading it, so decoding starts
    with the first piece.  The kernel sets a second flag once a piece is
    decoded, and the piece's copy back waits for that flag (a stream memory
    operation, cuStreamWaitValue32) on one of 8 copy-back streams, so outputs
@@ -411,7 +421,7 @@ typedef struct gmp_server gmp_server;
 typedef struct {
   uint64_t budget_bytes;  /* device arena for request buffers (default 32 GiB) */
   uint32_t n_lanes;       /* batches in flight at once (default 8); each lane is a context with
-                             its own scratch (about 1.7 MB per resident warp for 256 KiB blocks) */
+                             its own scratch (about 0.7 MB per block decoded at once, of 256 KiB) */
   uint32_t max_batch;     /* requests per launch (default 64; 1 = one launch per request) */
   uint32_t max_block_out; /* largest block output of any request (default 256 KiB) */
   uint32_t warps_per_cta; /* launch shape of the lanes' contexts (0 = default) */
@@ -464,7 +474,7 @@ void gmp_server_destroy(gmp_server* s);
    the largest block output of the stream (gmp_stream_info.max_block_out or
    block_size).  Limits: blocks of at most 256 KiB of output (larger:
    GMP_ERR_CAPACITY, and a block found larger on the device sets
-   GMP_STATUS_CAPACITY), decoded by 32 warps at a time.
+   GMP_STATUS_CAPACITY), decoded 32 at a time, by a CTA of 16 warps each.
    Set-up: the array's device address belongs to one CUDA context.  The
    first call in each context (on each device, and again after a
    cudaDeviceReset) looks it up with cudaGetSymbolAddress, which loads the
@@ -476,7 +486,8 @@ void gmp_server_destroy(gmp_server* s);
 int gmp_decompress_noalloc(const uint8_t* d_comp, size_t comp_bytes, const gmp_block_ref* d_index,
                            size_t n_blocks, uint32_t max_block_out, uint8_t* d_out, size_t out_cap,
                            int32_t* d_status, void* stream);
-/* The fixed limits of gmp_decompress_noalloc (any pointer may be NULL). */
+/* The fixed limits of gmp_decompress_noalloc (any pointer may be NULL); warps:
+   the blocks decoded at a time. */
 void gmp_noalloc_limits(uint32_t* max_block_out, uint32_t* warps, uint64_t* scratch_bytes);
 
 /* Last CUDA error string of this thread (for GMP_ERR_CUDA). */

@@ -194,10 +194,12 @@ class Context:
     def __init__(self, device: int | None = None, max_block_out: int = 256 << 10, warps_per_cta: int = 0,
                  ctas_per_sm: int = 0, collect_stats: bool = False, max_files: int = 65536, resolve: str = "auto",
                  concurrent: bool = False):
-        """resolve: "auto" (DE streams in one pass, others by MRR), "mrr" (MRR
+        """resolve: "auto" (the default kernels), "mrr" (Multi-Round Resolution
         always) or "sc" (sequential copying, the paper's baseline).
-        concurrent: the context's launches run beside other kernels (warps take
-        every block from the work counter instead of a fixed first block)."""
+        collect_stats: decode by the kernel that counts the paper's groups and
+        rounds.  concurrent: the context's launches run beside other kernels
+        (every block is taken from the work counter instead of a fixed first
+        one)."""
         torch = _torch()
         if not torch.cuda.is_available():
             raise RuntimeError("no CUDA device: the decoder runs only on the GPU")

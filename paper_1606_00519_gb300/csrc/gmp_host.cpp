@@ -250,7 +250,7 @@ static int context_alloc_scratch(gmp_context* c) {
   c->shape.warps_per_cta = wpc;
   c->shape.deep = per_sm > occ_wide;
   c->shape.smem_bytes = c->shape.deep ? smem_deep : smem_wide;
-  // one scratch slot per resident warp: the default kernel's 8-byte records,
+  // a scratch slot per block decoded at once: the default kernels' 8-byte records,
   // or records (16 B per sequence; a block holds at most out/3 + 1 sequences)
   // and the literal shadow (output layout plus 16 bytes of separation per
   // sub-block)

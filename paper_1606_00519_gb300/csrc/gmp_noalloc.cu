@@ -10,9 +10,9 @@
 // module and the call itself allocates nothing.  The caller still provides
 // the stream, the block index, the output buffer and the status word.
 //
-// Limits: blocks of at most kMaxBlockOut (256 KiB) of output, decoded by
-// kSlots (32) warps at a time.  The array holds one scratch slot per warp plus
-// a header with the work counter; every GPU that loads this library keeps
+// Limits: blocks of at most kMaxBlockOut (256 KiB) of output, decoded kSlots
+// (32) at a time, by a CTA of 16 warps each.  The array holds a scratch slot for
+// each plus a header with the work counter; every GPU that loads this library keeps
 // about 53 MB of it until the process exits.
 #include <cuda.h>
 #include <cuda_runtime.h>
