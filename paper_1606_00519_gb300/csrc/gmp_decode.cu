@@ -510,6 +510,7 @@ __device__ void decode_block(WarpSmem<LLB>& S, const KParams& P, const gmp_file_
     // ---- sub-block table: prefix sums of bit sizes, output sizes, sequences
     {
       uint32_t carry_bit = 0, carry_out = 0, carry_seq = 0;
+      uint64_t tb = 0, to = 0, ts = 0;  // overflow-safe totals
       for (uint32_t base = 0; base < K; base += 32) {
         uint32_t j = base + lane;
         uint32_t nb = 0, no = 0, ns = 0;
@@ -533,16 +534,11 @@ __device__ void decode_block(WarpSmem<LLB>& S, const KParams& P, const gmp_file_
         carry_bit += __shfl_sync(FULL, ib, 31);
         carry_out += __shfl_sync(FULL, io, 31);
         carry_seq += __shfl_sync(FULL, is, 31);
+        tb += nb;
+        to += no;
+        ts += ns;
       }
       if (lane == 0) S.u.a.sb_seq[K] = carry_seq;
-      // overflow-safe totals
-      uint64_t tb = 0, to = 0, ts = 0;
-      for (uint32_t j = lane; j < K; j += 32) {
-        const uint8_t* e = B + 192 + 12 * j;
-        tb += ld_u32_nc(e);
-        to += ld_u32_nc(e + 4);
-        ts += ld_u32_nc(e + 8);
-      }
   #pragma unroll
       for (int d = 16; d >= 1; d >>= 1) {
         tb += __shfl_xor_sync(FULL, tb, d);

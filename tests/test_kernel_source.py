@@ -58,5 +58,6 @@ def test_sizes_read_twice_are_bounded():
     # written one by one are read a second time, and cut to what is left
     found = functions(source("gmp_tile.cu"))
     assert [k for k, v in found.items() if re.search(r"192u? \+ 12u? \* j", v)] == ["sub_block_table"]
+    assert len(re.findall(r"192u? \+ 12u? \* j", source("gmp_decode.cu"))) == 1
     body = found["slow_group"]
     assert "out_bytes - w.g0" in body and "lits_end - lits" in body and "dist <= w.g0" in body
